@@ -185,7 +185,7 @@ typedef struct {
                                            each step that rebuilt; synchronises) */
     int64_t pair_checks_per_step;       /* resident chains: non-bonded pair slots one step
                                            evaluates, summed over replicas, with the pair list
-                                           each replica built last (64 per list item of 8 x 8
+                                           each replica built last (128 per list item of 8 x 16
                                            atoms, 28 per block of 8 with itself); periodic
                                            box: 64 per chunk of 8 list entries of an 8-slot
                                            cluster (synchronises) */

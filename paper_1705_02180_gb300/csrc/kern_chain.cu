@@ -16,19 +16,21 @@
 //
 // Pair list. Atoms are grouped in blocks of 8 consecutive chain atoms. For each
 // block I the list holds, in ascending order, every atom j of a later block that
-// lies within r_list = r_c + skin of some atom of I, in chunks of 8 (the last one
+// lies within r_list = r_c + skin of some atom of I, in chunks of 16 (the last one
 // padded with a far-away sentinel slot). A work item is one block against one
-// chunk (64 pairs) on a quarter warp: lane l keeps atom j_l of the chunk and takes
-// block atom l ^ t at its pair t, so the i-force accumulators move by one xor exchange
-// per pair while the j-force stays in place. Pairs inside a block form 28-pair
+// chunk (128 pairs) on a quarter warp: lane l keeps entries 2 l and 2 l + 1 of the chunk
+// and meets the four atom pairs of the block in xor order, two FP32 pairs per packed
+// operation, so the i-force accumulators move by xor exchanges while the j-forces stay in
+// place (64 replicas x 560 atoms: 22.4 us per step, against 26.7 with chunks of 8, one
+// entry per lane and scalar operations; the same bits). Pairs inside a block form 28-pair
 // items of their own. The list is rebuilt when a bound on the largest displacement
 // since the last build reaches skin/2, or after rebuild_every steps, so no pair
 // inside r_c is ever missing.
 //
 // Summation. Every pair term s (x_j - x_i) is rounded to an integer multiple of
-// 2^-13 kJ mol^-1 nm^-1 and summed in integers; bonded and bias terms are rounded
-// to 2^-20 units. The shared-memory partials are pairs of 32-bit words (a signed
-// integer part and an unsigned 2^-20 fraction part) added with 32-bit atomics, so
+// 2^-13 kJ mol^-1 nm^-1 and summed in integers, bonded terms likewise, bias-gradient
+// terms to 2^-20 units. The shared-memory partials are sums modulo 2^32, added with
+// 32-bit atomics, with coarse sums of the large terms beside them that fix the total, so
 // every sum is exact and independent of the order of the additions. Results are
 // therefore the same bits whichever warp or CTA takes an item, whatever the list
 // skin or rebuild cadence, and across a checkpoint and resume.
@@ -48,35 +50,100 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kChunk = 32;    // contacts / bonds / angles per work item (one per lane)
 
-// Shared-memory arrays of one CTA. Atom slots: nta real or padding slots plus 8 sentinel
-// slots (a block far from everything) that absorb the padding of list chunks.
-struct Shared {
-    float4* xq;         // (x, y, z, qs), nta + 8
-    float4* v;          // velocities (w: 1/m), nta
-    float4* xi;         // noise of the next O half step per atom (sd times Gaussian numbers);
-                        // w: the atom's |F_bias|^2 / m of the step just closed. During a list
-                        // rebuild it holds the block boxes and chunk counts instead.
-    float2* lj;         // (sigma/2, sqrt(24 eps)), nta + 8
-    int* FH[2];         // force partials of this CTA by parity of the evaluated step:
-    unsigned* FL[2];    //   integer part and 2^-20 fraction part, 3 x (nta + 8) each
-    int* GH[2];         // partials of sum_p (C - C0) C'(u) (x_p - x_i) over the native
-    unsigned* GL[2];    //   contacts this CTA evaluated (the bias gradient without its
-                        //   ratchet factor, which is known only once z is complete)
-    int* flag;          // force-range flag of the current evaluation
-    struct CacheItem* lc;  // this CTA's pair items when they fit (see CacheItem)
-    int nta, na8;       // atom slots; accumulator stride (nta + 8)
-    int lc_cap;         // capacity of lc in items
+extern __shared__ __align__(16) unsigned char smem_raw[];
+
+// A pair item held in shared memory: descriptor, exclusion masks and the chunk's entries
+// (the same data as the global item table, mask table and j entries, without their latency).
+struct __align__(16) CacheItem {
+    uint32_t desc, pad[3];
+    uint8_t xm[kListChunk];
+    uint16_t j[kListChunk];
 };
 
-// A pair item held in shared memory: descriptor, exclusion mask and the chunk's 8 entries
-// (the same data as the global item table, mask table and j entries, without their latency).
-struct CacheItem {
-    uint32_t desc, pad;
-    unsigned long long xm;
-    uint16_t j[8];
+// Two neighbouring atom slots 2 m and 2 m + 1, as the packed FP32 operations take them:
+// positions, scaled charges and LJ parameters (s = sigma/2, e = sqrt(24 eps)).
+struct __align__(16) AtomPair {
+    float4 xy;  // (x0, x1, y0, y1)
+    float4 zq;  // (z0, z1, q0, q1)
+    float4 lj;  // (s0, s1, e0, e1)
+};
+
+// Partials of one kind and parity: per atom slot three modular words, then, after those of all
+// slots, three coarse words per slot (see red3).
+struct Part {
+    unsigned* L;
+    int* H;
+};
+
+// Shared-memory arrays of one CTA, laid out from smem_raw by the slot count alone (every
+// address is an offset computed from nta, so that no pointers stay in registers). Atom slots:
+// nta real or padding slots plus 8 sentinel slots (a block far from everything) that absorb
+// the padding of list chunks. For both parities of the evaluated step, F: force partials of
+// this CTA in 2^-13 units; G: partials of sum_p (C - C0) C'(u) (x_p - x_i) over the native
+// contacts this CTA evaluated, in 2^-20 units (the bias gradient without its ratchet factor,
+// known only once z is complete).
+struct Shared {
+    int nta;       // atom slots
+    int lc_cap;    // capacity of lc in items
+    int fsh, gsh;  // coarse units of the F and G partials (TopoDev)
+    __device__ __forceinline__ int na8() const { return nta + 8; }
+    __device__ __forceinline__ AtomPair* pair() const { return (AtomPair*)smem_raw; }
+    // velocities (w: 1/m), nta
+    __device__ __forceinline__ float4* v() const { return (float4*)(smem_raw + 24 * na8()); }
+    // noise of the next O half step per atom (sd times Gaussian numbers); w: the atom's
+    // |F_bias|^2 / m of the step just closed. During a list rebuild it holds the block boxes
+    // and chunk counts instead.
+    __device__ __forceinline__ float4* xi() const { return v() + nta; }
+    __device__ __forceinline__ Part part(int k) const {
+        Part p;
+        p.L = (unsigned*)(smem_raw + 24 * na8() + 32 * nta + 24 * na8() * k);
+        p.H = (int*)(p.L + 3 * na8());
+        return p;
+    }
+    __device__ __forceinline__ Part F(int b) const { return part(b); }
+    __device__ __forceinline__ Part G(int b) const { return part(2 + b); }
+    // this CTA's pair items when they fit
+    __device__ __forceinline__ CacheItem* lc() const {
+        return (CacheItem*)(smem_raw + 120 * na8() + 32 * nta);
+    }
+};
+
+// Position with charge, and LJ parameters, of atom slot i.
+__device__ __forceinline__ float* slot_of(const Shared& sm, int i) {
+    return (float*)(sm.pair() + (i >> 1)) + (i & 1);
+}
+__device__ __forceinline__ float4 get_x(const Shared& sm, int i) {
+    const float* a = slot_of(sm, i);
+    return make_float4(a[0], a[2], a[4], a[6]);
+}
+__device__ __forceinline__ void put_x(const Shared& sm, int i, float4 x) {
+    float* a = slot_of(sm, i);
+    a[0] = x.x;
+    a[2] = x.y;
+    a[4] = x.z;
+    a[6] = x.w;
+}
+__device__ __forceinline__ float2 get_lj(const Shared& sm, int i) {
+    const float* a = slot_of(sm, i);
+    return make_float2(a[8], a[10]);
+}
+__device__ __forceinline__ void put_lj(const Shared& sm, int i, float2 lj) {
+    float* a = slot_of(sm, i);
+    a[8] = lj.x;
+    a[10] = lj.y;
+}
+
+// List slab of this replica or frame (see scps_internal.h for the layout).
+struct ListDev {
+    uint16_t* jl;               // j entries of all blocks
+    uint32_t* items;            // this CTA's item table
+    uint8_t* excl;              // exclusion masks of this CTA's items
+    int nbs;                    // blocks of the slab layout (nta / 8)
 };
 
 struct Scalars {
+    TopoDev tp;         // the replica's topology and list slab (shared memory: read where
+    ListDev list;       // needed instead of held in registers)
     int work_next[2];   // this CTA's work counter, by parity of the evaluated step
     int status;         // replica status (identical in every CTA of a cluster)
     int bias_on;
@@ -99,28 +166,6 @@ struct Scalars {
     long long red_d[2][kMaxTubeK];      // this CTA's share of sum_p (C_p - A_kp)^2 (2^-40), by parity
 };
 
-__device__ __forceinline__ Shared carve(void* base, int nta, int lc_cap) {
-    Shared s;
-    char* p = (char*)base;
-    const int na8 = nta + 8;
-    s.nta = nta;
-    s.na8 = na8;
-    s.xq = (float4*)p; p += sizeof(float4) * na8;
-    s.v = (float4*)p; p += sizeof(float4) * nta;
-    s.xi = (float4*)p; p += sizeof(float4) * nta;
-    for (int b = 0; b < 2; ++b) {
-        s.FH[b] = (int*)p; p += sizeof(int) * 3 * na8;
-        s.FL[b] = (unsigned*)p; p += sizeof(unsigned) * 3 * na8;
-        s.GH[b] = (int*)p; p += sizeof(int) * 3 * na8;
-        s.GL[b] = (unsigned*)p; p += sizeof(unsigned) * 3 * na8;
-    }
-    s.lj = (float2*)p; p += sizeof(float2) * na8;
-    s.lc = (CacheItem*)p;
-    s.lc_cap = lc_cap;
-    s.flag = nullptr;
-    return s;
-}
-
 __device__ __forceinline__ long long warp_sum_ll(long long v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
@@ -133,49 +178,65 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
-// Adds a 2^-20 fixed-point value to a (integer part, fraction part) accumulator.
-__device__ __forceinline__ void red_fix20(int* H, unsigned* L, int k, long long v) {
-    atomicAdd(&H[k], (int)(v >> 20));
-    atomicAdd(&L[k], (unsigned)(v & 0xfffffll));
+// Adds an integer vector to the partials of slot k: the modular words always, the coarse
+// words only when a component rounds to a non-zero multiple of 2^sh (rarely: one shared
+// atomic per component instead of the two of an integer part and a fraction part).
+__device__ __forceinline__ void red3(const Part& p, int k, int vx, int vy, int vz, int sh) {
+    unsigned* L = p.L + 3 * k;
+    atomicAdd(L, (unsigned)vx);
+    atomicAdd(L + 1, (unsigned)vy);
+    atomicAdd(L + 2, (unsigned)vz);
+    const unsigned half = 1u << (sh - 1);
+    if ((((unsigned)vx + half) | ((unsigned)vy + half) | ((unsigned)vz + half)) >> sh) {
+        const int hx = ((vx >> (sh - 1)) + 1) >> 1, hy = ((vy >> (sh - 1)) + 1) >> 1,
+                  hz = ((vz >> (sh - 1)) + 1) >> 1;
+        int* H = p.H + 3 * k;
+        if (hx) atomicAdd(H, hx);
+        if (hy) atomicAdd(H + 1, hy);
+        if (hz) atomicAdd(H + 2, hz);
+    }
 }
 
-// Adds an integer number of 2^-13 units (the pair terms).
-__device__ __forceinline__ void red_fix13(int* H, unsigned* L, int k, int v) {
-    atomicAdd(&H[k], v >> 13);
-    atomicAdd(&L[k], ((unsigned)v & 0x1fffu) << 7);
+// The same for 64-bit components (the slow path of a pair item).
+__device__ __forceinline__ void red3_64(const Part& p, int k, long long vx, long long vy,
+                                        long long vz, int sh) {
+    atomicAdd(p.L + 3 * k, (unsigned)vx);
+    atomicAdd(p.L + 3 * k + 1, (unsigned)vy);
+    atomicAdd(p.L + 3 * k + 2, (unsigned)vz);
+    atomicAdd(p.H + 3 * k, (int)(((vx >> (sh - 1)) + 1) >> 1));
+    atomicAdd(p.H + 3 * k + 1, (int)(((vy >> (sh - 1)) + 1) >> 1));
+    atomicAdd(p.H + 3 * k + 2, (int)(((vz >> (sh - 1)) + 1) >> 1));
+}
+
+// The exact total of coarse and modular sums (see coarse_shift).
+__device__ __forceinline__ long long join_coarse(long long h, unsigned l, int sh) {
+    const long long c = h << sh;
+    return c + (long long)(int)(l - (unsigned)c);
 }
 
 // Slow path of a pair term: s13 d (2^-13 units, rounded exactly as on the fast path, so the
 // sums are the same integers whichever path a pair takes) to atom i and its negative to atom
 // j, in 64-bit; a non-finite term or one above 1e9 kJ/mol/nm raises the force-range flag.
-__device__ __forceinline__ void add_pair13(const Shared& sm, int* H, unsigned* L, int i, int j,
-                                           float s13, float dx, float dy, float dz) {
+__device__ __forceinline__ void add_pair13(const Part& F, int* flag, int sh, int i, int j, float s13,
+                                           float dx, float dy, float dz) {
     const float tx = s13 * dx, ty = s13 * dy, tz = s13 * dz;
     const float lim = 8.192e12f;  // 1e9 in 2^-13 units
-    if (!(fabsf(tx) <= lim && fabsf(ty) <= lim && fabsf(tz) <= lim)) atomicOr(sm.flag, SCPS_FLAG_FORCE_RANGE);
-    const long long qx = __float2ll_rn(tx) * 128, qy = __float2ll_rn(ty) * 128,
-                    qz = __float2ll_rn(tz) * 128;  // 2^-13 to 2^-20 units
-    const int s = sm.na8;
-    red_fix20(H, L, i, qx);
-    red_fix20(H, L, s + i, qy);
-    red_fix20(H, L, 2 * s + i, qz);
-    red_fix20(H, L, j, -qx);
-    red_fix20(H, L, s + j, -qy);
-    red_fix20(H, L, 2 * s + j, -qz);
+    if (!(fabsf(tx) <= lim && fabsf(ty) <= lim && fabsf(tz) <= lim)) atomicOr(flag, SCPS_FLAG_FORCE_RANGE);
+    const long long qx = __float2ll_rn(tx), qy = __float2ll_rn(ty), qz = __float2ll_rn(tz);
+    red3_64(F, i, qx, qy, qz, sh);
+    red3_64(F, j, -qx, -qy, -qz, sh);
 }
 
 // Bonded terms: integer multiples of 2^-13 kJ mol^-1 nm^-1 (one conversion each); a term
 // that is non-finite or beyond 2.6e5 kJ mol^-1 nm^-1 (a bond stretched by more than 1 nm)
 // raises the force-range flag, which freezes the replica.
-__device__ __forceinline__ void add_term13(const Shared& sm, int* H, unsigned* L, int i, float fx,
-                                           float fy, float fz) {
-    const int s = sm.na8;
+__device__ __forceinline__ void add_term13(const Shared& sm, const Part& F, int* flag, int i,
+                                           float fx, float fy, float fz) {
     if (!(fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz))) < 2.6e5f) ||
         !(isfinite(fx) && isfinite(fy) && isfinite(fz)))
-        atomicOr(sm.flag, SCPS_FLAG_FORCE_RANGE);
-    red_fix13(H, L, i, __float2int_rn(fx * kPairScale));
-    red_fix13(H, L, s + i, __float2int_rn(fy * kPairScale));
-    red_fix13(H, L, 2 * s + i, __float2int_rn(fz * kPairScale));
+        atomicOr(flag, SCPS_FLAG_FORCE_RANGE);
+    red3(F, i, __float2int_rn(fx * kPairScale), __float2int_rn(fy * kPairScale),
+         __float2int_rn(fz * kPairScale), sm.fsh);
 }
 
 // Cluster helpers: CL == 1 degenerates to a plain CTA.
@@ -203,99 +264,142 @@ __device__ __forceinline__ int cta_rank() {
 // Pair items
 // ---------------------------------------------------------------------------
 
-// List slab of this replica or frame (see scps_internal.h for the layout).
-struct ListDev {
-    uint16_t* jl;               // j entries of all blocks
-    uint32_t* items;            // this CTA's item table
-    unsigned long long* excl;   // exclusion masks of this CTA's items
-    int nbs;                    // blocks of the slab layout (nta / 8)
-};
-
 __device__ __forceinline__ ListDev list_of(unsigned char* slab, int nta, int rank) {
     ListDev L;
     L.nbs = nta >> 3;
     L.jl = (uint16_t*)slab;
     const long long ib = list_items_bytes(L.nbs);
     L.items = (uint32_t*)(slab + list_jl_bytes(L.nbs) + (long long)rank * ib);
-    L.excl = (unsigned long long*)(slab + list_jl_bytes(L.nbs) + 2 * ib) +
-             (long long)rank * list_items_cap(L.nbs);
+    L.excl = slab + list_jl_bytes(L.nbs) + 2 * ib + (long long)rank * kListChunk * list_items_cap(L.nbs);
     return L;
 }
 
-// The 64 pairs of one item (block I against the chunk whose atom j this lane holds) on
-// a quarter warp, fast path: integer pair terms summed in 32-bit registers. Items near
-// their block (NEARX) take the excluded pairs from the item's mask xm. Returns false (and
-// adds nothing) when some |s| of the quarter warp exceeds pc.s_lim, for which the integer
-// sums of the item could overflow; the caller then takes the slow path.
+// One entry of an item against two block atoms (packed): adds the rounded terms to the
+// entry's sums fj and returns them for the block atoms. nx: exclusion bits of the two pairs.
 template <int ELEC, bool ENERGY, bool NEARX>
-__device__ __forceinline__ bool pair_item_fast(const Shared& sm, int* FH, unsigned* FL,
-                                               const TopoDev& tp, const PairConst& pc, int I, int j,
-                                               unsigned long long xm, int lane, long long& e18) {
+__device__ __forceinline__ void pair_two(const PairConst& pc, float4 xy, float4 zq, float4 lj2,
+                                         float4 xj, float2 lj, unsigned nx, float lim, int2& tx,
+                                         int2& ty, int2& tz, bool& bad, long long& ei) {
+    const float2 dx = add2(dup2(xj.x), neg2(make_float2(xy.x, xy.y))),
+                 dy = add2(dup2(xj.y), neg2(make_float2(xy.z, xy.w))),
+                 dz = add2(dup2(xj.z), neg2(make_float2(zq.x, zq.y)));
+    const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    bool ok0 = r2.x < pc.rc2, ok1 = r2.y < pc.rc2;
+    if (NEARX) {
+        ok0 = ok0 && !(nx & 1u);
+        ok1 = ok1 && !(nx & 2u);
+    }
+    float2 e;
+    float2 ms = pair_ms2<ELEC, ENERGY>(r2, add2(make_float2(lj2.x, lj2.y), dup2(lj.x)),
+                                       mul2(make_float2(lj2.z, lj2.w), dup2(lj.y)),
+                                       mul2(make_float2(zq.z, zq.w), dup2(xj.w)), pc, &e);
+    ms.x = ok0 ? ms.x : 0.0f;
+    ms.y = ok1 ? ms.y : 0.0f;
+    bad = bad || !(fabsf(ms.x) <= lim) || !(fabsf(ms.y) <= lim);
+    const float2 fx = mul2(ms, dx), fy = mul2(ms, dy), fz = mul2(ms, dz);
+    tx = make_int2(__float2int_rn(fx.x), __float2int_rn(fx.y));
+    ty = make_int2(__float2int_rn(fy.x), __float2int_rn(fy.y));
+    tz = make_int2(__float2int_rn(fz.x), __float2int_rn(fz.y));
+    if (ENERGY) {  // (e comes scaled by 2^13)
+        const float lim_e = kPairScale * kPairEMax, se = kPairEScale / kPairScale;
+        bad = bad || (ok0 && !(fabsf(e.x) < lim_e)) || (ok1 && !(fabsf(e.y) < lim_e));
+        ei += (ok0 ? __float2int_rn(e.x * se) : 0) + (ok1 ? __float2int_rn(e.y * se) : 0);
+    }
+}
+
+// The 128 pairs of one item (block I against a chunk of 16 list entries, of which this lane
+// holds j0 and j1) on a quarter warp, fast path: at iteration t lane l takes the block atoms
+// 2 m, 2 m + 1 with m = (l >> 1) ^ t against both entries, two pairs per packed operation.
+// The sums of the block atoms move by one xor exchange per iteration and component, those of
+// the entries stay in the lane; all are integers in 32-bit registers. Items near their block
+// (NEARX) take the excluded pairs from the masks xm (low byte entry j0, high byte j1). Returns
+// false (and adds nothing) when some |s| of the quarter warp exceeds pc.s_lim / 2, for which
+// the integer sums of the item (16 terms for a block atom) could overflow; the caller then
+// takes the slow path.
+//
+// Bound by the FMA pipe: about 33 packed operations per two pairs, and next to it the XU pipe
+// (two rsqrt, six conversions); two entries per lane halve the shared-memory loads and the
+// exchanges per pair, which would bind next.
+template <int ELEC, bool ENERGY, bool NEARX>
+__device__ __forceinline__ bool pair_item_fast(const Shared& sm, const Part& F,
+                                               const PairConst& pc, int I, int j0, int j1,
+                                               unsigned xm, int lane, long long& e18) {
     const int l8 = lane & 7, q = lane >> 3;
-    // bit t of xr: the pair this lane takes at iteration t (block atom l8 ^ t) is excluded
-    const unsigned xr = NEARX ? (unsigned)(xm >> (8 * l8)) & 0xffu : 0u;
-    const float4 xj = sm.xq[j];
-    const float2 lj = sm.lj[j];
-    const int i0 = 8 * I;
-    int fix = 0, fiy = 0, fiz = 0, fjx = 0, fjy = 0, fjz = 0;
+    float4 xa = get_x(sm, j0), xb = get_x(sm, j1);
+    float2 la = get_lj(sm, j0), lb = get_lj(sm, j1);
+    // the force scale goes in with the entry's eps and charge (a power of two: exact)
+    xa.w *= kPairScale;
+    xb.w *= kPairScale;
+    la.y *= kPairScale;
+    lb.y *= kPairScale;
+    const float lim = 0.5f * kPairScale * pc.s_lim;
+    int2 fix = {0, 0}, fiy = {0, 0}, fiz = {0, 0};
+    int fax = 0, fay = 0, faz = 0, fbx = 0, fby = 0, fbz = 0;
     long long ei = 0;
     bool bad = false;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const int i = (i0 | l8) ^ t;  // block atom l8 ^ t
-        const float4 xi = sm.xq[i];
-        const float2 li = sm.lj[i];
-        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        bool ok = r2 < pc.rc2;
-        if (NEARX) ok = ok && !((xr >> t) & 1u);
-        float e = 0.f;
-        float s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &e);
-        s = ok ? s : 0.0f;
-        bad = bad || !(fabsf(s) <= pc.s_lim);
-        if (ENERGY) bad = bad || (ok && !(fabsf(e) < kPairEMax));
-        const float s13 = s * kPairScale;
-        const int tx = __float2int_rn(s13 * dx), ty = __float2int_rn(s13 * dy),
-                  tz = __float2int_rn(s13 * dz);
-        fix += tx;
-        fiy += ty;
-        fiz += tz;
-        fjx -= tx;
-        fjy -= ty;
-        fjz -= tz;
-        if (ENERGY) ei += ok ? __float2int_rn(e * kPairEScale) : 0;
-        if (t < 7) {  // the sums of block atom l8 ^ t go to the lane that takes it next
-            fix = __shfl_xor_sync(kFull, fix, t ^ (t + 1));
-            fiy = __shfl_xor_sync(kFull, fiy, t ^ (t + 1));
-            fiz = __shfl_xor_sync(kFull, fiz, t ^ (t + 1));
+    for (int t = 0; t < 4; ++t) {
+        const int m = (l8 >> 1) ^ t;
+        const AtomPair& ap = sm.pair()[4 * I + m];
+        const float4 xy = ap.xy, zq = ap.zq, lj2 = ap.lj;
+        int2 ax, ay, az, bx, by, bz;
+        pair_two<ELEC, ENERGY, NEARX>(pc, xy, zq, lj2, xa, la, NEARX ? xm >> (2 * m) : 0u, lim, ax,
+                                      ay, az, bad, ei);
+        pair_two<ELEC, ENERGY, NEARX>(pc, xy, zq, lj2, xb, lb, NEARX ? xm >> (8 + 2 * m) : 0u, lim,
+                                      bx, by, bz, bad, ei);
+        // (the terms come out negated: they are the entries' share)
+        fax += ax.x + ax.y;
+        fay += ay.x + ay.y;
+        faz += az.x + az.y;
+        fbx += bx.x + bx.y;
+        fby += by.x + by.y;
+        fbz += bz.x + bz.y;
+        fix.x -= ax.x + bx.x;
+        fiy.x -= ay.x + by.x;
+        fiz.x -= az.x + bz.x;
+        fix.y -= ax.y + bx.y;
+        fiy.y -= ay.y + by.y;
+        fiz.y -= az.y + bz.y;
+        if (t < 3) {  // to the lane that takes these block atoms next
+            const int d = 2 * (t ^ (t + 1));
+            fix.x = __shfl_xor_sync(kFull, fix.x, d);
+            fiy.x = __shfl_xor_sync(kFull, fiy.x, d);
+            fiz.x = __shfl_xor_sync(kFull, fiz.x, d);
+            fix.y = __shfl_xor_sync(kFull, fix.y, d);
+            fiy.y = __shfl_xor_sync(kFull, fiy.y, d);
+            fiz.y = __shfl_xor_sync(kFull, fiz.y, d);
         }
     }
+    // lanes l and l ^ 1 hold shares of the same two block atoms: each keeps one of them
+    const bool odd = lane & 1;
+    const int kx = (odd ? fix.y : fix.x) + __shfl_xor_sync(kFull, odd ? fix.x : fix.y, 1);
+    const int ky = (odd ? fiy.y : fiy.x) + __shfl_xor_sync(kFull, odd ? fiy.x : fiy.y, 1);
+    const int kz = (odd ? fiz.y : fiz.x) + __shfl_xor_sync(kFull, odd ? fiz.x : fiz.y, 1);
     if ((__ballot_sync(kFull, bad) >> (8 * q)) & 0xffu) return false;
-    const int s3 = sm.na8, i = (i0 | l8) ^ 7;  // after the last exchange lane l holds atom l ^ 7
-    red_fix13(FH, FL, i, fix);
-    red_fix13(FH, FL, s3 + i, fiy);
-    red_fix13(FH, FL, 2 * s3 + i, fiz);
-    red_fix13(FH, FL, j, fjx);
-    red_fix13(FH, FL, s3 + j, fjy);
-    red_fix13(FH, FL, 2 * s3 + j, fjz);
+    red3(F, 8 * I + (l8 ^ 6), kx, ky, kz, sm.fsh);
+    red3(F, j0, fax, fay, faz, sm.fsh);
+    red3(F, j1, fbx, fby, fbz, sm.fsh);
     if (ENERGY) e18 += ei;
     return true;
 }
 
-// Slow path of an item: every pair term goes to both atoms in 64-bit fixed point (rounded
-// per pair as on the fast path) with the range check (a force beyond 1e9 kJ/mol/nm or a
-// non-finite one freezes the replica).
+// Slow path of an item, one entry per lane: every pair term goes to both atoms in 64-bit
+// (rounded per pair as on the fast path) with the range check (a force beyond 1e9 kJ/mol/nm
+// or a non-finite one freezes the replica).
 template <int ELEC, bool ENERGY>
-__device__ __noinline__ void pair_item_slow(const Shared& sm, int* FH, unsigned* FL,
-                                            const TopoDev& tp, const PairConst& pc, int I, int j,
-                                            int lane, long long& e18) {
-    const int l8 = lane & 7;
-    const float4 xj = sm.xq[j];
-    const float2 lj = sm.lj[j];
+__device__ __noinline__ long long pair_item_slow(Shared sm, int b, Scalars* sc, const RunParams& P,
+                                                 int I, int j) {
+    const int l8 = threadIdx.x & 7;
+    const Part F = sm.F(b);
+    const TopoDev& tp = sc->tp;
+    const PairConst& pc = P.pc;
+    long long e18 = 0;
+    const float4 xj = get_x(sm, j);
+    const float2 lj = get_lj(sm, j);
     for (int t = 0; t < 8; ++t) {
         const int i = 8 * I + ((l8 + t) & 7);
-        const float4 xi = sm.xq[i];
-        const float2 li = sm.lj[i];
+        const float4 xi = get_x(sm, i);
+        const float2 li = get_lj(sm, i);
         const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         bool ok = r2 < pc.rc2;
@@ -304,55 +408,64 @@ __device__ __noinline__ void pair_item_slow(const Shared& sm, int* FH, unsigned*
         if (!ok) continue;
         float e = 0.f;
         const float s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &e);
-        add_pair13(sm, FH, FL, i, j, s * kPairScale, dx, dy, dz);
+        add_pair13(F, &sc->flag[b], sm.fsh, i, j, s * kPairScale, dx, dy, dz);
         if (ENERGY) e18 += __float2ll_rn(e * kPairEScale);
     }
+    return e18;
 }
 
 // One batch of four pair items (one per quarter warp) from this CTA's item table.
 template <int ELEC, bool ENERGY>
-__device__ __forceinline__ void pair_batch(const Shared& sm, int* FH, unsigned* FL, const TopoDev& tp,
-                                           const PairConst& pc, const ListDev& L, int n_items,
-                                           bool cached, int batch, int lane, long long& e18) {
-    const int it = 4 * batch + (lane >> 3);
-    int I = 0, j = sm.nta;  // idle quarter: block 0 against the far sentinel slot (zero terms)
+__device__ __forceinline__ void pair_batch(const Shared& sm, Scalars& sc, const RunParams& P, int b,
+                                           int batch, int lane, long long& e18) {
+    const int it = 4 * batch + (lane >> 3), l8 = lane & 7;
+    int I = 0;  // idle quarter: block 0 against the far sentinel slot (zero terms)
+    unsigned jj = (unsigned)sm.nta * 0x10001u, xm = 0u;
     bool near = false;
-    unsigned long long xm = 0ull;
-    if (it < n_items) {
-        if (cached) {
-            const CacheItem& c = sm.lc[it];
+    if (it < sc.n_items) {
+        if (sc.cached) {
+            const CacheItem& c = sm.lc()[it];
             const uint32_t d = c.desc;
             I = (int)(d >> 17);
             near = (d >> 16) & 1u;
-            j = (int)c.j[lane & 7];
-            xm = c.xm;
+            jj = ((const unsigned*)c.j)[l8];
+            if (near) xm = ((const uint16_t*)c.xm)[l8];
         } else {
+            const ListDev& L = sc.list;
             const uint32_t d = __ldcg(L.items + it);
             I = (int)(d >> 17);
             near = (d >> 16) & 1u;
-            j = (int)__ldcg(L.jl + list_jl_off(L.nbs, I) + 8 * (int)(d & 0xffffu) + (lane & 7));
-            if (near) xm = __ldcg(L.excl + it);
+            jj = __ldcg((const unsigned*)(L.jl + list_jl_off(L.nbs, I) + kListChunk * (int)(d & 0xffffu)) + l8);
+            if (near) xm = __ldcg((const uint16_t*)(L.excl + (long long)kListChunk * it) + l8);
         }
     }
+    const int j0 = (int)(jj & 0xffffu), j1 = (int)(jj >> 16);
+    const Part F = sm.F(b);
     bool done;
     if (__any_sync(kFull, near))
-        done = pair_item_fast<ELEC, ENERGY, true>(sm, FH, FL, tp, pc, I, j, xm, lane, e18);
+        done = pair_item_fast<ELEC, ENERGY, true>(sm, F, P.pc, I, j0, j1, xm, lane, e18);
     else
-        done = pair_item_fast<ELEC, ENERGY, false>(sm, FH, FL, tp, pc, I, j, xm, lane, e18);
-    if (!done) pair_item_slow<ELEC, ENERGY>(sm, FH, FL, tp, pc, I, j, lane, e18);
+        done = pair_item_fast<ELEC, ENERGY, false>(sm, F, P.pc, I, j0, j1, 0u, lane, e18);
+    if (!done) {
+        const long long ea = pair_item_slow<ELEC, ENERGY>(sm, b, &sc, P, I, j0);
+        const long long eb = pair_item_slow<ELEC, ENERGY>(sm, b, &sc, P, I, j1);
+        if (ENERGY) e18 += ea + eb;
+    }
 }
 
 // The 28 pairs inside block I on a quarter warp: at round k = 1..4 lane l takes the pair
 // (l, (l + k) & 7) (round 4 on lanes 0..3 only), so every pair comes once; the second
 // atom's accumulators rotate one lane per round and return home with one exchange.
 template <int ELEC, bool ENERGY>
-__device__ __forceinline__ void diag_item(const Shared& sm, int* FH, unsigned* FL, const TopoDev& tp,
-                                          const PairConst& pc, int I, int lane, long long& e18) {
+__device__ __forceinline__ void diag_item(const Shared& sm, Scalars& sc, const PairConst& pc, int b0,
+                                          int I, int lane, long long& e18) {
+    const TopoDev& tp = sc.tp;
+    const Part F = sm.F(b0);
     const int l8 = lane & 7, q = lane >> 3;
     const int src = (lane & 24) | ((l8 + 1) & 7);
     const int i = 8 * I + l8;
-    const float4 xa = sm.xq[i];
-    const float2 la = sm.lj[i];
+    const float4 xa = get_x(sm, i);
+    const float2 la = get_lj(sm, i);
     const unsigned long long em = i < tp.n_atoms ? tp.excl[i] : 0ull;
     int fax = 0, fay = 0, faz = 0, fbx = 0, fby = 0, fbz = 0;
     long long ei = 0;
@@ -360,8 +473,8 @@ __device__ __forceinline__ void diag_item(const Shared& sm, int* FH, unsigned* F
 #pragma unroll
     for (int k = 1; k <= 4; ++k) {
         const int b = 8 * I + ((l8 + k) & 7);
-        const float4 xb = sm.xq[b];
-        const float2 lb = sm.lj[b];
+        const float4 xb = get_x(sm, b);
+        const float2 lb = get_lj(sm, b);
         const float dx = xb.x - xa.x, dy = xb.y - xa.y, dz = xb.z - xa.z;
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         const bool ok = r2 < pc.rc2 && (k < 4 || l8 < 4) && !((em >> (b - i + kExclWindow)) & 1ull);
@@ -390,24 +503,21 @@ __device__ __forceinline__ void diag_item(const Shared& sm, int* FH, unsigned* F
     fbx = __shfl_sync(kFull, fbx, home);
     fby = __shfl_sync(kFull, fby, home);
     fbz = __shfl_sync(kFull, fbz, home);
-    const int s3 = sm.na8;
     if (!((__ballot_sync(kFull, bad) >> (8 * q)) & 0xffu)) {
-        red_fix13(FH, FL, i, fax + fbx);
-        red_fix13(FH, FL, s3 + i, fay + fby);
-        red_fix13(FH, FL, 2 * s3 + i, faz + fbz);
+        red3(F, i, fax + fbx, fay + fby, faz + fbz, sm.fsh);
         if (ENERGY) e18 += ei;
         return;
     }
     for (int k = 1; k <= 4; ++k) {  // slow path (quarter-uniform)
         const int b = 8 * I + ((l8 + k) & 7);
-        const float4 xb = sm.xq[b];
-        const float2 lb = sm.lj[b];
+        const float4 xb = get_x(sm, b);
+        const float2 lb = get_lj(sm, b);
         const float dx = xb.x - xa.x, dy = xb.y - xa.y, dz = xb.z - xa.z;
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         if (!(r2 < pc.rc2 && (k < 4 || l8 < 4) && !((em >> (b - i + kExclWindow)) & 1ull))) continue;
         float e = 0.f;
         const float s = pair_s<ELEC, ENERGY>(r2, la.x + lb.x, la.y * lb.y, xa.w * xb.w, pc, &e);
-        add_pair13(sm, FH, FL, i, b, s * kPairScale, dx, dy, dz);
+        add_pair13(F, &sc.flag[b0], sm.fsh, i, b, s * kPairScale, dx, dy, dz);
         if (ENERGY) e18 += __float2ll_rn(e * kPairEScale);
     }
 }
@@ -417,26 +527,30 @@ __device__ __forceinline__ void diag_item(const Shared& sm, int* FH, unsigned* F
 // ---------------------------------------------------------------------------
 
 template <bool ENERGY>
-__device__ __forceinline__ float bond_term(const Shared& sm, int* H, unsigned* L, const TopoDev& tp,
-                                           int b) {
+__device__ __forceinline__ float bond_term(const Shared& sm, Scalars& sc, int par_, int b) {
+    const TopoDev& tp = sc.tp;
+    const Part F = sm.F(par_);
+    int* flag = &sc.flag[par_];
     const int2 ij = tp.bond_ij[b];
     const float2 par = tp.bond_par[b];
-    const float4 a = sm.xq[ij.x], c = sm.xq[ij.y];
+    const float4 a = get_x(sm, ij.x), c = get_x(sm, ij.y);
     const float dx = c.x - a.x, dy = c.y - a.y, dz = c.z - a.z;
     const float r = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
     const float dr = r - par.x;
     const float f = par.y * dr / r;
-    add_term13(sm, H, L, ij.x, f * dx, f * dy, f * dz);
-    add_term13(sm, H, L, ij.y, -f * dx, -f * dy, -f * dz);
+    add_term13(sm, F, flag, ij.x, f * dx, f * dy, f * dz);
+    add_term13(sm, F, flag, ij.y, -f * dx, -f * dy, -f * dz);
     return ENERGY ? 0.5f * par.y * dr * dr : 0.0f;
 }
 
 template <bool ENERGY>
-__device__ __forceinline__ float angle_term(const Shared& sm, int* H, unsigned* L, const TopoDev& tp,
-                                            int q) {
+__device__ __forceinline__ float angle_term(const Shared& sm, Scalars& sc, int par_, int q) {
+    const TopoDev& tp = sc.tp;
+    const Part F = sm.F(par_);
+    int* flag = &sc.flag[par_];
     const int4 ijk = tp.ang_ijk[q];
     const float2 par = tp.ang_par[q];
-    const float4 a = sm.xq[ijk.x], b = sm.xq[ijk.y], c = sm.xq[ijk.z];
+    const float4 a = get_x(sm, ijk.x), b = get_x(sm, ijk.y), c = get_x(sm, ijk.z);
     const float ux = a.x - b.x, uy = a.y - b.y, uz = a.z - b.z;
     const float wx = c.x - b.x, wy = c.y - b.y, wz = c.z - b.z;
     const float cx = uy * wz - uz * wy, cy = uz * wx - ux * wz, cz = ux * wy - uy * wx;
@@ -450,44 +564,40 @@ __device__ __forceinline__ float angle_term(const Shared& sm, int* H, unsigned* 
     const float au = cs / ru2, aw = cs / rw2;
     const float fix = g * fmaf(au, ux, -wx), fiy = g * fmaf(au, uy, -wy), fiz = g * fmaf(au, uz, -wz);
     const float fkx = g * fmaf(aw, wx, -ux), fky = g * fmaf(aw, wy, -uy), fkz = g * fmaf(aw, wz, -uz);
-    add_term13(sm, H, L, ijk.x, fix, fiy, fiz);
-    add_term13(sm, H, L, ijk.z, fkx, fky, fkz);
-    add_term13(sm, H, L, ijk.y, -(fix + fkx), -(fiy + fky), -(fiz + fkz));
+    add_term13(sm, F, flag, ijk.x, fix, fiy, fiz);
+    add_term13(sm, F, flag, ijk.z, fkx, fky, fkz);
+    add_term13(sm, F, flag, ijk.y, -(fix + fkx), -(fiy + fky), -(fiz + fkz));
     return ENERGY ? 0.5f * par.y * dth * dth : 0.0f;
 }
 
 // Adds h (x_p - x_i) to G_i and its negative to G_p (2^-20 fixed point). |h| <= |C - C0|
 // |dC/du| < 1 and h |x_p - x_i| stays far below 2^11, so one conversion to a 32-bit count
 // of 2^-20 units rounds exactly as the 64-bit conversion would.
-__device__ __forceinline__ void add_grad(const Shared& sm, int* GH, unsigned* GL, int i, int p,
-                                         float h, float dx, float dy, float dz) {
+__device__ __forceinline__ void add_grad(const Shared& sm, int b, int i, int p, float h, float dx,
+                                         float dy, float dz) {
     const float h20 = h * 1048576.0f;  // 2^20
     const int gx = __float2int_rn(h20 * dx), gy = __float2int_rn(h20 * dy),
               gz = __float2int_rn(h20 * dz);
-    const int s = sm.na8;
-    red_fix20(GH, GL, i, (long long)gx);
-    red_fix20(GH, GL, s + i, (long long)gy);
-    red_fix20(GH, GL, 2 * s + i, (long long)gz);
-    red_fix20(GH, GL, p, -(long long)gx);
-    red_fix20(GH, GL, s + p, -(long long)gy);
-    red_fix20(GH, GL, 2 * s + p, -(long long)gz);
+    const Part G = sm.G(b);
+    red3(G, i, gx, gy, gz, sm.gsh);
+    red3(G, p, -gx, -gy, -gz, sm.gsh);
 }
 
 // One native contact (i, p): (C - C0)^2 in float-float, returned as a 2^-40
 // fixed-point value. h (x_p - x_i) with h = (C - C0) dC/du goes to G_i and its
 // negative to G_p, so that grad_i (C - C0)^2 = -4 h (x_p - x_i) / r0^2 is
 // -4 G_i / r0^2 summed over the atom's contacts (Eq. zrMD, Eq. Cij).
-__device__ __forceinline__ long long contact_term(const Shared& sm, int* GH, unsigned* GL,
-                                                  const TopoDev& tp, const RunParams& P, int c) {
+__device__ __forceinline__ long long contact_term(const Shared& sm, const TopoDev& tp,
+                                                  const RunParams& P, int par_, int c) {
     const int2 ij = tp.con_ij[c];
-    const float4 a = sm.xq[ij.x], b = sm.xq[ij.y];
+    const float4 a = get_x(sm, ij.x), b = get_x(sm, ij.y);
     const ff r2 = ff_dist2(a, b);
     const ff u = ff_mul(r2, P.inv_r0sq_ff);
     const ff C = contact_C_ff(u);
     const float2 c0 = tp.con_C0[c];
     const ff d = ff_add(C, ff{-c0.x, -c0.y});
     const float h = (d.hi + d.lo) * contact_dC_du(u.hi);
-    add_grad(sm, GH, GL, ij.x, ij.y, h, b.x - a.x, b.y - a.y, b.z - a.z);
+    add_grad(sm, par_, ij.x, ij.y, h, b.x - a.x, b.y - a.y, b.z - a.z);
     return ff2fix40(ff_sqr(d));
 }
 
@@ -505,9 +615,9 @@ __device__ __forceinline__ void noise_chunk(const Shared& sm, const TopoDev& tp,
         const float sd = tp.noise_sd[i];
         // xyz only: w holds the atom's bias-functional term, which warp 0 may still be
         // summing while the next evaluation starts
-        sm.xi[i].x = sd * g.x;
-        sm.xi[i].y = sd * g.y;
-        sm.xi[i].z = sd * g.z;
+        sm.xi()[i].x = sd * g.x;
+        sm.xi()[i].y = sd * g.y;
+        sm.xi()[i].z = sd * g.z;
     }
 }
 
@@ -544,7 +654,7 @@ __device__ __forceinline__ void tube_pass1(const Shared& sm, const TopoDev& tp, 
     float C = 0.f;
     if (hl < nq) {
         const int2 ij = tp.con_ij[c0 + hl];
-        const float4 a = sm.xq[ij.x], q = sm.xq[ij.y];
+        const float4 a = get_x(sm, ij.x), q = get_x(sm, ij.y);
         const float dx = q.x - a.x, dy = q.y - a.y, dz = q.z - a.z;
         C = contact_C_f32(fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * P.inv_r0sq);
     }
@@ -589,8 +699,7 @@ __device__ __forceinline__ void tube_pass1(const Shared& sm, const TopoDev& tp, 
 // with the dot of contact L >> 1. The order of every sum is fixed. Two items per warp
 // keep twice the loads in flight per L2 round trip.
 __device__ __forceinline__ void tube_pass2(const Shared& sm, const Scalars& sc, const TopoDev& tp,
-                                           const RunParams& P, int* GH, unsigned* GL, int c0,
-                                           bool has, int lane) {
+                                           const RunParams& P, int b, int c0, bool has, int lane) {
     const int hl = lane & 15;
     const int nq = has ? min(kTubeItem, tp.n_contacts - c0) : 0;
     // the contact of half lane l (l < nq; clamped elsewhere) is read first, so that its
@@ -627,12 +736,12 @@ __device__ __forceinline__ void tube_pass2(const Shared& sm, const Scalars& sc, 
     // every lane stays to the end (all exchanges above are full-warp); lanes >= nq
     // of a half hold a copy of its last contact and add nothing
     const bool live = hl < nq;
-    const float4 a = sm.xq[ij.x], q = sm.xq[ij.y];
+    const float4 a = get_x(sm, ij.x), q = get_x(sm, ij.y);
     const float dx = q.x - a.x, dy = q.y - a.y, dz = q.z - a.z;
     const float u = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * P.inv_r0sq;
     const float C = contact_C_f32(u);
     const float h = live ? 2.0f * tp.tube_inv_n0 * (C * sc.gam_sum - dot) * contact_dC_du(u) : 0.f;
-    if (live) add_grad(sm, GH, GL, ij.x, ij.y, h, dx, dy, dz);
+    if (live) add_grad(sm, b, ij.x, ij.y, h, dx, dy, dz);
 }
 
 // Tube variables and their ratchets from the summed slice distances (warp 0):
@@ -729,48 +838,42 @@ struct AtomSums {
 template <int CL>
 __device__ __forceinline__ void load_sums(const Shared& sm, int b, int peer, int i, bool bias,
                                           AtomSums& a) {
-    const int s = sm.na8;
+    const Part F = sm.F(b), G = sm.G(b);
     int fh[3], gh[3];
     unsigned fl[3], gl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        fh[c] = sm.FH[b][c * s + i];
-        fl[c] = sm.FL[b][c * s + i];
-        gh[c] = bias ? sm.GH[b][c * s + i] : 0;
-        gl[c] = bias ? sm.GL[b][c * s + i] : 0u;
-    }
-    long long lo[3], glo[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        lo[c] = (long long)fl[c];
-        glo[c] = (long long)gl[c];
+        fh[c] = F.H[3 * i + c];
+        fl[c] = F.L[3 * i + c];
+        gh[c] = bias ? G.H[3 * i + c] : 0;
+        gl[c] = bias ? G.L[3 * i + c] : 0u;
     }
     if (CL == 2) {
-        const int* pFH = rank_ptr<CL>(sm.FH[b], peer);
-        const unsigned* pFL = rank_ptr<CL>(sm.FL[b], peer);
-        const int* pGH = rank_ptr<CL>(sm.GH[b], peer);
-        const unsigned* pGL = rank_ptr<CL>(sm.GL[b], peer);
+        const int* pFH = rank_ptr<CL>(F.H, peer) + 3 * i;
+        const unsigned* pFL = rank_ptr<CL>(F.L, peer) + 3 * i;
+        const int* pGH = rank_ptr<CL>(G.H, peer) + 3 * i;
+        const unsigned* pGL = rank_ptr<CL>(G.L, peer) + 3 * i;
         int rh[3], qh[3];
         unsigned rl[3], ql[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            rh[c] = pFH[c * s + i];
-            rl[c] = pFL[c * s + i];
-            qh[c] = bias ? pGH[c * s + i] : 0;
-            ql[c] = bias ? pGL[c * s + i] : 0u;
+            rh[c] = pFH[c];
+            rl[c] = pFL[c];
+            qh[c] = bias ? pGH[c] : 0;
+            ql[c] = bias ? pGL[c] : 0u;
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             fh[c] += rh[c];
             gh[c] += qh[c];
-            lo[c] += (long long)rl[c];
-            glo[c] += (long long)ql[c];
+            fl[c] += rl[c];
+            gl[c] += ql[c];
         }
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        a.f[c] = ((long long)fh[c] << 20) + lo[c];
-        a.g[c] = ((long long)gh[c] << 20) + glo[c];
+        a.f[c] = join_coarse(fh[c], fl[c], sm.fsh) * 128;  // 2^-13 to 2^-20 units
+        a.g[c] = join_coarse(gh[c], gl[c], sm.gsh);
     }
 }
 
@@ -787,16 +890,17 @@ __device__ __forceinline__ void load_sums(const Shared& sm, int b, int peer, int
 // the cluster; returns after a cluster barrier (the peer has finished reading this
 // CTA's counts, which share the xi array's space).
 template <int CL>
-__device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, float rlist2,
-                           const ListDev& L) {
+__device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
+    const TopoDev& tp = sc.tp;
+    const ListDev L = sc.list;
     const int n = tp.n_atoms, nb = (n + 7) >> 3;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int rank = cta_rank<CL>();
     // scratch in the xi array: boxes (2 nb float4), chunk counts, near-chunk counts
     // and the two prefix arrays (nb ints each)
-    float4* blo = sm.xi;
-    float4* bhi = sm.xi + nb;
-    int* cnt = (int*)(sm.xi + 2 * nb);
+    float4* blo = sm.xi();
+    float4* bhi = sm.xi() + nb;
+    int* cnt = (int*)(sm.xi() + 2 * nb);
     int* cntn = cnt + nb;
     int* pren = cntn + nb;
     int* pref = pren + nb;
@@ -806,7 +910,7 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
         float4 lo = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
         float4 hi = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
         for (int a = 8 * I; a < min(8 * I + 8, n); ++a) {
-            const float4 x = sm.xq[a];
+            const float4 x = get_x(sm, a);
             lo.x = fminf(lo.x, x.x);
             lo.y = fminf(lo.y, x.y);
             lo.z = fminf(lo.z, x.z);
@@ -825,7 +929,7 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
         const int I = __shfl_sync(kFull, m, 0) * CL + rank;
         if (I >= nb) break;
         const float4 bl = blo[I], bh = bhi[I];
-        const int i0 = 8 * I, ia = min(8, n - i0);
+        const int i0 = 8 * I;
         uint16_t* out = L.jl + list_jl_off(L.nbs, I);
         int count = 0, n_near = 0;
         for (int J0 = I + 1; J0 < nb; J0 += 32) {
@@ -846,12 +950,16 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
                 const int j = Jc >= 0 ? 8 * Jc + (lane & 7) : n;
                 bool hit = false;  // within sqrt(rlist2) of some atom of the block
                 if (j < n) {
-                    const float4 xj = sm.xq[j];
+                    const float4 xj = get_x(sm, j);
                     float dmin = 3.0e38f;
-                    for (int a = 0; a < ia; ++a) {
-                        const float4 xa = sm.xq[i0 + a];
-                        const float dx = xj.x - xa.x, dy = xj.y - xa.y, dz = xj.z - xa.z;
-                        dmin = fminf(dmin, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {  // (the padding slots of a last block are far)
+                        const float4 xy = sm.pair()[4 * I + m].xy, zq = sm.pair()[4 * I + m].zq;
+                        const float2 dx = add2(dup2(xj.x), neg2(make_float2(xy.x, xy.y))),
+                                     dy = add2(dup2(xj.y), neg2(make_float2(xy.z, xy.w))),
+                                     dz = add2(dup2(xj.z), neg2(make_float2(zq.x, zq.y)));
+                        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+                        dmin = fminf(dmin, fminf(r2.x, r2.y));
                     }
                     hit = dmin < rlist2;
                 }
@@ -862,11 +970,11 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
                 n_near += __popc(nm);
             }
         }
-        const int padded = (count + 7) & ~7;
-        if (lane < padded - count) out[count + lane] = (uint16_t)sm.nta;
+        const int chunks = (count + kListChunk - 1) / kListChunk;
+        if (lane < kListChunk * chunks - count) out[count + lane] = (uint16_t)sm.nta;
         if (lane == 0) {
-            cnt[I] = padded >> 3;
-            cntn[I] = (n_near + 7) >> 3;  // chunks whose first entry is near the block
+            cnt[I] = chunks;
+            cntn[I] = (n_near + kListChunk - 1) / kListChunk;  // chunks with an entry near the block
         }
     }
     __threadfence();  // entries are read back with L2 loads (also by the peer CTA)
@@ -905,7 +1013,7 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
             sc.n_diag = (nb - rank + CL - 1) / CL;
             sc.work_next[0] = 0;
             sc.work_next[1] = 0;
-            sc.pair_slots = 64ll * total + 28ll * nb;  // pairs evaluated per step with this list
+            sc.pair_slots = 8ll * kListChunk * total + 28ll * nb;  // pairs evaluated per step with this list
         }
         // the total number of near chunks, for the far items' numbering
         if (lane == 0) pref[nb] = runn;
@@ -920,44 +1028,38 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
             const int k = c < cn ? pren[I] + c : tot_near + pref[I] + (c - cn);
             if (k % CL == rank) {
                 const uint32_t d = ((uint32_t)I << 17) | ((uint32_t)(c < cn) << 16) | (uint32_t)c;
-                if (cached) {  // the chunk's 8 entries: one 16-byte load (chunks are 16-aligned)
-                    CacheItem& ci = sm.lc[k / CL];
+                if (cached) {  // the chunk's entries: two 16-byte loads (chunks are 32-aligned)
+                    CacheItem& ci = sm.lc()[k / CL];
+                    const uint4* e = (const uint4*)(L.jl + list_jl_off(L.nbs, I) + kListChunk * c);
                     ci.desc = d;
-                    ci.xm = 0ull;
-                    *(uint4*)ci.j = __ldcg((const uint4*)(L.jl + list_jl_off(L.nbs, I) + 8 * c));
+                    ((uint4*)ci.j)[0] = __ldcg(e);
+                    ((uint4*)ci.j)[1] = __ldcg(e + 1);
                 } else {
                     L.items[k / CL] = d;
                 }
             }
         }
-        __syncwarp();  // (the records above are complete before their masks are written)
-        // excluded pairs of the near items, in the order the lanes meet them (byte s, bit t:
-        // entry s with block atom s ^ t); four chunks per pass, eight lanes each, the
-        // block atoms' exclusion words held by lanes 0..7
+        // excluded pairs of the near items: one byte per entry, bit a for block atom a; two
+        // chunks per pass, 16 lanes each, the block atoms' exclusion words held by lanes 0..7
+        // (other items take no masks)
         const unsigned long long exa = (lane < 8 && 8 * I + lane < n) ? tp.excl[8 * I + lane] : 0ull;
         const uint16_t* e = L.jl + list_jl_off(L.nbs, I);
-        for (int c0 = 0; c0 < cn; c0 += 4) {
-            const int c = c0 + (lane >> 3), sl = lane & 7;
-            const int jj = c < cn ? (int)__ldcg(e + 8 * c + sl) : 0;
+        for (int c0 = 0; c0 < cn; c0 += 2) {
+            const int c = c0 + (lane >> 4), sl = lane & 15;
+            const int jj = c < cn ? (int)__ldcg(e + kListChunk * c + sl) : 0;
             unsigned byte = 0u;
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const int a = sl ^ t, i = 8 * I + a;
+            for (int a = 0; a < 8; ++a) {
                 const unsigned long long ex = __shfl_sync(kFull, exa, a);
-                const int dj = jj - i + kExclWindow;  // entries lie after the block
-                if (c < cn && dj < 2 * kExclWindow && ((ex >> dj) & 1ull)) byte |= 1u << t;
+                const int dj = jj - (8 * I + a) + kExclWindow;  // entries lie after the block
+                if (c < cn && dj < 2 * kExclWindow && ((ex >> dj) & 1ull)) byte |= 1u << a;
             }
-            unsigned long long m = (unsigned long long)byte << (8 * sl);
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) m |= __shfl_xor_sync(kFull, m, o);
-            if (sl == 0 && c < cn) {
-                const int k = pren[I] + c;
-                if (k % CL == rank) {
-                    if (cached)
-                        sm.lc[k / CL].xm = m;
-                    else
-                        L.excl[k / CL] = m;
-                }
+            const int k = c < cn ? pren[I] + c : 0;
+            if (c < cn && k % CL == rank) {
+                if (cached)
+                    sm.lc()[k / CL].xm[sl] = (uint8_t)byte;
+                else
+                    L.excl[(long long)kListChunk * (k / CL) + sl] = (uint8_t)byte;
             }
         }
     }
@@ -976,16 +1078,11 @@ __device__ void build_list(const Shared& sm, Scalars& sc, const TopoDev& tp, flo
 // Gaussian numbers of that step's O half step for all atoms (each CTA of a cluster
 // integrates every atom). On return the CTA is synchronised.
 template <int ELEC, bool ENERGY, int CL, bool TUBE>
-__device__ void evaluate(Shared& sm, Scalars& sc, const TopoDev& tp, const RunParams& P,
-                         const ListDev& L, int b, bool do_ratchet, uint32_t rep_id,
-                         long long noise_step) {
+__device__ void evaluate(const Shared& sm, Scalars& sc, const RunParams& P, int b, bool do_ratchet,
+                         uint32_t rep_id, long long noise_step) {
+    const TopoDev& tp = sc.tp;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int nt = tp.n_tiles;
-    int* FH = sm.FH[b];
-    unsigned* FL = sm.FL[b];
-    int* GH = sm.GH[b];
-    unsigned* GL = sm.GL[b];
-    sm.flag = &sc.flag[b];
     if (noise_step >= 0)
         for (int q = warp; q < nt; q += nw) noise_chunk(sm, tp, P, rep_id, noise_step, q, lane);
     const int rank = cta_rank<CL>();
@@ -1031,7 +1128,7 @@ __device__ void evaluate(Shared& sm, Scalars& sc, const TopoDev& tp, const RunPa
                 if (r < n_pb - m_mix) kp = m_mix + r; else kc = m_mix + r - (n_pb - m_mix);
             }
             if (kp >= 0) {
-                pair_batch<ELEC, ENERGY>(sm, FH, FL, tp, P.pc, L, sc.n_items, sc.cached, kp, lane, e18);
+                pair_batch<ELEC, ENERGY>(sm, sc, P, b, kp, lane, e18);
             } else {
                 const int g = kc * CL + rank;
                 if (tube) {
@@ -1041,23 +1138,23 @@ __device__ void evaluate(Shared& sm, Scalars& sc, const TopoDev& tp, const RunPa
                     }
                 } else {
                     const int c = g * kChunk + lane;
-                    if (c < ncon) zacc += contact_term(sm, GH, GL, tp, P, c);
+                    if (c < ncon) zacc += contact_term(sm, tp, P, b, c);
                 }
             }
         } else if (k < e_diag) {
             const int d = 4 * (k - e_pair) + (lane >> 3);
             const int I = d < sc.n_diag ? d * CL + rank : (sm.nta >> 3);
-            diag_item<ELEC, ENERGY>(sm, FH, FL, tp, P.pc, I, lane, e18);
+            diag_item<ELEC, ENERGY>(sm, sc, P.pc, b, I, lane, e18);
         } else if (k < e_bond) {
             const int q = ((k - e_diag) * CL + rank) * kChunk + lane;
             if (q < tp.n_bonds) {
-                const float eb = bond_term<ENERGY>(sm, FH, FL, tp, q);
+                const float eb = bond_term<ENERGY>(sm, sc, b, q);
                 if (ENERGY) e20 += f2fix(eb);
             }
         } else {
             const int q = ((k - e_bond) * CL + rank) * kChunk + lane;
             if (q < tp.n_angles) {
-                const float ea = angle_term<ENERGY>(sm, FH, FL, tp, q);
+                const float ea = angle_term<ENERGY>(sm, sc, b, q);
                 if (ENERGY) e20 += f2fix(ea);
             }
         }
@@ -1136,7 +1233,7 @@ __device__ void evaluate(Shared& sm, Scalars& sc, const TopoDev& tp, const RunPa
             if (2 * u * CL + rank >= n2) break;
             if (lane == 0) m2 = atomicAdd(counter2, 1);
             const int k = (2 * u + (lane >> 4)) * CL + rank;
-            tube_pass2(sm, sc, tp, P, GH, GL, k * kTubeItem, k < n2, lane);
+            tube_pass2(sm, sc, tp, P, b, k * kTubeItem, k < n2, lane);
         }
         cluster_barrier<CL>();  // the peer reads this CTA's G next
         if (tid == 0) sc.work_next2[b] = 0;
@@ -1158,38 +1255,34 @@ template <int ELEC, int CL, bool TUBE>
 __global__ void __launch_bounds__(CL == 2 ? kMaxThreadsPair : 1024, 1)
 k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, StateDev st,
            RunParams P, int nta, int lc_cap) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Scalars sc;
     const RepDev rep = reps[blockIdx.x / CL];  // this launch's replicas, in any order
     const int r = rep.index;
     const int rank = cta_rank<CL>();
-    const TopoDev tp = topos[rep.topo];
-    Shared sm = carve(smem_raw, nta, lc_cap);
-    const ListDev L = list_of(P.list_base + rep.list_off, nta, rank);
+    if (threadIdx.x == 0) {
+        sc.tp = topos[rep.topo];
+        sc.list = list_of(P.list_base + rep.list_off, nta, rank);
+    }
+    __syncthreads();
+    const TopoDev& tp = sc.tp;
+    const Shared sm = {nta, lc_cap, tp.f_shift, tp.g_shift};
     const int n = tp.n_atoms;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    for (int i = tid; i < sm.na8; i += blockDim.x) {
+    for (int i = tid; i < sm.na8(); i += blockDim.x) {
         if (i < n) {
             const float4 x = st.x[rep.atom_off + i];
-            sm.xq[i] = make_float4(x.x, x.y, x.z, tp.qs[i]);
-            sm.lj[i] = tp.lj[i];
+            put_x(sm, i, make_float4(x.x, x.y, x.z, tp.qs[i]));
+            put_lj(sm, i, tp.lj[i]);
             const float4 v = st.v[rep.atom_off + i];
-            sm.v[i] = make_float4(v.x, v.y, v.z, tp.inv_m[i]);
+            sm.v()[i] = make_float4(v.x, v.y, v.z, tp.inv_m[i]);
         } else {
-            sm.xq[i] = far_slot(i);
-            sm.lj[i] = make_float2(0.f, 0.f);
-            if (i < nta) sm.v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            put_x(sm, i, far_slot(i));
+            put_lj(sm, i, make_float2(0.f, 0.f));
+            if (i < nta) sm.v()[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
-    for (int i = tid; i < 3 * sm.na8; i += blockDim.x) {
-        for (int b = 0; b < 2; ++b) {
-            sm.FH[b][i] = 0;
-            sm.FL[b][i] = 0u;
-            sm.GH[b][i] = 0;
-            sm.GL[b][i] = 0u;
-        }
-    }
+    for (int i = tid; i < 24 * sm.na8(); i += blockDim.x) sm.F(0).L[i] = 0u;  // F and G, both parities
     if (tid == 0) {
         sc.zm = st.zm[r];
         sc.z = st.z[r];
@@ -1218,14 +1311,14 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
     const int peer = rank ^ 1;
     const float hdt = P.half_dt;
     if (sc.status == 0 && P.n_steps > 0) {
-        build_list<CL>(sm, sc, tp, P.rlist2, L);
+        build_list<CL>(sm, sc, P.rlist2);
         // displacement bound since the last build and steps since then (identical in every
         // thread of the cluster: same inputs, same arithmetic)
         float disp = 0.f;
         int since = 0;
         builds = 1;
         // the O half step that follows an evaluation uses the noise of the same step index
-        evaluate<ELEC, false, CL, TUBE>(sm, sc, tp, P, L, (int)(step & 1), true, rep.rep_id, step);
+        evaluate<ELEC, false, CL, TUBE>(sm, sc, P, (int)(step & 1), true, rep.rep_id, step);
         // position of `step` in the save cycle and ring slot of the next frame, kept as
         // counters so that the loop has no 64-bit divisions
         int save_phase = P.save_interval > 0 ? (int)(step % P.save_interval) : -1;
@@ -1245,25 +1338,26 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                     load_sums<CL>(sm, b, peer, i, bias, a);
                     // the other parity's partials were last read before this evaluation's
                     // cluster barrier (here and in the peer): clear them for the next one
+                    const Part Fn = sm.F(nb), Gn = sm.G(nb);
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
-                        sm.FH[nb][c * sm.na8 + i] = 0;
-                        sm.FL[nb][c * sm.na8 + i] = 0u;
-                        sm.GH[nb][c * sm.na8 + i] = 0;
-                        sm.GL[nb][c * sm.na8 + i] = 0u;
+                        Fn.L[3 * i + c] = 0u;
+                        Fn.H[3 * i + c] = 0;
+                        Gn.L[3 * i + c] = 0u;
+                        Gn.H[3 * i + c] = 0;
                     }
-                    float4 v = sm.v[i];
+                    float4 v = sm.v()[i];
                     const float im = v.w;
                     float fx = fix2f(a.f[0]), fy = fix2f(a.f[1]), fz = fix2f(a.f[2]);
                     if (bias) {
                         const float bx = kb * fix2f(a.g[0]), by = kb * fix2f(a.g[1]),
                                     bz = kb * fix2f(a.g[2]);
-                        if (do_b) sm.xi[i].w = (bx * bx + by * by + bz * bz) * im;
+                        if (do_b) sm.xi()[i].w = (bx * bx + by * by + bz * bz) * im;
                         fx += bx;
                         fy += by;
                         fz += bz;
                     }
-                    float4 x = sm.xq[i];
+                    float4 x = get_x(sm, i);
                     if (do_b) {  // B: closes the evaluated step
                         v.x = fmaf(hdt * im, fx, v.x);
                         v.y = fmaf(hdt * im, fy, v.y);
@@ -1283,7 +1377,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         x.x = fmaf(hdt, v.x, x.x);
                         x.y = fmaf(hdt, v.y, x.y);
                         x.z = fmaf(hdt, v.z, x.z);
-                        const float4 xi = sm.xi[i];  // drawn during the evaluation
+                        const float4 xi = sm.xi()[i];  // drawn during the evaluation
                         v.x = fmaf(P.c1, v.x, xi.x);
                         v.y = fmaf(P.c1, v.y, xi.y);
                         v.z = fmaf(P.c1, v.z, xi.z);
@@ -1294,9 +1388,9 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
                               isfinite(v.y) && isfinite(v.z)))
                             atomicOr(&sc.status, SCPS_FLAG_NONFINITE);
-                        sm.xq[i] = x;
+                        put_x(sm, i, x);
                     }
-                    sm.v[i] = v;
+                    sm.v()[i] = v;
                 }
             }
             if (do_a) {  // largest speed of the step (positive floats order as their bits)
@@ -1310,7 +1404,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             __syncthreads();
             if (warp == 0 && do_b && bias) {  // atoms in a fixed order, whatever the CTA shape
                 float tsum = 0.f;
-                for (int i = lane; i < n; i += 32) tsum += sm.xi[i].w;
+                for (int i = lane; i < n; i += 32) tsum += sm.xi()[i].w;
                 tsum = warp_sum_f(tsum);
                 if (lane == 0) sc.T += (double)P.dt / P.gamma * (double)tsum;
             }
@@ -1338,16 +1432,16 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             disp += hdt * sqrtf(2.0f * __uint_as_float(sc.vmax2[b]));
             ++since;
             if (disp >= 0.99f * P.skin_half || (P.rebuild_every > 0 && since >= P.rebuild_every)) {
-                build_list<CL>(sm, sc, tp, P.rlist2, L);
+                build_list<CL>(sm, sc, P.rlist2);
                 disp = 0.f;
                 since = 0;
                 ++builds;
             }
             const bool save_next = save_phase == 0;
             if (save_next)
-                evaluate<ELEC, true, CL, TUBE>(sm, sc, tp, P, L, nb, true, rep.rep_id, step);
+                evaluate<ELEC, true, CL, TUBE>(sm, sc, P, nb, true, rep.rep_id, step);
             else
-                evaluate<ELEC, false, CL, TUBE>(sm, sc, tp, P, L, nb, true, rep.rep_id, step);
+                evaluate<ELEC, false, CL, TUBE>(sm, sc, P, nb, true, rep.rep_id, step);
             if (sc.status != 0) break;  // force out of range: frozen before the update
         }
     }
@@ -1355,9 +1449,9 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
     // write back the state (rank 0; every CTA holds the same copy)
     if (rank == 0) {
         for (int i = tid; i < n; i += blockDim.x) {
-            const float4 x = sm.xq[i];
+            const float4 x = get_x(sm, i);
             st.x[rep.atom_off + i] = make_float4(x.x, x.y, x.z, 0.f);
-            const float4 v = sm.v[i];
+            const float4 v = sm.v()[i];
             st.v[rep.atom_off + i] = make_float4(v.x, v.y, v.z, 0.f);
         }
         if (tid == 0) {
@@ -1386,30 +1480,28 @@ __global__ void __launch_bounds__(1024, 1)
 k_eval_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __restrict__ X,
               double* __restrict__ U, float* __restrict__ F, double* __restrict__ Z, int nta,
               int lc_cap) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Scalars sc;
-    const TopoDev tp = *topo_ptr;
-    Shared sm = carve(smem_raw, nta, lc_cap);
-    const int n = tp.n_atoms;
     const long long f = blockIdx.x / CL;
     const int rank = cta_rank<CL>();
-    const ListDev L = list_of(P.list_base + (blockIdx.x / CL) * P.list_slab, nta, rank);
+    if (threadIdx.x == 0) {
+        sc.tp = *topo_ptr;
+        sc.list = list_of(P.list_base + (blockIdx.x / CL) * P.list_slab, nta, rank);
+    }
+    __syncthreads();
+    const TopoDev& tp = sc.tp;
+    const Shared sm = {nta, lc_cap, tp.f_shift, tp.g_shift};
+    const int n = tp.n_atoms;
     const float* xf = X + f * n * 3;
-    for (int i = threadIdx.x; i < sm.na8; i += blockDim.x) {
+    for (int i = threadIdx.x; i < sm.na8(); i += blockDim.x) {
         if (i < n) {
-            sm.xq[i] = make_float4(xf[3 * i], xf[3 * i + 1], xf[3 * i + 2], tp.qs[i]);
-            sm.lj[i] = tp.lj[i];
+            put_x(sm, i, make_float4(xf[3 * i], xf[3 * i + 1], xf[3 * i + 2], tp.qs[i]));
+            put_lj(sm, i, tp.lj[i]);
         } else {
-            sm.xq[i] = far_slot(i);
-            sm.lj[i] = make_float2(0.f, 0.f);
+            put_x(sm, i, far_slot(i));
+            put_lj(sm, i, make_float2(0.f, 0.f));
         }
     }
-    for (int i = threadIdx.x; i < 3 * sm.na8; i += blockDim.x) {
-        sm.FH[0][i] = 0;
-        sm.FL[0][i] = 0u;
-        sm.GH[0][i] = 0;
-        sm.GL[0][i] = 0u;
-    }
+    for (int i = threadIdx.x; i < 24 * sm.na8(); i += blockDim.x) sm.F(0).L[i] = 0u;  // F and G
     if (threadIdx.x == 0) {
         sc.zm = 0.0;
         sc.z = 0.0;
@@ -1418,24 +1510,24 @@ k_eval_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __
         sc.work_next[0] = 0;
     }
     cluster_barrier<CL>();  // every CTA of the cluster is initialised before any remote access
-    build_list<CL>(sm, sc, tp, P.rlist2, L);
-    evaluate<ELEC, true, CL, false>(sm, sc, tp, P, L, 0, false, 0u, -1);
+    build_list<CL>(sm, sc, P.rlist2);
+    evaluate<ELEC, true, CL, false>(sm, sc, P, 0, false, 0u, -1);
     if (F) {  // evaluate ends with a cluster barrier: every partial is complete
         float* ff_out = F + f * n * 3;
-        const int s = sm.na8;
-        const int* oH = rank_ptr<CL>(sm.FH[0], rank ^ 1);
-        const unsigned* oL = rank_ptr<CL>(sm.FL[0], rank ^ 1);
+        const Part own = sm.F(0);
+        const int* oH = rank_ptr<CL>(own.H, rank ^ 1);
+        const unsigned* oL = rank_ptr<CL>(own.L, rank ^ 1);
         for (int i = threadIdx.x + rank * blockDim.x; i < n; i += CL * blockDim.x) {
             float o[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                int h = sm.FH[0][c * s + i];
-                long long l = (long long)sm.FL[0][c * s + i];
+                int h = own.H[3 * i + c];
+                unsigned l = own.L[3 * i + c];
                 if (CL == 2) {
-                    h += oH[c * s + i];
-                    l += (long long)oL[c * s + i];
+                    h += oH[3 * i + c];
+                    l += oL[3 * i + c];
                 }
-                o[c] = fix2f(((long long)h << 20) + l);
+                o[c] = fix2f(join_coarse(h, l, sm.fsh) * 128);  // 2^-13 to 2^-20 units
             }
             ff_out[3 * i] = o[0];
             ff_out[3 * i + 1] = o[1];
@@ -1450,8 +1542,8 @@ k_eval_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __
 }
 
 // Shared-memory bytes of the resident kernels for nta atom slots (plus the 8 sentinel
-// slots): positions, velocities, the xi array, LJ parameters and the two parities of force and
-// bias-gradient partials (integer and fraction words).
+// slots): positions with charges and LJ parameters, velocities, the xi array and the two
+// parities of force and bias-gradient partials (modular and coarse words).
 size_t resident_smem_bytes(int nta) {
     const size_t na8 = (size_t)nta + 8;
     return sizeof(float4) * (na8 + 2 * (size_t)nta) + sizeof(float2) * na8 +
@@ -1486,13 +1578,13 @@ size_t resident_smem_limit() {
     return (size_t)optin > stat ? (size_t)optin - stat : 0;
 }
 
-constexpr int kMaxCacheItems = 16384;
+constexpr int kMaxCacheItems = 8192;
 
 // Dynamic shared memory of a launch with CTAs of `threads` threads: the resident state plus
-// a cache of pair items (CacheItem, 32 B) in what the state leaves free; CTAs of up to 512
+// a cache of pair items (CacheItem, 64 B) in what the state leaves free; CTAs of up to 512
 // threads keep room for a second CTA on their SM. Sets *lc_cap to the cache's capacity.
 static size_t launch_smem(int nta, int threads, int cl, int* lc_cap) {
-    const int cl_items_per_slot = cl == 2 ? 2 : 4;
+    const int cl_items_per_slot = cl == 2 ? 1 : 2;
     const size_t base = resident_smem_bytes(nta);
     size_t lim = resident_smem_limit();
     if (threads <= 512) {
@@ -1507,7 +1599,7 @@ static size_t launch_smem(int nta, int threads, int cl, int* lc_cap) {
     }
     size_t cap = lim > base ? (lim - base) / sizeof(CacheItem) : 0;
     // no more than the lists of compact chains need (about 1.8 x 80 pairs per atom in items
-    // of 64, per CTA): shared memory and the L1 cache share the SM's storage, and the L1
+    // of 128, per CTA): shared memory and the L1 cache share the SM's storage, and the L1
     // serves the topology tables; longer tables stay in global memory
     cap = std::min(cap, std::min((size_t)kMaxCacheItems, (size_t)(cl_items_per_slot * nta)));
     *lc_cap = (int)cap;

@@ -290,6 +290,13 @@ int build_topology(scps_system* s, const scps_topology_desc& t, TopoHost& h) {
     td.n_angles = t.n_angles;
     td.ang_ijk = d_aijk;
     td.ang_par = d_apar;
+    // most terms one force partial can take: a pair term per other atom (each added alone on
+    // the slow path), one for the atom's own block, and its bonds and angles
+    std::vector<int> bonded(n, 0);
+    for (int b = 0; b < 2 * t.n_bonds; ++b) bonded[t.bonds[b]]++;
+    for (int a = 0; a < 3 * t.n_angles; ++a) bonded[t.angles[a]]++;
+    td.f_shift = coarse_shift((long long)n + 1 + *std::max_element(bonded.begin(), bonded.end()));
+    td.g_shift = coarse_shift(0);
     td.n_contacts = 0;
     td.con_ij = nullptr;
     td.con_C0 = nullptr;
@@ -831,6 +838,9 @@ int scps_set_bias(scps_system* s, const scps_bias_desc* b) {
                 off[pairs[c].x + 1]++;
                 off[pairs[c].y + 1]++;
             }
+            int con_max = 0;
+            for (int i = 0; i < n; ++i) con_max = std::max(con_max, off[i + 1]);
+            s->topos[t].dev.g_shift = coarse_shift(con_max);
             for (int i = 0; i < n; ++i) off[i + 1] += off[i];
             std::vector<int> fill(off.begin(), off.end() - 1);
             std::vector<int2> nbr((size_t)2 * nc);

@@ -90,6 +90,26 @@ __device__ __forceinline__ float fix2f(long long v) {
 }
 
 // ---------------------------------------------------------------------------
+// Two FP32 values per instruction (sm_100 and later). Each half is rounded as the scalar
+// operation would round it, so the packed forms give the same bits; the FMA pipe takes two
+// cycles for one of them, so its rate is the same and the issue slots halve (measured: 1.8
+// packed against 3.65 scalar warp instructions per clock and SM).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// 1/sqrt(x) with denormal x taken as zero: the bits of rsqrtf for every normal x, without
+// the rescaling that rsqrtf carries for denormal ones.
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// ---------------------------------------------------------------------------
 // float-float ("double-single") arithmetic (Dekker 1971; Knuth TwoSum;
 // FMA-based TwoProd). Used for the native-contact terms of z, whose 1e-9
 // relative budget is beyond FP32 while FP64 runs at 1/64 of the FP32 rate here.
@@ -251,6 +271,32 @@ __device__ __forceinline__ LJPair lj_pair(float sig, float eps24, const PairCons
     return q;
 }
 
+// Shifted-force pair energy phi(r) - phi(rc) + (r - rc) (-phi'(rc)) from the parts of the
+// force evaluation (inv_r = 1/r, s6 = (sigma/r)^6, c6 = (sigma/rc)^6, fc = -phi'(rc)).
+template <int ELEC>
+__device__ __forceinline__ float pair_e(float r2, float inv_r, float s6, float c6, float eps24,
+                                        float qq, float fc, const PairConst& pc) {
+    const float inv_r2 = inv_r * inv_r;
+    const float r = r2 * inv_r;
+    const float e_lj = eps24 * (1.0f / 6.0f) * (s6 * s6 - s6);
+    const float e_ljc = eps24 * (1.0f / 6.0f) * (c6 * c6 - c6);
+    float ec, ecc;
+    if (ELEC == ELEC_DDIEL) {
+        ec = 0.5f * qq * inv_r2;
+        ecc = 0.5f * qq * pc.inv_rc2;
+    } else if (ELEC == ELEC_RF) {
+        ec = qq * (inv_r + pc.krf * r2 - pc.crf);
+        ecc = 0.0f;  // the RF form already vanishes at r_c
+    } else if (ELEC == ELEC_PLAIN) {
+        ec = qq * inv_r;
+        ecc = qq * pc.inv_rc;
+    } else {
+        ec = 0.0f;
+        ecc = 0.0f;
+    }
+    return (e_lj - e_ljc) + (ec - ecc) + (r - pc.rc) * fc;
+}
+
 template <int ELEC, bool ENERGY>
 __device__ __forceinline__ float pair_s_lj(float r2, const LJPair& q, float qq, const PairConst& pc,
                                            float* e) {
@@ -276,28 +322,47 @@ __device__ __forceinline__ float pair_s_lj(float r2, const LJPair& q, float qq, 
     }
     // s = phi'(r)/r - phi'(rc)/r = -(a_lj inv_r2 + cr) + (a_ljc / rc + cc) inv_r
     const float s = fmaf(fmaf(q.a_ljc, pc.inv_rc, cc), inv_r, -fmaf(a_lj, inv_r2, cr));
-    if (ENERGY) {
-        // phi_sf(r) = phi(r) - phi(rc) + (r - rc) * (-phi'(rc))
-        const float r = r2 * inv_r;
-        const float e_lj = q.eps24 * (1.0f / 6.0f) * (s6 * s6 - s6);
-        const float e_ljc = q.eps24 * (1.0f / 6.0f) * (q.c6 * q.c6 - q.c6);
-        float ec, ecc;
-        if (ELEC == ELEC_DDIEL) {
-            ec = 0.5f * qq * inv_r2;
-            ecc = 0.5f * qq * pc.inv_rc2;
-        } else if (ELEC == ELEC_RF) {
-            ec = qq * (inv_r + pc.krf * r2 - pc.crf);
-            ecc = 0.0f;  // the RF form already vanishes at r_c
-        } else if (ELEC == ELEC_PLAIN) {
-            ec = qq * inv_r;
-            ecc = qq * pc.inv_rc;
-        } else {
-            ec = 0.0f;
-            ecc = 0.0f;
-        }
-        *e = (e_lj - e_ljc) + (ec - ecc) + (r - pc.rc) * fmaf(q.a_ljc, pc.inv_rc, cc);
-    }
+    if (ENERGY)
+        *e = pair_e<ELEC>(r2, inv_r, s6, q.c6, q.eps24, qq, fmaf(q.a_ljc, pc.inv_rc, cc), pc);
     return s;
+}
+
+// Two pairs at a time: returns -2^13 s of pair_s_lj for both and, when ENERGY, 2^13 times
+// their energies in *e (the 2^-13 fixed-point scale comes in with the caller's eps24 and qq,
+// the sign with the negated constants; both are exact), from the same operations in the same
+// order.
+template <int ELEC, bool ENERGY>
+__device__ __forceinline__ float2 pair_ms2(float2 r2, float2 sig, float2 eps24, float2 qq,
+                                           const PairConst& pc, float2* e) {
+    const float2 ir = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+    const float2 ir2 = mul2(ir, ir);
+    const float2 sig2 = mul2(sig, sig);
+    const float2 s2 = mul2(sig2, ir2);
+    const float2 s6 = mul2(mul2(s2, s2), s2);
+    const float2 a_lj = mul2(mul2(eps24, s6), fma2(dup2(2.0f), s6, dup2(-1.0f)));
+    const float2 c2 = mul2(sig2, dup2(pc.inv_rc2));
+    const float2 c6 = mul2(mul2(c2, c2), c2);
+    const float2 a_ljc = mul2(mul2(eps24, c6), fma2(dup2(2.0f), c6, dup2(-1.0f)));
+    float2 cr, ncc;  // coulomb part of -phi'(r)/r, and minus that of -phi'(r_c)
+    if (ELEC == ELEC_DDIEL) {
+        cr = mul2(mul2(qq, ir2), ir2);
+        ncc = mul2(qq, dup2(-pc.inv_rc3));
+    } else if (ELEC == ELEC_RF) {
+        cr = mul2(qq, fma2(ir2, ir, dup2(-2.0f * pc.krf)));
+        ncc = mul2(qq, dup2(-fmaf(pc.inv_rc2, 1.0f, -2.0f * pc.krf * pc.rc)));
+    } else if (ELEC == ELEC_PLAIN) {
+        cr = mul2(mul2(qq, ir2), ir);
+        ncc = mul2(qq, dup2(-pc.inv_rc2));
+    } else {
+        cr = dup2(0.0f);
+        ncc = dup2(-0.0f);
+    }
+    const float2 nfc = fma2(a_ljc, dup2(-pc.inv_rc), ncc);  // minus the force at r_c
+    if (ENERGY) {
+        e->x = pair_e<ELEC>(r2.x, ir.x, s6.x, c6.x, eps24.x, qq.x, -nfc.x, pc);
+        e->y = pair_e<ELEC>(r2.y, ir.y, s6.y, c6.y, eps24.y, qq.y, -nfc.y, pc);
+    }
+    return fma2(nfc, ir, fma2(a_lj, ir2, cr));
 }
 
 template <int ELEC, bool ENERGY>

@@ -39,7 +39,19 @@ struct TopoDev {
     const float* tube_A;       // tube bias: average contact maps <C(t'_k)>, stored [item of
                                // kTubeItem contacts][K][contact of the item], zero-padded
     float tube_inv_n0;         // tube bias: 1 / sum_p C0_p^2 (the norm of Eq. sX)
+    int f_shift, g_shift;      // coarse unit of the force / bias-gradient partials (coarse_shift)
 };
+
+// Partials of the resident chain kernels: each is a 32-bit sum modulo 2^32 of integer terms
+// and a signed coarse sum of round(term / 2^shift), which most terms leave at zero. The
+// coarse sum is within (number of terms) 2^(shift - 1) of the total, so that sum and the
+// modular one give the total exactly while that stays below 2^31 (see join_coarse). The
+// largest shift for which it does, up to 2^22 units (512 kJ mol^-1 nm^-1 of a force).
+inline int coarse_shift(long long max_terms) {
+    int shift = 22;
+    while (shift > 1 && max_terms << (shift - 1) >= 1ll << 31) --shift;
+    return shift;
+}
 
 constexpr int kMaxTubeK = 128;  // reference slices of the contact-map tube bias
 constexpr int kTubeItem = 8;    // contacts per work item of the tube passes (and of the
@@ -57,28 +69,31 @@ struct RepDev {
 };
 
 // Pair list of a chain replica in global memory (one slab per replica, laid out for a
-// launch with nta atom slots, nbs = nta / 8 blocks of 8 atoms):
+// launch with nta atom slots, nbs = nta / 8 blocks of 8 atoms; nbs is a multiple of 4):
 //   j entries (uint16): for block I, the atoms j of later blocks within the list radius
-//     of some atom of the block, ascending, padded to a multiple of 8 with the sentinel
-//     slot nta; block I owns 8 (nbs - 1 - I) entries from offset list_jl_off(nbs, I);
+//     of some atom of the block, ascending, padded to a multiple of kListChunk with the
+//     sentinel slot nta; block I owns room for its 8 (nbs - 1 - I) later atoms in whole
+//     chunks, from offset list_jl_off(nbs, I);
 //   item tables (uint32), one per CTA of a cluster: (I << 17 | near << 16 | chunk);
-//   exclusion masks (uint64), one per item of those tables: bit 8 s + t set when chunk entry s
-//     and block atom s ^ t form an excluded pair (items near their block only).
+//   exclusion masks (kListChunk bytes), one per item of those tables: bit a of byte s set when
+//     chunk entry s and block atom a form an excluded pair (items near their block only).
+constexpr int kListChunk = 16;
 __host__ __device__ __forceinline__ long long list_jl_off(int nbs, int I) {
-    return 8ll * ((long long)I * (nbs - 1) - (long long)I * (I - 1) / 2);
+    // sum over k < I of 16 ceil((nbs - 1 - k) / 2)
+    return 16ll * ((long long)I * (nbs >> 1) - ((long long)I * I >> 2));
 }
 __host__ __device__ __forceinline__ long long list_jl_bytes(int nbs) {
-    return ((2ll * 4ll * nbs * (nbs - 1)) + 15) & ~15ll;
+    return 2ll * list_jl_off(nbs, nbs) + 32;
 }
 __host__ __device__ __forceinline__ long long list_items_cap(int nbs) {
-    return (long long)nbs * (nbs - 1) / 2 + 8;
+    return (long long)nbs * nbs / 4 + 8;
 }
 __host__ __device__ __forceinline__ long long list_items_bytes(int nbs) {
     return (4 * list_items_cap(nbs) + 15) & ~15ll;
 }
 __host__ __device__ __forceinline__ long long list_slab_bytes(int nta) {
     const int nbs = nta / 8;
-    return list_jl_bytes(nbs) + 2 * list_items_bytes(nbs) + 2 * 8 * list_items_cap(nbs);
+    return list_jl_bytes(nbs) + 2 * list_items_bytes(nbs) + 2 * kListChunk * list_items_cap(nbs);
 }
 
 // Replica state and outputs (device pointers).
