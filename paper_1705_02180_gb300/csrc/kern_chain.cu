@@ -19,9 +19,9 @@
 // lies within r_list = r_c + skin of some atom of I, in chunks of 16 (the last one
 // padded with a far-away sentinel slot). A work item is one block against one
 // chunk (128 pairs) on a quarter warp: lane l keeps entries 2 l and 2 l + 1 of the chunk
-// and meets the four atom pairs of the block in xor order, two FP32 pairs per packed
-// operation, so the i-force accumulators move by xor exchanges while the j-forces stay in
-// place (64 replicas x 560 atoms: 22.4 us per step, against 26.7 with chunks of 8, one
+// and takes block atom l ^ t against both at its iteration t, two FP32 pairs per packed
+// operation, so the i-force accumulators move by one xor exchange per iteration while the
+// j-forces stay in place (64 replicas x 560 atoms: 21.8 us per step, against 26.7 with chunks of 8, one
 // entry per lane and scalar operations; the same bits). Pairs inside a block form 28-pair
 // items of their own. The list is rebuilt when a bound on the largest displacement
 // since the last build reaches skin/2, or after rebuild_every steps, so no pair
@@ -60,14 +60,6 @@ struct __align__(16) CacheItem {
     uint16_t j[kListChunk];
 };
 
-// Two neighbouring atom slots 2 m and 2 m + 1, as the packed FP32 operations take them:
-// positions, scaled charges and LJ parameters (s = sigma/2, e = sqrt(24 eps)).
-struct __align__(16) AtomPair {
-    float4 xy;  // (x0, x1, y0, y1)
-    float4 zq;  // (z0, z1, q0, q1)
-    float4 lj;  // (s0, s1, e0, e1)
-};
-
 // Partials of one kind and parity: per atom slot three modular words, then, after those of all
 // slots, three coarse words per slot (see red3).
 struct Part {
@@ -87,7 +79,10 @@ struct Shared {
     int lc_cap;    // capacity of lc in items
     int fsh, gsh;  // coarse units of the F and G partials (TopoDev)
     __device__ __forceinline__ int na8() const { return nta + 8; }
-    __device__ __forceinline__ AtomPair* pair() const { return (AtomPair*)smem_raw; }
+    // positions with scaled charges, nta + 8
+    __device__ __forceinline__ float4* xq() const { return (float4*)smem_raw; }
+    // LJ parameters (sigma/2, sqrt(24 eps)), nta + 8
+    __device__ __forceinline__ float2* lj() const { return (float2*)(smem_raw + 16 * na8()); }
     // velocities (w: 1/m), nta
     __device__ __forceinline__ float4* v() const { return (float4*)(smem_raw + 24 * na8()); }
     // noise of the next O half step per atom (sd times Gaussian numbers); w: the atom's
@@ -107,31 +102,6 @@ struct Shared {
         return (CacheItem*)(smem_raw + 120 * na8() + 32 * nta);
     }
 };
-
-// Position with charge, and LJ parameters, of atom slot i.
-__device__ __forceinline__ float* slot_of(const Shared& sm, int i) {
-    return (float*)(sm.pair() + (i >> 1)) + (i & 1);
-}
-__device__ __forceinline__ float4 get_x(const Shared& sm, int i) {
-    const float* a = slot_of(sm, i);
-    return make_float4(a[0], a[2], a[4], a[6]);
-}
-__device__ __forceinline__ void put_x(const Shared& sm, int i, float4 x) {
-    float* a = slot_of(sm, i);
-    a[0] = x.x;
-    a[2] = x.y;
-    a[4] = x.z;
-    a[6] = x.w;
-}
-__device__ __forceinline__ float2 get_lj(const Shared& sm, int i) {
-    const float* a = slot_of(sm, i);
-    return make_float2(a[8], a[10]);
-}
-__device__ __forceinline__ void put_lj(const Shared& sm, int i, float2 lj) {
-    float* a = slot_of(sm, i);
-    a[8] = lj.x;
-    a[10] = lj.y;
-}
 
 // List slab of this replica or frame (see scps_internal.h for the layout).
 struct ListDev {
@@ -208,12 +178,6 @@ __device__ __forceinline__ void red3_64(const Part& p, int k, long long vx, long
     atomicAdd(p.H + 3 * k + 2, (int)(((vz >> (sh - 1)) + 1) >> 1));
 }
 
-// The exact total of coarse and modular sums (see coarse_shift).
-__device__ __forceinline__ long long join_coarse(long long h, unsigned l, int sh) {
-    const long long c = h << sh;
-    return c + (long long)(int)(l - (unsigned)c);
-}
-
 // Slow path of a pair term: s13 d (2^-13 units, rounded exactly as on the fast path, so the
 // sums are the same integers whichever path a pair takes) to atom i and its negative to atom
 // j, in 64-bit; a non-finite term or one above 1e9 kJ/mol/nm raises the force-range flag.
@@ -274,109 +238,78 @@ __device__ __forceinline__ ListDev list_of(unsigned char* slab, int nta, int ran
     return L;
 }
 
-// One entry of an item against two block atoms (packed): adds the rounded terms to the
-// entry's sums fj and returns them for the block atoms. nx: exclusion bits of the two pairs.
-template <int ELEC, bool ENERGY, bool NEARX>
-__device__ __forceinline__ void pair_two(const PairConst& pc, float4 xy, float4 zq, float4 lj2,
-                                         float4 xj, float2 lj, unsigned nx, float lim, int2& tx,
-                                         int2& ty, int2& tz, bool& bad, long long& ei) {
-    const float2 dx = add2(dup2(xj.x), neg2(make_float2(xy.x, xy.y))),
-                 dy = add2(dup2(xj.y), neg2(make_float2(xy.z, xy.w))),
-                 dz = add2(dup2(xj.z), neg2(make_float2(zq.x, zq.y)));
-    const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-    bool ok0 = r2.x < pc.rc2, ok1 = r2.y < pc.rc2;
-    if (NEARX) {
-        ok0 = ok0 && !(nx & 1u);
-        ok1 = ok1 && !(nx & 2u);
-    }
-    float2 e;
-    float2 ms = pair_ms2<ELEC, ENERGY>(r2, add2(make_float2(lj2.x, lj2.y), dup2(lj.x)),
-                                       mul2(make_float2(lj2.z, lj2.w), dup2(lj.y)),
-                                       mul2(make_float2(zq.z, zq.w), dup2(xj.w)), pc, &e);
-    ms.x = ok0 ? ms.x : 0.0f;
-    ms.y = ok1 ? ms.y : 0.0f;
-    bad = bad || !(fabsf(ms.x) <= lim) || !(fabsf(ms.y) <= lim);
-    const float2 fx = mul2(ms, dx), fy = mul2(ms, dy), fz = mul2(ms, dz);
-    tx = make_int2(__float2int_rn(fx.x), __float2int_rn(fx.y));
-    ty = make_int2(__float2int_rn(fy.x), __float2int_rn(fy.y));
-    tz = make_int2(__float2int_rn(fz.x), __float2int_rn(fz.y));
-    if (ENERGY) {  // (e comes scaled by 2^13)
-        const float lim_e = kPairScale * kPairEMax, se = kPairEScale / kPairScale;
-        bad = bad || (ok0 && !(fabsf(e.x) < lim_e)) || (ok1 && !(fabsf(e.y) < lim_e));
-        ei += (ok0 ? __float2int_rn(e.x * se) : 0) + (ok1 ? __float2int_rn(e.y * se) : 0);
-    }
-}
-
 // The 128 pairs of one item (block I against a chunk of 16 list entries, of which this lane
-// holds j0 and j1) on a quarter warp, fast path: at iteration t lane l takes the block atoms
-// 2 m, 2 m + 1 with m = (l >> 1) ^ t against both entries, two pairs per packed operation.
-// The sums of the block atoms move by one xor exchange per iteration and component, those of
-// the entries stay in the lane; all are integers in 32-bit registers. Items near their block
-// (NEARX) take the excluded pairs from the masks xm (low byte entry j0, high byte j1). Returns
-// false (and adds nothing) when some |s| of the quarter warp exceeds pc.s_lim / 2, for which
-// the integer sums of the item (16 terms for a block atom) could overflow; the caller then
-// takes the slow path.
+// holds j0 and j1) on a quarter warp, fast path: at iteration t lane l takes block atom l ^ t
+// against both entries, the two pairs in one packed operation. The sums of the block atoms
+// move by one xor exchange per iteration and component, those of the entries stay in the
+// lane; all are integers in 32-bit registers. Items near their block (NEARX) take the excluded
+// pairs from the masks xm (low byte entry j0, high byte j1). Returns false (and adds nothing)
+// when some |s| of the quarter warp exceeds pc.s_lim / 2, for which the integer sums of the
+// item (16 terms for a block atom) could overflow; the caller then takes the slow path.
 //
-// Bound by the FMA pipe: about 33 packed operations per two pairs, and next to it the XU pipe
-// (two rsqrt, six conversions); two entries per lane halve the shared-memory loads and the
-// exchanges per pair, which would bind next.
+// Bound by the FMA pipe: 33 packed operations per two pairs, and next to it the XU pipe (two
+// rsqrt, six conversions, 2.1 clocks each). Packing the two entries, which stay in registers,
+// rather than two block atoms needs no register copies of (x, x) for the other operand: the
+// six operations that meet the block atom are scalar ones.
 template <int ELEC, bool ENERGY, bool NEARX>
 __device__ __forceinline__ bool pair_item_fast(const Shared& sm, const Part& F,
                                                const PairConst& pc, int I, int j0, int j1,
                                                unsigned xm, int lane, long long& e18) {
     const int l8 = lane & 7, q = lane >> 3;
-    float4 xa = get_x(sm, j0), xb = get_x(sm, j1);
-    float2 la = get_lj(sm, j0), lb = get_lj(sm, j1);
-    // the force scale goes in with the entry's eps and charge (a power of two: exact)
-    xa.w *= kPairScale;
-    xb.w *= kPairScale;
-    la.y *= kPairScale;
-    lb.y *= kPairScale;
+    const Entries n = pack_entries(sm.xq()[j0], sm.xq()[j1], sm.lj()[j0], sm.lj()[j1]);
     const float lim = 0.5f * kPairScale * pc.s_lim;
-    int2 fix = {0, 0}, fiy = {0, 0}, fiz = {0, 0};
+    int fix = 0, fiy = 0, fiz = 0;
     int fax = 0, fay = 0, faz = 0, fbx = 0, fby = 0, fbz = 0;
     long long ei = 0;
     bool bad = false;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int m = (l8 >> 1) ^ t;
-        const AtomPair& ap = sm.pair()[4 * I + m];
-        const float4 xy = ap.xy, zq = ap.zq, lj2 = ap.lj;
-        int2 ax, ay, az, bx, by, bz;
-        pair_two<ELEC, ENERGY, NEARX>(pc, xy, zq, lj2, xa, la, NEARX ? xm >> (2 * m) : 0u, lim, ax,
-                                      ay, az, bad, ei);
-        pair_two<ELEC, ENERGY, NEARX>(pc, xy, zq, lj2, xb, lb, NEARX ? xm >> (8 + 2 * m) : 0u, lim,
-                                      bx, by, bz, bad, ei);
+    for (int t = 0; t < 8; ++t) {
+        const int a = l8 ^ t, i = 8 * I + a;
+        const float4 xi = sm.xq()[i];
+        const float2 li = sm.lj()[i];
+        const float2 dx = make_float2(n.x.x - xi.x, n.x.y - xi.x),
+                     dy = make_float2(n.y.x - xi.y, n.y.y - xi.y),
+                     dz = make_float2(n.z.x - xi.z, n.z.y - xi.z);
+        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+        bool ok0 = r2.x < pc.rc2, ok1 = r2.y < pc.rc2;
+        if (NEARX) {
+            ok0 = ok0 && !((xm >> a) & 1u);
+            ok1 = ok1 && !((xm >> (8 + a)) & 1u);
+        }
+        const LJPair2 lj = lj_pair2(make_float2(li.x + n.s.x, li.x + n.s.y),
+                                    make_float2(li.y * n.e.x, li.y * n.e.y), pc);
+        float2 e;
+        float2 ms = pair_ms2<ELEC, ENERGY>(r2, lj, make_float2(xi.w * n.q.x, xi.w * n.q.y), pc, &e);
+        ms.x = ok0 ? ms.x : 0.0f;
+        ms.y = ok1 ? ms.y : 0.0f;
+        bad = bad || !(fabsf(ms.x) <= lim) || !(fabsf(ms.y) <= lim);
+        const float2 fx = mul2(ms, dx), fy = mul2(ms, dy), fz = mul2(ms, dz);
         // (the terms come out negated: they are the entries' share)
-        fax += ax.x + ax.y;
-        fay += ay.x + ay.y;
-        faz += az.x + az.y;
-        fbx += bx.x + bx.y;
-        fby += by.x + by.y;
-        fbz += bz.x + bz.y;
-        fix.x -= ax.x + bx.x;
-        fiy.x -= ay.x + by.x;
-        fiz.x -= az.x + bz.x;
-        fix.y -= ax.y + bx.y;
-        fiy.y -= ay.y + by.y;
-        fiz.y -= az.y + bz.y;
-        if (t < 3) {  // to the lane that takes these block atoms next
-            const int d = 2 * (t ^ (t + 1));
-            fix.x = __shfl_xor_sync(kFull, fix.x, d);
-            fiy.x = __shfl_xor_sync(kFull, fiy.x, d);
-            fiz.x = __shfl_xor_sync(kFull, fiz.x, d);
-            fix.y = __shfl_xor_sync(kFull, fix.y, d);
-            fiy.y = __shfl_xor_sync(kFull, fiy.y, d);
-            fiz.y = __shfl_xor_sync(kFull, fiz.y, d);
+        const int ax = __float2int_rn(fx.x), bx = __float2int_rn(fx.y);
+        const int ay = __float2int_rn(fy.x), by = __float2int_rn(fy.y);
+        const int az = __float2int_rn(fz.x), bz = __float2int_rn(fz.y);
+        if (ENERGY) {  // (e comes scaled by 2^13)
+            const float lim_e = kPairScale * kPairEMax, se = kPairEScale / kPairScale;
+            bad = bad || (ok0 && !(fabsf(e.x) < lim_e)) || (ok1 && !(fabsf(e.y) < lim_e));
+            ei += (ok0 ? __float2int_rn(e.x * se) : 0) + (ok1 ? __float2int_rn(e.y * se) : 0);
+        }
+        fax += ax;
+        fay += ay;
+        faz += az;
+        fbx += bx;
+        fby += by;
+        fbz += bz;
+        fix -= ax + bx;
+        fiy -= ay + by;
+        fiz -= az + bz;
+        if (t < 7) {  // the sums of block atom l8 ^ t go to the lane that takes it next
+            fix = __shfl_xor_sync(kFull, fix, t ^ (t + 1));
+            fiy = __shfl_xor_sync(kFull, fiy, t ^ (t + 1));
+            fiz = __shfl_xor_sync(kFull, fiz, t ^ (t + 1));
         }
     }
-    // lanes l and l ^ 1 hold shares of the same two block atoms: each keeps one of them
-    const bool odd = lane & 1;
-    const int kx = (odd ? fix.y : fix.x) + __shfl_xor_sync(kFull, odd ? fix.x : fix.y, 1);
-    const int ky = (odd ? fiy.y : fiy.x) + __shfl_xor_sync(kFull, odd ? fiy.x : fiy.y, 1);
-    const int kz = (odd ? fiz.y : fiz.x) + __shfl_xor_sync(kFull, odd ? fiz.x : fiz.y, 1);
     if ((__ballot_sync(kFull, bad) >> (8 * q)) & 0xffu) return false;
-    red3(F, 8 * I + (l8 ^ 6), kx, ky, kz, sm.fsh);
+    red3(F, 8 * I + (l8 ^ 7), fix, fiy, fiz, sm.fsh);  // lane l ends with atom l ^ 7's sums
     red3(F, j0, fax, fay, faz, sm.fsh);
     red3(F, j1, fbx, fby, fbz, sm.fsh);
     if (ENERGY) e18 += ei;
@@ -394,12 +327,12 @@ __device__ __noinline__ long long pair_item_slow(Shared sm, int b, Scalars* sc, 
     const TopoDev& tp = sc->tp;
     const PairConst& pc = P.pc;
     long long e18 = 0;
-    const float4 xj = get_x(sm, j);
-    const float2 lj = get_lj(sm, j);
+    const float4 xj = sm.xq()[j];
+    const float2 lj = sm.lj()[j];
     for (int t = 0; t < 8; ++t) {
         const int i = 8 * I + ((l8 + t) & 7);
-        const float4 xi = get_x(sm, i);
-        const float2 li = get_lj(sm, i);
+        const float4 xi = sm.xq()[i];
+        const float2 li = sm.lj()[i];
         const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         bool ok = r2 < pc.rc2;
@@ -464,8 +397,8 @@ __device__ __forceinline__ void diag_item(const Shared& sm, Scalars& sc, const P
     const int l8 = lane & 7, q = lane >> 3;
     const int src = (lane & 24) | ((l8 + 1) & 7);
     const int i = 8 * I + l8;
-    const float4 xa = get_x(sm, i);
-    const float2 la = get_lj(sm, i);
+    const float4 xa = sm.xq()[i];
+    const float2 la = sm.lj()[i];
     const unsigned long long em = i < tp.n_atoms ? tp.excl[i] : 0ull;
     int fax = 0, fay = 0, faz = 0, fbx = 0, fby = 0, fbz = 0;
     long long ei = 0;
@@ -473,8 +406,8 @@ __device__ __forceinline__ void diag_item(const Shared& sm, Scalars& sc, const P
 #pragma unroll
     for (int k = 1; k <= 4; ++k) {
         const int b = 8 * I + ((l8 + k) & 7);
-        const float4 xb = get_x(sm, b);
-        const float2 lb = get_lj(sm, b);
+        const float4 xb = sm.xq()[b];
+        const float2 lb = sm.lj()[b];
         const float dx = xb.x - xa.x, dy = xb.y - xa.y, dz = xb.z - xa.z;
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         const bool ok = r2 < pc.rc2 && (k < 4 || l8 < 4) && !((em >> (b - i + kExclWindow)) & 1ull);
@@ -510,8 +443,8 @@ __device__ __forceinline__ void diag_item(const Shared& sm, Scalars& sc, const P
     }
     for (int k = 1; k <= 4; ++k) {  // slow path (quarter-uniform)
         const int b = 8 * I + ((l8 + k) & 7);
-        const float4 xb = get_x(sm, b);
-        const float2 lb = get_lj(sm, b);
+        const float4 xb = sm.xq()[b];
+        const float2 lb = sm.lj()[b];
         const float dx = xb.x - xa.x, dy = xb.y - xa.y, dz = xb.z - xa.z;
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         if (!(r2 < pc.rc2 && (k < 4 || l8 < 4) && !((em >> (b - i + kExclWindow)) & 1ull))) continue;
@@ -533,7 +466,7 @@ __device__ __forceinline__ float bond_term(const Shared& sm, Scalars& sc, int pa
     int* flag = &sc.flag[par_];
     const int2 ij = tp.bond_ij[b];
     const float2 par = tp.bond_par[b];
-    const float4 a = get_x(sm, ij.x), c = get_x(sm, ij.y);
+    const float4 a = sm.xq()[ij.x], c = sm.xq()[ij.y];
     const float dx = c.x - a.x, dy = c.y - a.y, dz = c.z - a.z;
     const float r = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
     const float dr = r - par.x;
@@ -550,7 +483,7 @@ __device__ __forceinline__ float angle_term(const Shared& sm, Scalars& sc, int p
     int* flag = &sc.flag[par_];
     const int4 ijk = tp.ang_ijk[q];
     const float2 par = tp.ang_par[q];
-    const float4 a = get_x(sm, ijk.x), b = get_x(sm, ijk.y), c = get_x(sm, ijk.z);
+    const float4 a = sm.xq()[ijk.x], b = sm.xq()[ijk.y], c = sm.xq()[ijk.z];
     const float ux = a.x - b.x, uy = a.y - b.y, uz = a.z - b.z;
     const float wx = c.x - b.x, wy = c.y - b.y, wz = c.z - b.z;
     const float cx = uy * wz - uz * wy, cy = uz * wx - ux * wz, cz = ux * wy - uy * wx;
@@ -590,7 +523,7 @@ __device__ __forceinline__ void add_grad(const Shared& sm, int b, int i, int p, 
 __device__ __forceinline__ long long contact_term(const Shared& sm, const TopoDev& tp,
                                                   const RunParams& P, int par_, int c) {
     const int2 ij = tp.con_ij[c];
-    const float4 a = get_x(sm, ij.x), b = get_x(sm, ij.y);
+    const float4 a = sm.xq()[ij.x], b = sm.xq()[ij.y];
     const ff r2 = ff_dist2(a, b);
     const ff u = ff_mul(r2, P.inv_r0sq_ff);
     const ff C = contact_C_ff(u);
@@ -654,7 +587,7 @@ __device__ __forceinline__ void tube_pass1(const Shared& sm, const TopoDev& tp, 
     float C = 0.f;
     if (hl < nq) {
         const int2 ij = tp.con_ij[c0 + hl];
-        const float4 a = get_x(sm, ij.x), q = get_x(sm, ij.y);
+        const float4 a = sm.xq()[ij.x], q = sm.xq()[ij.y];
         const float dx = q.x - a.x, dy = q.y - a.y, dz = q.z - a.z;
         C = contact_C_f32(fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * P.inv_r0sq);
     }
@@ -736,7 +669,7 @@ __device__ __forceinline__ void tube_pass2(const Shared& sm, const Scalars& sc, 
     // every lane stays to the end (all exchanges above are full-warp); lanes >= nq
     // of a half hold a copy of its last contact and add nothing
     const bool live = hl < nq;
-    const float4 a = get_x(sm, ij.x), q = get_x(sm, ij.y);
+    const float4 a = sm.xq()[ij.x], q = sm.xq()[ij.y];
     const float dx = q.x - a.x, dy = q.y - a.y, dz = q.z - a.z;
     const float u = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) * P.inv_r0sq;
     const float C = contact_C_f32(u);
@@ -910,7 +843,7 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
         float4 lo = make_float4(3.0e38f, 3.0e38f, 3.0e38f, 0.f);
         float4 hi = make_float4(-3.0e38f, -3.0e38f, -3.0e38f, 0.f);
         for (int a = 8 * I; a < min(8 * I + 8, n); ++a) {
-            const float4 x = get_x(sm, a);
+            const float4 x = sm.xq()[a];
             lo.x = fminf(lo.x, x.x);
             lo.y = fminf(lo.y, x.y);
             lo.z = fminf(lo.z, x.z);
@@ -950,16 +883,13 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
                 const int j = Jc >= 0 ? 8 * Jc + (lane & 7) : n;
                 bool hit = false;  // within sqrt(rlist2) of some atom of the block
                 if (j < n) {
-                    const float4 xj = get_x(sm, j);
+                    const float4 xj = sm.xq()[j];
                     float dmin = 3.0e38f;
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) {  // (the padding slots of a last block are far)
-                        const float4 xy = sm.pair()[4 * I + m].xy, zq = sm.pair()[4 * I + m].zq;
-                        const float2 dx = add2(dup2(xj.x), neg2(make_float2(xy.x, xy.y))),
-                                     dy = add2(dup2(xj.y), neg2(make_float2(xy.z, xy.w))),
-                                     dz = add2(dup2(xj.z), neg2(make_float2(zq.x, zq.y)));
-                        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-                        dmin = fminf(dmin, fminf(r2.x, r2.y));
+                    for (int a = 0; a < 8; ++a) {  // (the padding slots of a last block are far)
+                        const float4 xa = sm.xq()[i0 + a];
+                        const float dx = xj.x - xa.x, dy = xj.y - xa.y, dz = xj.z - xa.z;
+                        dmin = fminf(dmin, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
                     }
                     hit = dmin < rlist2;
                 }
@@ -1272,13 +1202,13 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
     for (int i = tid; i < sm.na8(); i += blockDim.x) {
         if (i < n) {
             const float4 x = st.x[rep.atom_off + i];
-            put_x(sm, i, make_float4(x.x, x.y, x.z, tp.qs[i]));
-            put_lj(sm, i, tp.lj[i]);
+            sm.xq()[i] = make_float4(x.x, x.y, x.z, tp.qs[i]);
+            sm.lj()[i] = tp.lj[i];
             const float4 v = st.v[rep.atom_off + i];
             sm.v()[i] = make_float4(v.x, v.y, v.z, tp.inv_m[i]);
         } else {
-            put_x(sm, i, far_slot(i));
-            put_lj(sm, i, make_float2(0.f, 0.f));
+            sm.xq()[i] = far_slot(i);
+            sm.lj()[i] = make_float2(0.f, 0.f);
             if (i < nta) sm.v()[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
@@ -1357,7 +1287,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         fy += by;
                         fz += bz;
                     }
-                    float4 x = get_x(sm, i);
+                    float4 x = sm.xq()[i];
                     if (do_b) {  // B: closes the evaluated step
                         v.x = fmaf(hdt * im, fx, v.x);
                         v.y = fmaf(hdt * im, fy, v.y);
@@ -1388,7 +1318,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
                               isfinite(v.y) && isfinite(v.z)))
                             atomicOr(&sc.status, SCPS_FLAG_NONFINITE);
-                        put_x(sm, i, x);
+                        sm.xq()[i] = x;
                     }
                     sm.v()[i] = v;
                 }
@@ -1449,7 +1379,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
     // write back the state (rank 0; every CTA holds the same copy)
     if (rank == 0) {
         for (int i = tid; i < n; i += blockDim.x) {
-            const float4 x = get_x(sm, i);
+            const float4 x = sm.xq()[i];
             st.x[rep.atom_off + i] = make_float4(x.x, x.y, x.z, 0.f);
             const float4 v = sm.v()[i];
             st.v[rep.atom_off + i] = make_float4(v.x, v.y, v.z, 0.f);
@@ -1494,11 +1424,11 @@ k_eval_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __
     const float* xf = X + f * n * 3;
     for (int i = threadIdx.x; i < sm.na8(); i += blockDim.x) {
         if (i < n) {
-            put_x(sm, i, make_float4(xf[3 * i], xf[3 * i + 1], xf[3 * i + 2], tp.qs[i]));
-            put_lj(sm, i, tp.lj[i]);
+            sm.xq()[i] = make_float4(xf[3 * i], xf[3 * i + 1], xf[3 * i + 2], tp.qs[i]);
+            sm.lj()[i] = tp.lj[i];
         } else {
-            put_x(sm, i, far_slot(i));
-            put_lj(sm, i, make_float2(0.f, 0.f));
+            sm.xq()[i] = far_slot(i);
+            sm.lj()[i] = make_float2(0.f, 0.f);
         }
     }
     for (int i = threadIdx.x; i < 24 * sm.na8(); i += blockDim.x) sm.F(0).L[i] = 0u;  // F and G

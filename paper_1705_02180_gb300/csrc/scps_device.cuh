@@ -327,22 +327,33 @@ __device__ __forceinline__ float pair_s_lj(float r2, const LJPair& q, float qq, 
     return s;
 }
 
+// LJ constants of two pairs (see LJPair).
+struct LJPair2 {
+    float2 sig2, eps24, c6, a_ljc;
+};
+
+__device__ __forceinline__ LJPair2 lj_pair2(float2 sig, float2 eps24, const PairConst& pc) {
+    LJPair2 q;
+    q.sig2 = mul2(sig, sig);
+    q.eps24 = eps24;
+    const float2 c2 = mul2(q.sig2, dup2(pc.inv_rc2));
+    q.c6 = mul2(mul2(c2, c2), c2);
+    q.a_ljc = mul2(mul2(eps24, q.c6), fma2(dup2(2.0f), q.c6, dup2(-1.0f)));
+    return q;
+}
+
 // Two pairs at a time: returns -2^13 s of pair_s_lj for both and, when ENERGY, 2^13 times
 // their energies in *e (the 2^-13 fixed-point scale comes in with the caller's eps24 and qq,
 // the sign with the negated constants; both are exact), from the same operations in the same
 // order.
 template <int ELEC, bool ENERGY>
-__device__ __forceinline__ float2 pair_ms2(float2 r2, float2 sig, float2 eps24, float2 qq,
+__device__ __forceinline__ float2 pair_ms2(float2 r2, const LJPair2& q, float2 qq,
                                            const PairConst& pc, float2* e) {
     const float2 ir = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
     const float2 ir2 = mul2(ir, ir);
-    const float2 sig2 = mul2(sig, sig);
-    const float2 s2 = mul2(sig2, ir2);
+    const float2 s2 = mul2(q.sig2, ir2);
     const float2 s6 = mul2(mul2(s2, s2), s2);
-    const float2 a_lj = mul2(mul2(eps24, s6), fma2(dup2(2.0f), s6, dup2(-1.0f)));
-    const float2 c2 = mul2(sig2, dup2(pc.inv_rc2));
-    const float2 c6 = mul2(mul2(c2, c2), c2);
-    const float2 a_ljc = mul2(mul2(eps24, c6), fma2(dup2(2.0f), c6, dup2(-1.0f)));
+    const float2 a_lj = mul2(mul2(q.eps24, s6), fma2(dup2(2.0f), s6, dup2(-1.0f)));
     float2 cr, ncc;  // coulomb part of -phi'(r)/r, and minus that of -phi'(r_c)
     if (ELEC == ELEC_DDIEL) {
         cr = mul2(mul2(qq, ir2), ir2);
@@ -357,12 +368,50 @@ __device__ __forceinline__ float2 pair_ms2(float2 r2, float2 sig, float2 eps24, 
         cr = dup2(0.0f);
         ncc = dup2(-0.0f);
     }
-    const float2 nfc = fma2(a_ljc, dup2(-pc.inv_rc), ncc);  // minus the force at r_c
+    const float2 nfc = fma2(q.a_ljc, dup2(-pc.inv_rc), ncc);  // minus the force at r_c
     if (ENERGY) {
-        e->x = pair_e<ELEC>(r2.x, ir.x, s6.x, c6.x, eps24.x, qq.x, -nfc.x, pc);
-        e->y = pair_e<ELEC>(r2.y, ir.y, s6.y, c6.y, eps24.y, qq.y, -nfc.y, pc);
+        e->x = pair_e<ELEC>(r2.x, ir.x, s6.x, q.c6.x, q.eps24.x, qq.x, -nfc.x, pc);
+        e->y = pair_e<ELEC>(r2.y, ir.y, s6.y, q.c6.y, q.eps24.y, qq.y, -nfc.y, pc);
     }
     return fma2(nfc, ir, fma2(a_lj, ir2, cr));
+}
+
+// The exact total of a coarse sum h (units of 2^sh) and a sum l modulo 2^32 (coarse_shift).
+__device__ __forceinline__ long long join_coarse(long long h, unsigned l, int sh) {
+    const long long c = h << sh;
+    return c + (long long)(int)(l - (unsigned)c);
+}
+
+constexpr float kIntMagic = 12582912.0f;  // 1.5 2^23: a + kIntMagic holds round(a), |a| < 2^22
+constexpr int kIntMagicBits = 0x4B400000;
+
+// Integers t + kIntMagicBits of two rounded values: one packed addition, and a conversion
+// only for the rare values beyond 2^22 units (512 kJ mol^-1 nm^-1 of a force).
+__device__ __forceinline__ int2 round2_biased(float2 v) {
+    const float2 m = add2(v, dup2(kIntMagic));
+    int2 r = make_int2(__float_as_int(m.x), __float_as_int(m.y));
+    if (!(fmaxf(fabsf(v.x), fabsf(v.y)) < 4194304.0f)) {  // (NaN only where the caller rejects it)
+        r.x = (int)((unsigned)__float2int_rn(v.x) + (unsigned)kIntMagicBits);
+        r.y = (int)((unsigned)__float2int_rn(v.y) + (unsigned)kIntMagicBits);
+    }
+    return r;
+}
+
+// Two list entries j of one lane, packed by component: positions, charges and sqrt(24 eps)
+// (both with the force scale 2^13, a power of two: exact), sigma / 2.
+struct Entries {
+    float2 x, y, z, q, s, e;
+};
+
+__device__ __forceinline__ Entries pack_entries(float4 a, float4 b, float2 la, float2 lb) {
+    Entries n;
+    n.x = make_float2(a.x, b.x);
+    n.y = make_float2(a.y, b.y);
+    n.z = make_float2(a.z, b.z);
+    n.q = make_float2(a.w * kPairScale, b.w * kPairScale);
+    n.s = make_float2(la.x, lb.x);
+    n.e = make_float2(la.y * kPairScale, lb.y * kPairScale);
+    return n;
 }
 
 template <int ELEC, bool ENERGY>
