@@ -12,7 +12,7 @@
 //                        its atoms, each with the periodic shift of its cluster
 //                        (the cluster takes the minimum image pair by pair where
 //                        that shift might not hold until the next rebuild)
-//   pairs                one warp per cluster, four chunks of 8 entries at a
+//   pairs                one warp per cluster, 64 list entries at a
 //                        time on quarter warps, every pair once; all force
 //                        terms summed in fixed point (order-free)
 //   chain                one CTA per replica: bonds, angles, z(X) of Eq.
@@ -34,6 +34,12 @@ constexpr unsigned kFullB = 0xffffffffu;
 constexpr int kNumKeys = 8192;  // ncol^2 * nz <= kNumKeys
 constexpr int kMaxCols = 256;   // ncol <= 16
 constexpr int kSortThreads = 1024;
+// k_box_pairs: warps (clusters) per CTA and warps per SM. One warp per CTA: the lists of a
+// tile's clusters differ in length, and warps of one CTA would wait for the longest (16 x
+// 24 560 sites: 388 us against 423 with four). 20 warps leave 96 registers each; 24 and 28
+// take 398 and 408 us, since the kernel is bound by its instruction mix, not by latency.
+constexpr int kPairWarps = 1;
+constexpr int kPairRegWarps = 20;
 
 __device__ __forceinline__ float wrapc(float x, float L, float invL) {
     return x - L * floorf(x * invL);
@@ -41,6 +47,13 @@ __device__ __forceinline__ float wrapc(float x, float L, float invL) {
 
 __device__ __forceinline__ float min_img(float d, float L, float invL) {
     return d - L * rintf(d * invL);
+}
+
+// The same for two differences (rint by the addition that drops the fraction bits, exact for
+// quotients below 2^22).
+__device__ __forceinline__ float2 min_img2(float2 d, float L, float invL) {
+    const float2 q = add2(mul2(d, dup2(invL)), dup2(12582912.0f));
+    return fma2(dup2(-L), add2(q, dup2(-12582912.0f)), d);
 }
 
 // number of lanes whose (key, lane) is below this lane's
@@ -478,88 +491,146 @@ __global__ void __launch_bounds__(128) k_box_list(BoxDev B, StateDev st, int r0)
     }
 }
 
-// The 64 pairs of one chunk (8 list entries) with the 8 atoms of the i cluster, on a quarter
-// warp: lane l holds entry j_l; at iteration t it takes cluster atom l ^ t, so the i-force
-// sums move by one xor exchange per iteration (after the eighth, xor 7, lane l holds atom
-// l's again) while the j force stays in the lane. Each pair term s (x_j - x_i) is rounded to
-// 2^-13 units and summed in 32-bit registers. FIRST: quarter 0 holds the cluster's own
-// slots, whose pairs count once (j slot after i slot). EXCL: exclusion masks (clusters holding chain atoms); MINIMG:
-// per-pair minimum image; FAST: every atom has the reference LJ parameters, whose pair
-// constants U are computed once. Returns false for the quarters where some |s| exceeds
-// pc.s_lim (their 32-bit sums could overflow; the caller redoes those chunks pair by pair).
-template <int ELEC, bool ENERGY, bool EXCL, bool MINIMG, bool FAST, bool FIRST>
-__device__ __forceinline__ bool box_chunk(const BoxDev& B, const PairConst& pc, const LJPair& U,
-                                          const float4* sx, const float2* sp, const int* sid,
-                                          const unsigned long long* sem, float4 xj, float2 lj,
-                                          int idj, int lane, int& fix, int& fiy, int& fiz,
-                                          int& fjx, int& fjy, int& fjz, long long& e18) {
+// The i cluster of a warp in shared memory.
+struct BoxCluster {
+    float4 x[8];  // (x, y, z, qs)
+    float2 lj[8];
+    int id[8];
+    unsigned long long ex[8];  // exclusion masks of its chain atoms
+};
+
+// Adds an integer vector (2^-13 units) to the force sums of slot s (acc: the replica's three
+// modular, then three coarse arrays of np words); the coarse words only when a component rounds
+// to a non-zero multiple of 2^kBoxShift. (Six words per slot side by side, which need fewer
+// address computations, touch more sectors per atomic: 409 against 388 us.)
+__device__ __forceinline__ void box_red3(const BoxDev& B, unsigned* acc, int s, int vx, int vy, int vz) {
+    unsigned* L = acc + s;
+    const size_t np = (size_t)B.np;
+    atomicAdd(L, (unsigned)vx);
+    atomicAdd(L + np, (unsigned)vy);
+    atomicAdd(L + 2 * np, (unsigned)vz);
+    const unsigned half = 1u << (kBoxShift - 1);
+    if ((((unsigned)vx + half) | ((unsigned)vy + half) | ((unsigned)vz + half)) >> kBoxShift) {
+        int* H = (int*)L + 3 * np;
+        const int hx = ((vx >> (kBoxShift - 1)) + 1) >> 1, hy = ((vy >> (kBoxShift - 1)) + 1) >> 1,
+                  hz = ((vz >> (kBoxShift - 1)) + 1) >> 1;
+        if (hx) atomicAdd(H, hx);
+        if (hy) atomicAdd(H + np, hy);
+        if (hz) atomicAdd(H + 2 * np, hz);
+    }
+}
+
+// The same for one 64-bit component (d = 0, 1, 2).
+__device__ __forceinline__ void box_red64(const BoxDev& B, unsigned* acc, int s, int d, long long v) {
+    unsigned* L = acc + s + d * (size_t)B.np;
+    atomicAdd(L, (unsigned)v);
+    const int h = (int)(((v >> (kBoxShift - 1)) + 1) >> 1);
+    if (h) atomicAdd((int*)L + 3 * (size_t)B.np, h);
+}
+
+// The pairs of two list entries per lane with the 8 atoms of the i cluster: at iteration t
+// lane l takes cluster atom (l & 7) ^ t against both entries, the two pairs in one packed
+// operation. The i sums move by one xor exchange per iteration and component inside a quarter
+// warp and come home with the last (fi, lane l: atom l & 7; with the entries' sign); the j sums
+// stay in the lane (fj). Each pair term s (x_j - x_i) is rounded to 2^-13 units and summed in
+// 32-bit registers. MASKED: bit a of the low (first entry) or second byte of xm leaves out the
+// pair with cluster atom a (the cluster's own slots, whose pairs count once, excluded pairs,
+// and with the per-pair minimum image, MINIMG, empty slots). FAST: every atom has the reference
+// LJ parameters, whose pair constants U are computed once. Returns false for the quarters where
+// some |s| exceeds pc.s_lim / 2 (their 32-bit sums of 16 terms could overflow; the caller
+// redoes them pair by pair).
+//
+// FAST takes 24 packed operations, two rsqrt and six roundings per two pairs; all roundings as
+// conversions would make the XU pipe (2.1 clocks an instruction) the bound, so z goes through
+// the FMA pipe instead.
+template <int ELEC, bool ENERGY, bool MASKED, bool MINIMG, bool FAST>
+__device__ __forceinline__ bool box_chunk(const BoxDev& B, const PairConst& pc, const LJPair2& U,
+                                          const BoxCluster& ci, const Entries& n, unsigned xm,
+                                          int lane, int* fi, int (*fj)[3], long long& e18) {
     const int l8 = lane & 7, q = lane >> 3;
+    const float lim = 0.5f * kPairScale * pc.s_lim;
+    int fx = 0, fy = 0, ax = 0, ay = 0, bx = 0, by = 0;
+    unsigned fz = 0u, az = 0u, bz = 0u;  // (z terms carry kIntMagicBits: sums modulo 2^32)
     long long ech = 0;
     bool bad = false;
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-        const int ii = l8 ^ t;
-        const float4 xi = sx[ii];
-        float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+        const int a = l8 ^ t;
+        const float4 xi = ci.x[a];
+        float2 dx = make_float2(n.x.x - xi.x, n.x.y - xi.x), dy = make_float2(n.y.x - xi.y, n.y.y - xi.y),
+               dz = make_float2(n.z.x - xi.z, n.z.y - xi.z);
         if (MINIMG) {
-            dx = min_img(dx, B.L, B.invL);
-            dy = min_img(dy, B.L, B.invL);
-            dz = min_img(dz, B.L, B.invL);
+            dx = min_img2(dx, B.L, B.invL);
+            dy = min_img2(dy, B.L, B.invL);
+            dz = min_img2(dz, B.L, B.invL);
         }
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        bool ok = r2 < pc.rc2;
-        if (FIRST) ok = ok && (q != 0 || l8 > ii);
-        if (MINIMG || EXCL) {
-            const int idi = sid[ii];
-            if (MINIMG) ok = ok && idj >= 0 && idi >= 0;
-            if (EXCL) {
-                const unsigned dj = (unsigned)(idj - idi + kExclWindow);
-                if (dj < 2u * kExclWindow && idj < B.n_chain) ok = ok && !((sem[ii] >> dj) & 1ull);
-            }
+        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+        bool ok0 = r2.x < pc.rc2, ok1 = r2.y < pc.rc2;
+        if (MASKED) {
+            ok0 = ok0 && !((xm >> a) & 1u);
+            ok1 = ok1 && !((xm >> (8 + a)) & 1u);
         }
-        float ep = 0.f, s;
-        if (FAST) {
-            s = pair_s_lj<ELEC, ENERGY>(r2, U, xi.w * xj.w, pc, &ep);
-        } else {
-            const float2 li = sp[ii];
-            s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &ep);
+        LJPair2 Q = U;
+        if (!FAST) {
+            const float2 li = ci.lj[a];
+            Q = lj_pair2(make_float2(li.x + n.s.x, li.x + n.s.y), make_float2(li.y * n.e.x, li.y * n.e.y), pc);
         }
-        s = ok ? s : 0.0f;
-        bad = bad || !(fabsf(s) <= pc.s_lim);
-        if (ENERGY) bad = bad || (ok && !(fabsf(ep) < kPairEMax));
-        const float s13 = s * kPairScale;
-        const int tx = __float2int_rn(s13 * dx), ty = __float2int_rn(s13 * dy),
-                  tz = __float2int_rn(s13 * dz);
-        fix += tx;
-        fiy += ty;
-        fiz += tz;
-        fjx -= tx;
-        fjy -= ty;
-        fjz -= tz;
-        if (ENERGY) ech += ok ? __float2int_rn(ep * kPairEScale) : 0;
-        const int m = t < 7 ? t ^ (t + 1) : 7;  // to the lane that takes atom l8 ^ t next
-        fix = __shfl_xor_sync(kFullB, fix, m);
-        fiy = __shfl_xor_sync(kFullB, fiy, m);
-        fiz = __shfl_xor_sync(kFullB, fiz, m);
+        float2 e;
+        float2 ms = pair_ms2<ELEC, ENERGY>(r2, Q, make_float2(xi.w * n.q.x, xi.w * n.q.y), pc, &e);
+        ms.x = ok0 ? ms.x : 0.0f;
+        ms.y = ok1 ? ms.y : 0.0f;
+        bad = bad || !(fabsf(ms.x) <= lim) || !(fabsf(ms.y) <= lim);
+        if (ENERGY) {  // (e comes scaled by 2^13)
+            const float lim_e = kPairScale * kPairEMax, se = kPairEScale / kPairScale;
+            bad = bad || (ok0 && !(fabsf(e.x) < lim_e)) || (ok1 && !(fabsf(e.y) < lim_e));
+            ech += (ok0 ? __float2int_rn(e.x * se) : 0) + (ok1 ? __float2int_rn(e.y * se) : 0);
+        }
+        const float2 tx = mul2(ms, dx), ty = mul2(ms, dy), tz = mul2(ms, dz);
+        const int cx = __float2int_rn(tx.x), dx_ = __float2int_rn(tx.y);
+        const int cy = __float2int_rn(ty.x), dy_ = __float2int_rn(ty.y);
+        const int2 iz = round2_biased(tz);
+        ax += cx;
+        ay += cy;
+        az += (unsigned)iz.x;
+        bx += dx_;
+        by += dy_;
+        bz += (unsigned)iz.y;
+        fx += cx + dx_;
+        fy += cy + dy_;
+        fz += (unsigned)iz.x + (unsigned)iz.y;
+        const int m = t < 7 ? t ^ (t + 1) : 7;  // to the lane that takes atom a next
+        fx = __shfl_xor_sync(kFullB, fx, m);
+        fy = __shfl_xor_sync(kFullB, fy, m);
+        fz = __shfl_xor_sync(kFullB, fz, m);
     }
+    // the biases of the z sums: 8 terms of an entry, 16 of a cluster atom
+    const unsigned bias8 = 8u * (unsigned)kIntMagicBits;
+    fi[0] = fx;
+    fi[1] = fy;
+    fi[2] = (int)(fz - 2u * bias8);
+    fj[0][0] = ax;
+    fj[0][1] = ay;
+    fj[0][2] = (int)(az - bias8);
+    fj[1][0] = bx;
+    fj[1][1] = by;
+    fj[1][2] = (int)(bz - bias8);
     const bool good = !((__ballot_sync(kFullB, bad) >> (8 * q)) & 0xffu);
     if (ENERGY && good) e18 += ech;
     return good;
 }
 
-// Slow path of one chunk (the quarter of a chunk that failed the fast path): every pair
-// term, rounded to 2^-13 units as on the fast path, goes to both slots' 64-bit
-// accumulators, so the forces are the same integers on either path.
-template <int ELEC, bool ENERGY, bool EXCL, bool MINIMG>
-__device__ __noinline__ void box_chunk_slow(const BoxDev& B, const PairConst& pc, const float4* sx,
-                                            const float2* sp, const int* sid,
-                                            const unsigned long long* sem, float4 xj, float2 lj,
-                                            int idj, int sj, int si0, bool first, int lane,
-                                            unsigned long long* acc, long long& e18) {
-    const int l8 = lane & 7, q = lane >> 3;
+// Slow path of the entries of a quarter that failed the fast path, one entry per lane: every
+// pair term, rounded to 2^-13 units as on the fast path, goes to both slots' sums in
+// 64-bit, so the forces are the same integers on either path.
+template <int ELEC, bool ENERGY, bool MINIMG>
+__device__ __noinline__ long long box_chunk_slow(const BoxDev& B, const PairConst& pc,
+                                                 const BoxCluster& ci, float4 xj, float2 lj, int sj,
+                                                 int si0, unsigned xm, unsigned* acc) {
+    const int l8 = threadIdx.x & 7;
+    long long e18 = 0;
     for (int t = 0; t < 8; ++t) {
         const int ii = (l8 + t) & 7;
-        const float4 xi = sx[ii];
+        const float4 xi = ci.x[ii];
         float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
         if (MINIMG) {
             dx = min_img(dx, B.L, B.invL);
@@ -567,117 +638,142 @@ __device__ __noinline__ void box_chunk_slow(const BoxDev& B, const PairConst& pc
             dz = min_img(dz, B.L, B.invL);
         }
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        bool ok = r2 < pc.rc2;
-        if (first) ok = ok && (q != 0 || l8 > ii);
-        const int idi = sid[ii];
-        if (MINIMG) ok = ok && idj >= 0 && idi >= 0;
-        if (EXCL) {
-            const unsigned dj = (unsigned)(idj - idi + kExclWindow);
-            if (dj < 2u * kExclWindow && idj < B.n_chain) ok = ok && !((sem[ii] >> dj) & 1ull);
-        }
-        if (!ok) continue;
+        if (!(r2 < pc.rc2) || ((xm >> ii) & 1u)) continue;
         float ep = 0.f;
-        const float2 li = sp[ii];
+        const float2 li = ci.lj[ii];
         const float s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &ep);
         const float s13 = s * kPairScale;
-        const long long tx = __float2ll_rn(s13 * dx) * 128, ty = __float2ll_rn(s13 * dy) * 128,
-                        tz = __float2ll_rn(s13 * dz) * 128;  // 2^-13 to 2^-20 units
-        const int si = si0 + ii;
-        const size_t np = (size_t)B.np;
-        atomicAdd(&acc[si], (unsigned long long)tx);
-        atomicAdd(&acc[np + si], (unsigned long long)ty);
-        atomicAdd(&acc[2 * np + si], (unsigned long long)tz);
-        atomicAdd(&acc[sj], (unsigned long long)(-tx));
-        atomicAdd(&acc[np + sj], (unsigned long long)(-ty));
-        atomicAdd(&acc[2 * np + sj], (unsigned long long)(-tz));
+        const long long tx = __float2ll_rn(s13 * dx), ty = __float2ll_rn(s13 * dy),
+                        tz = __float2ll_rn(s13 * dz);
+        box_red64(B, acc, si0 + ii, 0, tx);
+        box_red64(B, acc, si0 + ii, 1, ty);
+        box_red64(B, acc, si0 + ii, 2, tz);
+        box_red64(B, acc, sj, 0, -tx);
+        box_red64(B, acc, sj, 1, -ty);
+        box_red64(B, acc, sj, 2, -tz);
         if (ENERGY) e18 += __float2ll_rn(ep * kPairEScale);
     }
+    return e18;
 }
 
 // Non-bonded forces of one 8-slot i cluster on one warp, each pair once (Newton's third
-// law): its list in chunks of 8 entries, four chunks at a time (quarter q takes chunk
-// 4 k + q). After a chunk each lane adds its j sums to the entry's slot (three 64-bit
-// atomics, in 2^-20 units) and its i sums to 64-bit registers, which go to the cluster's
-// slots at the end, summed over the quarters. Entries carry their periodic shift unless
-// MINIMG; padding entries sit far away from everything (MINIMG tests ids instead).
+// law): its list 64 entries at a time, two per lane. After a chunk each lane adds its entries'
+// sums to their slots and its share of a cluster atom's sums to 64-bit registers, which go to
+// the cluster's slots at the end. Entries
+// carry their periodic shift unless MINIMG; padding entries sit far away from everything.
 template <int ELEC, bool ENERGY, bool EXCL, bool MINIMG>
 __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDev& tp,
                                                    const RunParams& P, int r, int c, int lane,
-                                                   bool ipure, const float4* sx, const float2* sp,
-                                                   const int* sid, const unsigned long long* sem) {
+                                                   bool ipure, const BoxCluster& ci) {
     const size_t base = (size_t)r * B.np;
-    const size_t ci = (size_t)r * 4 * B.nt + c;
-    const uint32_t* lst = B.ent + ci * B.max_ent;
-    const int n = B.nent[ci];
-    unsigned long long* acc = (unsigned long long*)(B.facc + 3 * base);
+    const size_t cl = (size_t)r * 4 * B.nt + c;
+    const uint32_t* lst = B.ent + cl * B.max_ent;
+    const int n = B.nent[cl];
+    unsigned* acc = B.facc + 6 * base;
     const float2 ref = tp.lj[B.n_atoms - 1];
-    const LJPair U = lj_pair(ref.x + ref.x, ref.y * ref.y, P.pc);
-    long long ax = 0, ay = 0, az = 0;  // this lane's share of cluster atom (lane & 7), 2^-13
+    const LJPair u1 = lj_pair(ref.x + ref.x, ref.y * ref.y, P.pc);
+    const LJPair2 U = {dup2(u1.sig2), dup2(u1.eps24 * kPairScale), dup2(u1.c6), dup2(u1.a_ljc * kPairScale)};
+    const int l8 = lane & 7;
+    unsigned empty = 0u;  // empty slots of the cluster
+    if (MINIMG) empty = __ballot_sync(kFullB, lane < 8 && ci.id[l8] < 0) & 0xffu;
+    long long ai[3] = {};  // minus this lane's share of cluster atom l8
     long long e18 = 0;
-    for (int k0 = 0; k0 < n; k0 += 32) {
-        const int k = k0 + lane;
-        const uint32_t e = k < n ? __ldg(lst + k) : (kBoxNoSlot | (1u << 30));
+    auto entry = [&](int k) -> uint32_t { return k < n ? __ldg(lst + k) : (kBoxNoSlot | (1u << 30)); };
+    auto position = [&](uint32_t e) -> float4 {
         const int sj = (int)(e & kBoxNoSlot);
-        const bool real = sj != (int)kBoxNoSlot;
-        float4 xj = make_float4(1.0e18f, 0.f, 0.f, 0.f);  // beyond any cutoff
-        float2 lj = make_float2(0.f, 0.f);
-        int idj = -1;
-        if (real) {
-            xj = B.pos[base + sj];
-            if (!MINIMG) {
-                xj.x = fmaf((float)((int)((e >> 24) & 3u) - 1), B.L, xj.x);
-                xj.y = fmaf((float)((int)((e >> 26) & 3u) - 1), B.L, xj.y);
-                xj.z = fmaf((float)((int)((e >> 28) & 3u) - 1), B.L, xj.z);
-            }
-            if (EXCL || MINIMG) idj = B.id[base + sj];  // ids serve exclusions and the image test
+        return sj != (int)kBoxNoSlot ? B.pos[base + sj]
+                                     : make_float4(1.0e18f, 0.f, 0.f, 0.f);  // beyond any cutoff
+    };
+    auto shifted = [&](uint32_t e, float4 x) -> float4 {
+        if (!MINIMG) {
+            x.x = fmaf((float)((int)((e >> 24) & 3u) - 1), B.L, x.x);
+            x.y = fmaf((float)((int)((e >> 26) & 3u) - 1), B.L, x.y);
+            x.z = fmaf((float)((int)((e >> 28) & 3u) - 1), B.L, x.z);
+        }
+        return x;
+    };
+    auto mask = [&](uint32_t e, int k) -> unsigned {
+        const int sj = (int)(e & kBoxNoSlot);
+        if (sj == (int)kBoxNoSlot) return MINIMG ? 0xffu : 0u;
+        unsigned m = k < 8 ? (0xffu << k) & 0xffu : 0u;  // own slots: j slot after i slot
+        if (MINIMG) m |= empty;
+        if (EXCL) {
+            const int idj = B.id[base + sj];
+            if (MINIMG && idj < 0) m = 0xffu;
+            if (idj >= 0 && idj < B.n_chain)
+                for (int a = 0; a < 8; ++a) {
+                    const unsigned dj = (unsigned)(idj - ci.id[a] + kExclWindow);
+                    if (dj < 2u * kExclWindow && ((ci.ex[a] >> dj) & 1ull)) m |= 1u << a;
+                }
+        }
+        return m;
+    };
+    auto entry_lj = [&](uint32_t e) {
+        const int sj = (int)(e & kBoxNoSlot);
+        return sj != (int)kBoxNoSlot ? B.par[base + sj] : make_float2(0.f, 0.f);
+    };
+    // the next chunk's positions and the entries after it are loaded before a chunk is computed
+    uint32_t en[2] = {entry(lane), entry(32 + lane)};
+    float4 xn[2] = {position(en[0]), position(en[1])};
+    uint32_t e2[2] = {entry(64 + lane), entry(96 + lane)};
+    for (int k0 = 0; k0 < n; k0 += 64) {
+        const uint32_t e[2] = {en[0], en[1]};
+        const float4 x[2] = {shifted(e[0], xn[0]), shifted(e[1], xn[1])};
+        float2 lj[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            en[k] = e2[k];
+            xn[k] = position(en[k]);
+            e2[k] = entry(k0 + 128 + 32 * k + lane);
         }
         bool fast = false;
-        if constexpr (!EXCL && !MINIMG) fast = __all_sync(kFullB, ipure && ((e >> 30) & 1u));
-        if (real && !fast) lj = B.par[base + sj];  // the fast path takes the reference constants
-        int fix = 0, fiy = 0, fiz = 0, fjx = 0, fjy = 0, fjz = 0;
+        if constexpr (!EXCL && !MINIMG) fast = __all_sync(kFullB, ipure && ((e[0] & e[1]) >> 30 & 1u));
+        if (!fast) {
+            lj[0] = entry_lj(e[0]);
+            lj[1] = entry_lj(e[1]);
+        }
+        const Entries en = pack_entries(x[0], x[1], lj[0], lj[1]);
+        unsigned xm = 0u;
+        if (EXCL || MINIMG || k0 == 0) xm = mask(e[0], k0 + lane) | (mask(e[1], k0 + 32 + lane) << 8);
+        int fi[3], fj[2][3];
         bool good;
-        if (k0 == 0) {
+        if (EXCL || MINIMG || k0 == 0) {
             if (fast)
-                good = box_chunk<ELEC, ENERGY, false, false, true, true>(
-                    B, P.pc, U, sx, sp, sid, sem, xj, lj, idj, lane, fix, fiy, fiz, fjx, fjy, fjz, e18);
+                good = box_chunk<ELEC, ENERGY, true, MINIMG, true>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
             else
-                good = box_chunk<ELEC, ENERGY, EXCL, MINIMG, false, true>(
-                    B, P.pc, U, sx, sp, sid, sem, xj, lj, idj, lane, fix, fiy, fiz, fjx, fjy, fjz, e18);
+                good = box_chunk<ELEC, ENERGY, true, MINIMG, false>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
         } else {
             if (fast)
-                good = box_chunk<ELEC, ENERGY, false, false, true, false>(
-                    B, P.pc, U, sx, sp, sid, sem, xj, lj, idj, lane, fix, fiy, fiz, fjx, fjy, fjz, e18);
+                good = box_chunk<ELEC, ENERGY, false, MINIMG, true>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
             else
-                good = box_chunk<ELEC, ENERGY, EXCL, MINIMG, false, false>(
-                    B, P.pc, U, sx, sp, sid, sem, xj, lj, idj, lane, fix, fiy, fiz, fjx, fjy, fjz, e18);
+                good = box_chunk<ELEC, ENERGY, false, MINIMG, false>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
         }
         if (good) {
-            ax += fix;
-            ay += fiy;
-            az += fiz;
-            if (real) {
-                atomicAdd(&acc[sj], (unsigned long long)((long long)fjx * 128));
-                atomicAdd(&acc[B.np + sj], (unsigned long long)((long long)fjy * 128));
-                atomicAdd(&acc[2 * (size_t)B.np + sj], (unsigned long long)((long long)fjz * 128));
+#pragma unroll
+            for (int d = 0; d < 3; ++d) ai[d] += fi[d];
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int sj = (int)(e[k] & kBoxNoSlot);
+            if (sj == (int)kBoxNoSlot) continue;
+            if (good) {
+                box_red3(B, acc, sj, fj[k][0], fj[k][1], fj[k][2]);
+            } else {  // (the slow path uses the general form)
+                e18 += box_chunk_slow<ELEC, ENERGY, MINIMG>(B, P.pc, ci, shifted(e[k], position(e[k])),
+                                                           entry_lj(e[k]), sj, 8 * c,
+                                                           (xm >> (8 * k)) & 0xffu, acc);
             }
-        } else {
-            if (real && fast) lj = B.par[base + sj];  // the slow path uses the general form
-            box_chunk_slow<ELEC, ENERGY, EXCL, MINIMG>(B, P.pc, sx, sp, sid, sem, xj, lj, idj, sj,
-                                                      8 * c, k0 == 0, lane, acc, e18);
         }
     }
     // the four quarters' shares of each cluster atom
-    ax += __shfl_xor_sync(kFullB, ax, 8);
-    ay += __shfl_xor_sync(kFullB, ay, 8);
-    az += __shfl_xor_sync(kFullB, az, 8);
-    ax += __shfl_xor_sync(kFullB, ax, 16);
-    ay += __shfl_xor_sync(kFullB, ay, 16);
-    az += __shfl_xor_sync(kFullB, az, 16);
-    if (lane < 8 && sid[lane] >= 0) {
-        const int si = 8 * c + lane;
-        atomicAdd(&acc[si], (unsigned long long)(ax * 128));
-        atomicAdd(&acc[B.np + si], (unsigned long long)(ay * 128));
-        atomicAdd(&acc[2 * (size_t)B.np + si], (unsigned long long)(az * 128));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ai[d] += __shfl_xor_sync(kFullB, ai[d], 8);
+        ai[d] += __shfl_xor_sync(kFullB, ai[d], 16);
+    }
+    if (lane < 8 && ci.id[lane] >= 0) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) box_red64(B, acc, 8 * c + lane, d, -ai[d]);
     }
     if (ENERGY) {
 #pragma unroll
@@ -688,45 +784,45 @@ __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDe
 
 // Non-bonded forces: one warp per 8-slot i cluster, the variant chosen by its flags.
 template <int ELEC, bool ENERGY>
-__global__ void __launch_bounds__(128, 8) k_box_pairs(BoxDev B, const TopoDev* __restrict__ topo,
-                                                   RunParams P, int r0) {
-    __shared__ float4 sx[4][8];
-    __shared__ float2 sp[4][8];
-    __shared__ int sid[4][8];
-    __shared__ unsigned long long sem[4][8];
+__global__ void __launch_bounds__(32 * kPairWarps, kPairRegWarps / kPairWarps) k_box_pairs(BoxDev B, const TopoDev* __restrict__ topo,
+                                                                 RunParams P, int r0) {
+    __shared__ BoxCluster ci[kPairWarps];
     const int r = blockIdx.y + r0;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c = blockIdx.x * 4 + w;
+    const int c = blockIdx.x * kPairWarps + w;
     if (c >= 4 * B.nt) return;
     const TopoDev& tp = *topo;
     if (lane < 8) {
         const size_t sl = (size_t)r * B.np + 8 * c + lane;
-        sx[w][lane] = B.pos[sl];
-        sp[w][lane] = B.par[sl];
+        ci[w].x[lane] = B.pos[sl];
+        ci[w].lj[lane] = B.par[sl];
         const int a = B.id[sl];
-        sid[w][lane] = a;
-        sem[w][lane] = (a >= 0 && a < B.n_chain) ? tp.excl[a] : 0ull;
+        ci[w].id[lane] = a;
+        ci[w].ex[lane] = (a >= 0 && a < B.n_chain) ? tp.excl[a] : 0ull;
     }
     __syncwarp();
     const int fl = B.cflag[(size_t)r * 4 * B.nt + c];
     const bool pure = (fl & 4) != 0;
     switch (fl & 3) {
-        case 0: box_cluster_forces<ELEC, ENERGY, false, false>(B, tp, P, r, c, lane, pure, sx[w], sp[w], sid[w], sem[w]); break;
-        case 1: box_cluster_forces<ELEC, ENERGY, true, false>(B, tp, P, r, c, lane, pure, sx[w], sp[w], sid[w], sem[w]); break;
-        default: box_cluster_forces<ELEC, ENERGY, true, true>(B, tp, P, r, c, lane, pure, sx[w], sp[w], sid[w], sem[w]); break;
+        case 0: box_cluster_forces<ELEC, ENERGY, false, false>(B, tp, P, r, c, lane, pure, ci[w]); break;
+        case 1: box_cluster_forces<ELEC, ENERGY, true, false>(B, tp, P, r, c, lane, pure, ci[w]); break;
+        default: box_cluster_forces<ELEC, ENERGY, true, true>(B, tp, P, r, c, lane, pure, ci[w]); break;
     }
 }
 
 // Total non-bonded force on slot s of replica r (fixed point), which is cleared for the
 // next evaluation.
 __device__ __forceinline__ float4 take_nb_force(const BoxDev& B, int r, int s) {
-    const size_t base = (size_t)r * B.np;
-    long long* acc = B.facc + 3 * base;
-    float4 f = make_float4(fix2f(acc[s]), fix2f(acc[B.np + s]), fix2f(acc[2 * B.np + s]), 0.f);
-    acc[s] = 0;
-    acc[B.np + s] = 0;
-    acc[2 * B.np + s] = 0;
-    return f;
+    const size_t np = (size_t)B.np;
+    unsigned* L = B.facc + 6 * (size_t)r * np + s;
+    float f[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {  // 2^-13 to 2^-20 units
+        f[d] = fix2f(join_coarse((int)L[(3 + d) * np], L[d * np], kBoxShift) * 128);
+        L[d * np] = 0u;
+        L[(3 + d) * np] = 0u;
+    }
+    return make_float4(f[0], f[1], f[2], 0.f);
 }
 
 // Chain terms of one replica: bonds, angles (minimum image), z and the ratchet,
@@ -1014,13 +1110,13 @@ static void box_rebuild(const BoxDev& B, const TopoDev* topo, const StateDev& st
 // Pair forces of replicas [r0, r0 + nr).
 static void box_pairs_launch(const BoxDev& B, const TopoDev* topo, const RunParams& P, int r0, int nr,
                              int elec, bool energy, cudaStream_t s) {
-    const dim3 gg((4 * B.nt + 3) / 4, nr);
+    const dim3 gg((4 * B.nt + kPairWarps - 1) / kPairWarps, nr);
 #define PAIRS(E)                                                                                \
     switch (elec) {                                                                             \
-        case ELEC_DDIEL: k_box_pairs<ELEC_DDIEL, E><<<gg, 128, 0, s>>>(B, topo, P, r0); break;  \
-        case ELEC_RF: k_box_pairs<ELEC_RF, E><<<gg, 128, 0, s>>>(B, topo, P, r0); break;        \
-        case ELEC_PLAIN: k_box_pairs<ELEC_PLAIN, E><<<gg, 128, 0, s>>>(B, topo, P, r0); break;  \
-        default: k_box_pairs<ELEC_NONE, E><<<gg, 128, 0, s>>>(B, topo, P, r0); break;           \
+        case ELEC_DDIEL: k_box_pairs<ELEC_DDIEL, E><<<gg, 32 * kPairWarps, 0, s>>>(B, topo, P, r0); break;  \
+        case ELEC_RF: k_box_pairs<ELEC_RF, E><<<gg, 32 * kPairWarps, 0, s>>>(B, topo, P, r0); break;        \
+        case ELEC_PLAIN: k_box_pairs<ELEC_PLAIN, E><<<gg, 32 * kPairWarps, 0, s>>>(B, topo, P, r0); break;  \
+        default: k_box_pairs<ELEC_NONE, E><<<gg, 32 * kPairWarps, 0, s>>>(B, topo, P, r0); break;           \
     }
     if (energy) {
         PAIRS(true)

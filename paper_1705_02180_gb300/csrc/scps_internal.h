@@ -158,8 +158,9 @@ struct BoxDev {
     float2* par;      // (sigma/2, sqrt(24 eps))
     int* id;          // atom id of each slot, -1 for padding
     int* id2;         // sort buffer of id
-    long long* facc;  // [replica][3][np] non-bonded force on the slot, fixed point 2^-20
-                      // (order-free sums; cleared by whoever consumes it)
+    unsigned* facc;   // [replica][6][np] non-bonded force on the slot: three sums modulo 2^32 of
+                      // 2^-13 units, then three coarse sums (int) in units of 2^kBoxShift
+                      // (order-free; cleared by whoever consumes them)
     long long* epair; // [replica] pair energy of energy evaluations, fixed point 2^-18
                       // (cleared by whoever consumes it)
     float4* pos2;     // sort buffers
@@ -190,6 +191,7 @@ struct BoxDev {
     double* eb;       // [replica] bonded energy (save steps)
 };
 
+constexpr int kBoxShift = 21;  // a slot takes at most 2047 chunk sums (join_coarse stays exact)
 constexpr uint32_t kBoxNoSlot = 0x7fffffu;  // padding entry of a box pair list
 
 // Step graphs of the periodic box (variants: regular, last step of a call, save step, save
