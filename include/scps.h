@@ -126,9 +126,9 @@ typedef struct {
     int32_t max_frames;     /* frames kept per replica (the oldest are overwritten) */
     /* execution */
     int32_t exec;           /* SCPS_EXEC_* */
-    int32_t cluster_size;   /* CTAs per replica in RESIDENT form: 0 = auto, 1 or 2 */
+    int32_t cluster_size;   /* CTAs per replica in RESIDENT form: 0 = auto (1, 2 or 4), 1 or 2 */
     int32_t threads;        /* threads per CTA in RESIDENT form: 0 = auto, else 128..1024
-                               (at most 768 with cluster_size 2) */
+                               (at most 768 in a cluster of CTAs) */
     int32_t steps_per_graph;/* device-loop steps per CUDA-graph node: 0 = auto */
     /* pair lists */
     double skin;            /* list buffer r_list - r_c (nm); 0 = default (0.15 for the periodic

@@ -20,6 +20,7 @@
 namespace scps {
 size_t resident_smem_bytes(int nta);
 size_t resident_smem_limit();
+int chain_max_clusters(int cl, int nta, int threads);
 size_t box_chain_smem_limit();
 size_t box_chain_smem(int n_chain, int n_contacts);
 cudaError_t launch_resident(int elec, int cluster, const TopoDev* topos, const RepDev* reps,
@@ -328,6 +329,30 @@ void drop_graphs(scps_system* s) {
     s->graph_defs.clear();
 }
 
+// CTAs per replica when the caller leaves the choice open: two while they leave no SM without a
+// replica of its own; four where the replicas are few enough for all clusters to run at once
+// and large enough to gain from it (us per step, one to twenty replicas: 1200 atoms 37.9
+// against 47.7 with two, 560 atoms 18.0 against 20.8, 304 atoms 11.0 against 11.1; a second
+// wave of clusters would double the time, and eight CTAs lose to the reads of each other's
+// partials: 46.7, 25.3 and 15.6).
+int auto_cluster(int R, int nta, int n_sm, int threads) {
+    if (threads > kMaxThreadsPair || 2 * R > n_sm) return 1;
+    if (nta >= 448 && 4 * R <= n_sm &&
+        R <= chain_max_clusters(4, nta, threads ? threads : kMaxThreadsPair))
+        return 4;
+    return 2;
+}
+
+// CTAs per frame of a frame evaluation: two while they fit the SMs, four and eight only well
+// below that, since a cluster needs its SMs in one GPC (3 frames of 1199 atoms: 67, 51 and 47
+// us with two, four and eight; 9 frames of 560: 39, 35, 33; 20 of 304: 29, 26, 30; 50 of 560:
+// 42, 48, 76).
+int eval_cluster(long long nf, int n_sm) {
+    if (10 * nf <= n_sm) return 8;
+    if (5 * nf <= n_sm) return 4;
+    return 2 * nf <= n_sm ? 2 : 1;
+}
+
 int tile_atoms(int n) { return ((n + kTile - 1) / kTile) * kTile; }
 
 // Launch groups of the resident form. plan 0: one group, replicas by decreasing
@@ -335,8 +360,8 @@ int tile_atoms(int n) { return ((n + kTile - 1) / kTile) * kTile; }
 // group per size class (tile-rounded atom count), each with shared memory for its
 // own size. Every group gets the given cluster size and threads per CTA.
 int set_groups(scps_system* s, int plan, int cluster, int threads) {
-    if (cluster == 2 && threads > kMaxThreadsPair)
-        return fail(SCPS_ERR_INVALID_ARG, "a 2-CTA cluster takes at most %d threads per CTA",
+    if (cluster > 1 && threads > kMaxThreadsPair)
+        return fail(SCPS_ERR_INVALID_ARG, "a CTA cluster takes at most %d threads per CTA",
                     kMaxThreadsPair);
     const int R = s->d.n_replicas;
     std::vector<int> order(R);
@@ -593,13 +618,13 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
         if (rc) return bail(rc);
         int n_sm = 0;
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
-        // a 2-CTA cluster per replica when the replicas alone leave SMs idle
-        s->cluster = d->cluster_size
-                         ? d->cluster_size
-                         : (2 * R <= n_sm && d->threads <= kMaxThreadsPair ? 2 : 1);
+        s->cluster = d->cluster_size ? d->cluster_size
+                     : s->is_box || d->exec != SCPS_EXEC_RESIDENT
+                         ? (2 * R <= n_sm && d->threads <= kMaxThreadsPair ? 2 : 1)
+                         : auto_cluster(R, s->nta, n_sm, d->threads);
         const bool one_cta_per_sm = (long long)R * s->cluster <= n_sm;
         s->threads = d->threads ? d->threads : (one_cta_per_sm ? 1024 : auto_threads(s->nta));
-        if (s->cluster == 2 && !d->threads) s->threads = std::min(s->threads, kMaxThreadsPair);
+        if (s->cluster > 1 && !d->threads) s->threads = std::min(s->threads, kMaxThreadsPair);
         s->steps_per_graph = d->steps_per_graph > 0 ? d->steps_per_graph : 1000;
         if (!s->is_box && d->exec == SCPS_EXEC_RESIDENT) {
             const size_t smem = resident_smem_bytes(s->nta);
@@ -700,6 +725,7 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
     P.half_dt = (float)(0.5 * d->dt);
     P.c1 = (float)std::exp(-d->gamma * d->dt);
     P.gamma = d->gamma;
+    P.dt_over_gamma = (double)P.dt / P.gamma;
     P.key0 = (uint32_t)(d->seed & 0xffffffffull);
     P.key1 = (uint32_t)(d->seed >> 32);
     P.save_interval = d->save_interval;
@@ -1088,14 +1114,14 @@ int scps_energy_forces(scps_system* s, int32_t topo, int64_t n_frames, const flo
     }
     P.list_base = s->d_eval_lists;
     P.list_slab = s->eval_slab;
-    // few frames (a checkpoint segment): a 2-CTA cluster per frame, 1024 threads per CTA,
-    // so that the frames spread over the SMs; many frames: one CTA each
+    // few frames: a cluster of 1024-thread CTAs per frame, so that the frames spread over the
+    // SMs; many frames: one CTA each
     int n_sm = 0;
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
     const int n3 = 3 * th.n;
     for (long long f0 = 0; f0 < n_frames; f0 += per_launch) {
         const long long nf = std::min(per_launch, n_frames - f0);
-        const int cl = 2 * nf <= n_sm ? 2 : 1;
+        const int cl = eval_cluster(nf, n_sm);
         const int threads = nf * cl <= n_sm ? 1024 : auto_threads(nta);
         SCPS_CU(launch_eval(s->d.elec, s->d_topos + topo, P, X + f0 * n3, U + f0,
                             F ? F + f0 * n3 : nullptr, z ? z + f0 : nullptr, nf, nta, threads, cl,

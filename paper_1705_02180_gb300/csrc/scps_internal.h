@@ -56,7 +56,7 @@ inline int coarse_shift(long long max_terms) {
 constexpr int kMaxTubeK = 128;  // reference slices of the contact-map tube bias
 constexpr int kTubeItem = 8;    // contacts per work item of the tube passes (and of the
                                 // blocks in which the reference maps are stored)
-constexpr int kMaxThreadsPair = 768;  // threads per CTA of a 2-CTA cluster (80 registers each)
+constexpr int kMaxThreadsPair = 768;  // threads per CTA of a cluster (80 registers each)
 
 // Per-replica addressing.
 struct RepDev {
@@ -88,12 +88,16 @@ __host__ __device__ __forceinline__ long long list_jl_bytes(int nbs) {
 __host__ __device__ __forceinline__ long long list_items_cap(int nbs) {
     return (long long)nbs * nbs / 4 + 8;
 }
+// items of one CTA of a cluster of cl (item k goes to CTA k % cl)
+__host__ __device__ __forceinline__ long long list_items_part(int nbs, int cl) {
+    return list_items_cap(nbs) / cl + 2;
+}
 __host__ __device__ __forceinline__ long long list_items_bytes(int nbs) {
-    return (4 * list_items_cap(nbs) + 15) & ~15ll;
+    return (4 * (list_items_cap(nbs) + 16) + 31) & ~31ll;
 }
 __host__ __device__ __forceinline__ long long list_slab_bytes(int nta) {
     const int nbs = nta / 8;
-    return list_jl_bytes(nbs) + 2 * list_items_bytes(nbs) + 2 * kListChunk * list_items_cap(nbs);
+    return list_jl_bytes(nbs) + list_items_bytes(nbs) + kListChunk * (list_items_cap(nbs) + 16);
 }
 
 // Replica state and outputs (device pointers).
@@ -123,6 +127,7 @@ struct StateDev {
 struct RunParams {
     int n_replicas;
     float dt, half_dt, c1;        // c1 = exp(-gamma dt)
+    double dt_over_gamma;         // (FP32 dt) / gamma, the weight of the bias functional
     double k_R;
     int bias;                     // 0 none, 1 contacts, 2 toy
     float inv_r0sq;               // 1 / r0^2 (FP32)
