@@ -1,9 +1,11 @@
 // Hessian-vector products H(X_t) V_t of the physical potential, one cluster of CL
-// CTAs per frame (CL = 2 splits the block rows, bonds and angles between the two
-// CTAs; each then writes half of the atoms, summing its and the peer's partials). Used by
+// CTAs per frame (CL > 1 splits the block rows, bonds and angles between the
+// CTAs; each then writes its share of the atoms, summing the partials of all). Used by
 // the double backward of the energy (the gradient of sum_t |grad U(X_t)|^2 is
 // sum_t 2 H(X_t) grad U(X_t); the Onsager-Machlup action of Eq. (SOM) contains (grad U)^2).
-// Pairs come in items of two 8-atom blocks whose boxes lie within r_c, on quarter warps.
+// A warp takes a row of an 8-atom block I against up to 32 later blocks: the blocks whose
+// boxes lie within r_c, of these the atoms within r_c of some atom of I, and these 64 at a
+// time, two per lane, the two pairs of a lane in packed FP32 operations.
 //
 // For a pair term phi(r) with d = x_j - x_i and w = v_j - v_i:
 //   (Hv)_j = phi'' (d.w) d / r^2 + (phi'/r) (w - (d.w) d / r^2),  (Hv)_i = -(Hv)_j,
@@ -11,9 +13,12 @@
 // For an angle term k/2 (theta - theta0)^2:
 //   H v = k (grad theta . v) grad theta + k (theta - theta0) D_v(grad theta),
 // D_v being the directional derivative along v, written out by hand below.
-// Each item sums its j terms in FP32 in a fixed order (the i terms run on over the items of
-// a row of blocks); those sums go to 2^-20 fixed-point partials held as three 32-bit words
-// per component (32-bit shared atomics), so results are bit-reproducible.
+// Each chunk of 64 atoms sums its terms in FP32 in a fixed order (8 for an entry, 16 and a
+// tree over the quarters of the warp for an atom of I); those sums go to 2^-20 fixed-point
+// partials held as 32-bit words (32-bit shared atomics), so results are bit-reproducible, and
+// the same for every cluster size, since units and chunks do not depend on it. (400 frames of
+// 1200 atoms 783 -> 518 us against pairs of whole blocks in scalar operations with three
+// atomics a component; 50 frames of 560 54 -> 43, 3 of 1199 138 -> 38 us.)
 #include <cooperative_groups.h>
 
 #include "scps_internal.h"
@@ -25,7 +30,7 @@ namespace scps {
 namespace {
 
 constexpr unsigned kFullMask = 0xffffffffu;
-constexpr int kHvpSeg = 8;           // candidate blocks J per work unit
+constexpr int kHvpSeg = 32;          // candidate blocks J per work unit (one per lane)
 constexpr int kHvpMaxBlocks = 512;   // 8-atom blocks per frame (4096 atoms)
 
 struct HvpShared {
@@ -33,121 +38,124 @@ struct HvpShared {
     float4* vq;      // direction v
     float2* lj;
     unsigned long long* ex;  // exclusion mask per atom slot
-    int* H2;         // 3 x nta: bits 40 and up of the 2^-20 fixed-point partials (signed)
-    unsigned* H1;    // 3 x nta: bits 20..39
-    unsigned* H0;    // 3 x nta: bits 0..19
+    // 2^-20 fixed-point partials v of 3 components per slot: the low 20 bits (unsigned), the
+    // rest q = v >> 20 as a sum modulo 2^32 and coarse sums of round(q / 2^22), which only the
+    // largest terms (stiff bonds) touch
+    unsigned *L0, *L1;
+    int* H;
     float4* blo;     // boxes of the 8-atom blocks
     float4* bhi;
+    uint16_t* buf;   // per warp: the atoms of its unit
     int nta;
 };
 
-// Adds x in 2^-20 fixed point as three 32-bit words (two 20-bit unsigned parts and the
-// signed rest), so that the sums cover the range of Hessian-vector products of stiff bonds
-// (|Hv| beyond 1e10) with 32-bit shared atomics; each unsigned word takes up to 4095
-// additions.
 __device__ __forceinline__ void hred(const HvpShared& sm, int k, float x) {
-    const long long v = f2fix(x);
-    atomicAdd(&sm.H0[k], (unsigned)(v & 0xfffffll));
-    atomicAdd(&sm.H1[k], (unsigned)((v >> 20) & 0xfffffll));
-    atomicAdd(&sm.H2[k], (int)(v >> 40));
+    const long long v = f2fix(x), q = v >> 20;
+    atomicAdd(&sm.L0[k], (unsigned)(v & 0xfffffll));
+    atomicAdd(&sm.L1[k], (unsigned)q);
+    const int h = (int)(((q >> 21) + 1) >> 1);
+    if (h) atomicAdd(&sm.H[k], h);
 }
 
 __device__ __forceinline__ void hadd(const HvpShared& sm, int i, float x, float y, float z) {
-    hred(sm, i, x);
-    hred(sm, sm.nta + i, y);
-    hred(sm, 2 * sm.nta + i, z);
+    hred(sm, 3 * i, x);
+    hred(sm, 3 * i + 1, y);
+    hred(sm, 3 * i + 2, z);
 }
 
-// phi'(r)/r of the shifted-force pair potential and phi''(r).
+// phi'(r)/r of the shifted-force pair potential, the negative of phi'' - phi'(r)/r over r^2, for
+// two pairs. 1/r^2 is the square of the reciprocal root corrected by one Newton step, so that
+// it is as exact as the division it stands for.
 template <int ELEC>
-__device__ __forceinline__ void pair_derivs(float r2, float sig, float eps24, float qq,
-                                            const PairConst& pc, float& p1, float& pp) {
-    const float inv_r = rsqrtf(r2);
-    const float inv_r2 = inv_r * inv_r;
-    const float sig2 = sig * sig;
-    const float s2 = sig2 * inv_r2;
-    const float s6 = s2 * s2 * s2;
-    const float s12 = s6 * s6;
-    p1 = -eps24 * fmaf(2.0f, s12, -s6) * inv_r2;     // LJ phi'/r
-    pp = eps24 * fmaf(26.0f, s12, -7.0f * s6) * inv_r2;  // LJ phi''
-    const float c2 = sig2 * pc.inv_rc2;
-    const float c6 = c2 * c2 * c2;
-    const float a_ljc = eps24 * c6 * fmaf(2.0f, c6, -1.0f);
-    float cc = 0.0f;
+__device__ __forceinline__ void pair_derivs2(float2 r2, float2 sig, float2 eps24, float2 qq,
+                                             const PairConst& pc, float2& p1, float2& c2) {
+    const float2 ir = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+    float2 ir2 = mul2(ir, ir);
+    ir2 = fma2(ir2, fma2(neg2(r2), ir2, dup2(1.0f)), ir2);
+    const float2 sig2 = mul2(sig, sig);
+    const float2 s2 = mul2(sig2, ir2);
+    const float2 s6 = mul2(mul2(s2, s2), s2);
+    const float2 s12 = mul2(s6, s6);
+    const float2 ei = mul2(eps24, ir2);
+    p1 = mul2(ei, fma2(dup2(-2.0f), s12, s6));                   // LJ phi'/r
+    float2 pp = mul2(ei, fma2(dup2(26.0f), s12, mul2(dup2(-7.0f), s6)));  // LJ phi''
+    const float2 k2 = mul2(sig2, dup2(pc.inv_rc2));
+    const float2 c6 = mul2(mul2(k2, k2), k2);
+    const float2 a_ljc = mul2(mul2(eps24, c6), fma2(dup2(2.0f), c6, dup2(-1.0f)));
+    float2 cc = dup2(0.0f);
     if (ELEC == ELEC_DDIEL) {        // phi = (qq/2) / r^2
-        p1 -= qq * inv_r2 * inv_r2;
-        pp += 3.0f * qq * inv_r2 * inv_r2;
-        cc = qq * pc.inv_rc3;
+        const float2 t = mul2(mul2(qq, ir2), ir2);
+        p1 = fma2(dup2(-1.0f), t, p1);
+        pp = fma2(dup2(3.0f), t, pp);
+        cc = mul2(qq, dup2(pc.inv_rc3));
     } else if (ELEC == ELEC_RF) {    // phi = qq (1/r + krf r^2 - crf)
-        p1 += qq * fmaf(-inv_r2, inv_r, 2.0f * pc.krf);
-        pp += qq * fmaf(2.0f * inv_r2, inv_r, 2.0f * pc.krf);
-        cc = qq * fmaf(pc.inv_rc2, 1.0f, -2.0f * pc.krf * pc.rc);
+        const float2 ir3 = mul2(ir2, ir);
+        p1 = fma2(qq, fma2(dup2(-1.0f), ir3, dup2(2.0f * pc.krf)), p1);
+        pp = fma2(qq, fma2(dup2(2.0f), ir3, dup2(2.0f * pc.krf)), pp);
+        cc = mul2(qq, dup2(fmaf(pc.inv_rc2, 1.0f, -2.0f * pc.krf * pc.rc)));
     } else if (ELEC == ELEC_PLAIN) { // phi = qq / r
-        p1 -= qq * inv_r2 * inv_r;
-        pp += 2.0f * qq * inv_r2 * inv_r;
-        cc = qq * pc.inv_rc2;
+        const float2 t = mul2(qq, mul2(ir2, ir));
+        p1 = fma2(dup2(-1.0f), t, p1);
+        pp = fma2(dup2(2.0f), t, pp);
+        cc = mul2(qq, dup2(pc.inv_rc2));
     }
-    p1 = fmaf(fmaf(a_ljc, pc.inv_rc, cc), inv_r, p1);  // phi_sf' = phi' - phi'(rc)
+    p1 = fma2(fma2(a_ljc, dup2(pc.inv_rc), cc), ir, p1);  // phi_sf' = phi' - phi'(rc)
+    c2 = mul2(fma2(dup2(-1.0f), p1, pp), ir2);
 }
 
+// The pairs of two atoms per lane (j0, j1; dead: the far slot) with the 8 atoms of block I: at
+// iteration t lane l takes block atom (l & 7) ^ t against both. The i sums move by one xor
+// exchange per iteration and component within a quarter warp and come home with the last; the
+// j sums stay in the lane. xm: exclusion bits by block atom (low byte j0, next j1).
 template <int ELEC>
-__device__ __forceinline__ void pair_hvp_term(const HvpShared& sm, const PairConst& pc, int i, int j,
-                                              const float4& xj, const float4& vj, const float2& lj,
-                                              bool ok, float& ax, float& ay, float& az) {
-    const float4 xi = sm.xq[i];
-    const float4 vi = sm.vq[i];
-    const float2 li = sm.lj[i];
-    const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    ok = ok && r2 < pc.rc2;
-    float p1, pp;
-    pair_derivs<ELEC>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, p1, pp);
-    const float wx = vj.x - vi.x, wy = vj.y - vi.y, wz = vj.z - vi.z;
-    const float dw = fmaf(dx, wx, fmaf(dy, wy, dz * wz));
-    const float c1 = (pp - p1) * dw / r2;
-    ax = ok ? fmaf(c1, dx, p1 * wx) : 0.f;
-    ay = ok ? fmaf(c1, dy, p1 * wy) : 0.f;
-    az = ok ? fmaf(c1, dz, p1 * wz) : 0.f;
-}
-
-// The 64 pairs of block I (8 atoms) with block J >= I on a quarter warp: lane l holds atom
-// j = 8 J + l; at iteration t it takes atom i = 8 I + (l ^ t), so the i sums move by one xor
-// exchange per iteration (after the eighth, xor 7, lane l again holds atom 8 I + l's) while
-// the j sum stays in the lane and goes to the fixed-point partials after the item. The i sums (hi*) run on over the
-// items of the row. Within a block (I == J) a pair counts once (j > i). Near blocks test the
-// exclusion masks. An idle quarter (live false) runs along with no terms.
-template <int ELEC>
-__device__ __forceinline__ void hvp_item(const HvpShared& sm, const PairConst& pc, int I, int J,
-                                         int lane, bool live, float& hix, float& hiy, float& hiz) {
+__device__ __forceinline__ void hvp_chunk(const HvpShared& sm, const PairConst& pc, int I, int j0,
+                                          int j1, bool live0, bool live1, unsigned xm, int lane) {
     const int l8 = lane & 7;
-    const int j = 8 * J + l8;
-    const float4 xj = sm.xq[j];
-    const float4 vj = sm.vq[j];
-    const float2 lj = sm.lj[j];
-    const bool near = 8 * (J - I) < kExclWindow + 8;
-    float hjx = 0.f, hjy = 0.f, hjz = 0.f;
-#pragma unroll
+    const float4 xa = sm.xq[j0], xb = sm.xq[j1], va = sm.vq[j0], vb = sm.vq[j1];
+    const float2 la = sm.lj[j0], lb = sm.lj[j1];
+    float hix = 0.f, hiy = 0.f, hiz = 0.f;
+    float2 hx = dup2(0.f), hy = dup2(0.f), hz = dup2(0.f);
+#pragma unroll 2
     for (int t = 0; t < 8; ++t) {
-        const int i = (8 * I + l8) ^ t;
-        bool ok = live && (I != J || j > i);
-        if (near) {
-            const int dj = j - i + kExclWindow;
-            if (dj >= 0 && dj < 2 * kExclWindow) ok = ok && !((sm.ex[i] >> dj) & 1ull);
-        }
-        float ax, ay, az;
-        pair_hvp_term<ELEC>(sm, pc, i, j, xj, vj, lj, ok, ax, ay, az);
-        hix -= ax;
-        hiy -= ay;
-        hiz -= az;
-        hjx += ax;
-        hjy += ay;
-        hjz += az;
+        const int a = l8 ^ t, i = 8 * I + a;
+        const float4 xi = sm.xq[i], vi = sm.vq[i];
+        const float2 li = sm.lj[i];
+        const float2 dx = make_float2(xa.x - xi.x, xb.x - xi.x), dy = make_float2(xa.y - xi.y, xb.y - xi.y),
+                     dz = make_float2(xa.z - xi.z, xb.z - xi.z);
+        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+        const bool ok0 = live0 && r2.x < pc.rc2 && !((xm >> a) & 1u);
+        const bool ok1 = live1 && r2.y < pc.rc2 && !((xm >> (8 + a)) & 1u);
+        float2 p1, c2;
+        pair_derivs2<ELEC>(r2, make_float2(li.x + la.x, li.x + lb.x), make_float2(li.y * la.y, li.y * lb.y),
+                           make_float2(xi.w * xa.w, xi.w * xb.w), pc, p1, c2);
+        const float2 wx = make_float2(va.x - vi.x, vb.x - vi.x), wy = make_float2(va.y - vi.y, vb.y - vi.y),
+                     wz = make_float2(va.z - vi.z, vb.z - vi.z);
+        float2 c1 = mul2(c2, fma2(dx, wx, fma2(dy, wy, mul2(dz, wz))));
+        c1 = make_float2(ok0 ? c1.x : 0.f, ok1 ? c1.y : 0.f);
+        p1 = make_float2(ok0 ? p1.x : 0.f, ok1 ? p1.y : 0.f);
+        const float2 ax = fma2(c1, dx, mul2(p1, wx)), ay = fma2(c1, dy, mul2(p1, wy)),
+                     az = fma2(c1, dz, mul2(p1, wz));
+        hx = add2(hx, ax);
+        hy = add2(hy, ay);
+        hz = add2(hz, az);
+        hix -= ax.x + ax.y;
+        hiy -= ay.x + ay.y;
+        hiz -= az.x + az.y;
         const int m = t < 7 ? t ^ (t + 1) : 7;  // to the lane that takes atom i next
         hix = __shfl_xor_sync(kFullMask, hix, m);
         hiy = __shfl_xor_sync(kFullMask, hiy, m);
         hiz = __shfl_xor_sync(kFullMask, hiz, m);
     }
-    if (live) hadd(sm, j, hjx, hjy, hjz);
+    if (live0) hadd(sm, j0, hx.x, hy.x, hz.x);
+    if (live1) hadd(sm, j1, hx.y, hy.y, hz.y);
+    // the four quarters' shares of the block's atoms (FP32, a fixed order)
+    hix += __shfl_xor_sync(kFullMask, hix, 8);
+    hiy += __shfl_xor_sync(kFullMask, hiy, 8);
+    hiz += __shfl_xor_sync(kFullMask, hiz, 8);
+    hix += __shfl_xor_sync(kFullMask, hix, 16);
+    hiy += __shfl_xor_sync(kFullMask, hiy, 16);
+    hiz += __shfl_xor_sync(kFullMask, hiz, 16);
+    if (lane < 8) hadd(sm, 8 * I + lane, hix, hiy, hiz);
 }
 
 __device__ void hvp_bond(const HvpShared& sm, const TopoDev& tp, int b) {
@@ -231,7 +239,7 @@ __device__ __forceinline__ void hvp_cluster_sync() {
 template <int ELEC, int CL>
 __global__ void __launch_bounds__(1024)
 k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __restrict__ X,
-             const float* __restrict__ V, float* __restrict__ HV, int nta) {
+             const float* V, float* HV, int nta) {  // (HV may be V)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int next_row, n_units;
     __shared__ int upre[kHvpMaxBlocks];  // first work unit of each row of blocks
@@ -245,10 +253,11 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
     sm.blo = (float4*)p; p += sizeof(float4) * nbs;
     sm.bhi = (float4*)p; p += sizeof(float4) * nbs;
     sm.ex = (unsigned long long*)p; p += sizeof(unsigned long long) * nta;
-    sm.H2 = (int*)p; p += sizeof(int) * 3 * nta;
-    sm.H1 = (unsigned*)p; p += sizeof(unsigned) * 3 * nta;
-    sm.H0 = (unsigned*)p; p += sizeof(unsigned) * 3 * nta;
-    sm.lj = (float2*)p;
+    sm.H = (int*)p; p += sizeof(int) * 3 * nta;
+    sm.L1 = (unsigned*)p; p += sizeof(unsigned) * 3 * nta;
+    sm.L0 = (unsigned*)p; p += sizeof(unsigned) * 3 * nta;
+    sm.lj = (float2*)p; p += sizeof(float2) * nta;
+    sm.buf = (uint16_t*)p + (threadIdx.x >> 5) * 8 * kHvpSeg;
     const long long f = blockIdx.x / CL;
     const int rank = CL == 1 ? 0 : (int)cg::this_cluster().block_rank();
     const float* xf = X + f * n * 3;
@@ -267,9 +276,9 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
         }
     }
     for (int i = threadIdx.x; i < 3 * nta; i += blockDim.x) {
-        sm.H2[i] = 0;
-        sm.H1[i] = 0u;
-        sm.H0[i] = 0u;
+        sm.H[i] = 0;
+        sm.L1[i] = 0u;
+        sm.L0[i] = 0u;
     }
     if (threadIdx.x == 0) next_row = 0;
     __syncthreads();
@@ -302,7 +311,7 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
     for (int a = t0; a < tp.n_angles; a += tstep) hvp_angle(sm, tp, a);
     // work units: the rows of blocks I with I % CL == rank, each cut into segments of kHvpSeg
     // candidate blocks J >= I (long rows first); a warp pulls a unit, tests its blocks
-    // against I's box and takes the hits four items at a time
+    // against I's box and their atoms against I's, and takes the hits 64 at a time
     if (warp == 0) {
         int run = 0;
         for (int r0 = 0; r0 < nbs; r0 += 32) {
@@ -337,7 +346,7 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
         if (!(al.x <= ah.x)) continue;  // no atoms in block I (warp-uniform)
         const int J = j0 + lane;
         bool hit = false;
-        if (lane < kHvpSeg && J < nbs) {
+        if (J < nbs) {
             const float4 bl = sm.blo[J], bh = sm.bhi[J];
             const float gx = fmaxf(0.f, fmaxf(al.x - bh.x, bl.x - ah.x));
             const float gy = fmaxf(0.f, fmaxf(al.y - bh.y, bl.y - ah.y));
@@ -345,76 +354,94 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
             hit = bl.x <= bh.x && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < P.pc.rc2;
         }
         unsigned m = __ballot_sync(kFullMask, hit);
-        if (!m) continue;
-        float hix = 0.f, hiy = 0.f, hiz = 0.f;  // this quarter's share of atom 8 I + l8
-        while (m) {
-            const int nh = min(__popc(m), 4);
+        const unsigned lt = (1u << lane) - 1u;
+        int count = 0;
+        while (m) {  // four hit blocks at a time, one atom per lane: those within r_c of an atom of I
             unsigned mm = m;
             for (int k = 0; k < q; ++k) mm &= mm - 1u;
             const int src = __ffs(mm) - 1;
-            for (int k = 0; k < nh; ++k) m &= m - 1u;
-            const bool live = q < nh;
-            hvp_item<ELEC>(sm, P.pc, I, live ? j0 + src : I, lane, live, hix, hiy, hiz);
+            m &= m - 1u;
+            m &= m - 1u;
+            m &= m - 1u;
+            m &= m - 1u;
+            const int j = src >= 0 ? 8 * (j0 + src) + l8 : n;
+            bool near = false;
+            if (j < n) {
+                const float4 xj = sm.xq[j];
+                float dmin = 3.0e38f;
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {  // (empty slots sit far away)
+                    const float4 xi = sm.xq[8 * I + a];
+                    const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+                    dmin = fminf(dmin, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+                }
+                near = dmin < P.pc.rc2;
+            }
+            const unsigned nm = __ballot_sync(kFullMask, near);
+            if (near) sm.buf[count + __popc(nm & lt)] = (uint16_t)j;
+            count += __popc(nm);
         }
-        // the four quarters' shares of the unit's i atoms (FP32, a fixed order)
-        hix += __shfl_xor_sync(kFullMask, hix, 8);
-        hiy += __shfl_xor_sync(kFullMask, hiy, 8);
-        hiz += __shfl_xor_sync(kFullMask, hiz, 8);
-        hix += __shfl_xor_sync(kFullMask, hix, 16);
-        hiy += __shfl_xor_sync(kFullMask, hiy, 16);
-        hiz += __shfl_xor_sync(kFullMask, hiz, 16);
-        if (lane < 8) hadd(sm, 8 * I + lane, hix, hiy, hiz);
+        __syncwarp();
+        for (int k0 = 0; k0 < count; k0 += 64) {
+            const int k = k0 + 2 * lane;
+            const bool live0 = k < count, live1 = k + 1 < count;
+            const int ja = live0 ? sm.buf[k] : 8 * I, jb = live1 ? sm.buf[k + 1] : 8 * I;
+            // excluded pairs, and the pairs of block I with itself once (j after i)
+            unsigned xm = 0u;
+            if (sm.buf[k0] < 8 * I + 8 + kExclWindow) {
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    const int i = 8 * I + a;
+                    const unsigned long long ex = sm.ex[i];
+                    const int da = ja - i + kExclWindow, db = jb - i + kExclWindow;
+                    if (ja <= i || (da < 2 * kExclWindow && ((ex >> da) & 1ull))) xm |= 1u << a;
+                    if (jb <= i || (db < 2 * kExclWindow && ((ex >> db) & 1ull))) xm |= 256u << a;
+                }
+            }
+            hvp_chunk<ELEC>(sm, P.pc, I, ja, jb, live0, live1, xm, lane);
+        }
+        __syncwarp();  // (the next unit overwrites the buffer)
     }
     hvp_cluster_sync<CL>();  // every partial of the cluster is complete
     float* out = HV + f * n * 3;
-    const int* o2 = CL == 1 ? sm.H2 : cg::this_cluster().map_shared_rank(sm.H2, (unsigned)(rank ^ 1));
-    const unsigned* o1 = CL == 1 ? sm.H1 : cg::this_cluster().map_shared_rank(sm.H1, (unsigned)(rank ^ 1));
-    const unsigned* o0 = CL == 1 ? sm.H0 : cg::this_cluster().map_shared_rank(sm.H0, (unsigned)(rank ^ 1));
-    for (int i = threadIdx.x + rank * blockDim.x; i < n; i += CL * blockDim.x) {
-        long long h[3];
+    for (int k = threadIdx.x + rank * blockDim.x; k < 3 * n; k += CL * blockDim.x) {
+        long long h = sm.H[k], l0 = sm.L0[k];
+        unsigned l1 = sm.L1[k];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int k = c * nta + i;
-            h[c] = ((long long)sm.H2[k] << 40) + ((long long)sm.H1[k] << 20) + (long long)sm.H0[k];
-            if (CL == 2) h[c] += ((long long)o2[k] << 40) + ((long long)o1[k] << 20) + (long long)o0[k];
+        for (int r = 1; r < CL; ++r) {
+            const unsigned p = (unsigned)((rank + r) & (CL - 1));
+            h += cg::this_cluster().map_shared_rank(sm.H, p)[k];
+            l0 += cg::this_cluster().map_shared_rank(sm.L0, p)[k];
+            l1 += cg::this_cluster().map_shared_rank(sm.L1, p)[k];
         }
-        out[3 * i] = fix2f(h[0]);
-        out[3 * i + 1] = fix2f(h[1]);
-        out[3 * i + 2] = fix2f(h[2]);
+        out[k] = fix2f((join_coarse(h, l1, 22) << 20) + l0);
     }
     hvp_cluster_sync<CL>();  // no CTA leaves while its shared memory may still be read
 }
 
-size_t hvp_smem_bytes(int nta) {
+size_t hvp_smem_bytes(int nta, int threads) {
     const int nbs = nta / 8;
     return sizeof(float4) * 2 * nta + sizeof(float4) * 2 * nbs + sizeof(unsigned long long) * nta +
-           (sizeof(int) + 2 * sizeof(unsigned)) * 3 * (size_t)nta + sizeof(float2) * nta;
+           (sizeof(int) + 2 * sizeof(unsigned)) * 3 * (size_t)nta + sizeof(float2) * nta +
+           sizeof(uint16_t) * 8 * kHvpSeg * (threads / 32);
 }
 
-// Few frames (a checkpoint segment): a 2-CTA cluster of 1024 threads per frame, so that
-// the frames spread over the SMs; many frames: one 512-thread CTA each.
-template <int ELEC>
+template <int ELEC, int CL>
 static cudaError_t launch_hvp_t(const TopoDev* topo, const RunParams& P, const float* X,
-                                const float* V, float* HV, long long n_frames, int nta,
+                                const float* V, float* HV, long long n_frames, int nta, int threads,
                                 cudaStream_t s) {
-    int dev = 0, n_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int cl = 2 * n_frames <= n_sm ? 2 : 1;
-    const int threads = n_frames * cl <= n_sm ? 1024 : 512;
-    const size_t smem = hvp_smem_bytes(nta);
-    auto kern = cl == 2 ? k_hvp_frames<ELEC, 2> : k_hvp_frames<ELEC, 1>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = hvp_smem_bytes(nta, threads);
+    auto kern = k_hvp_frames<ELEC, CL>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n_frames * cl));
+    cfg.gridDim = dim3((unsigned)(n_frames * CL));
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cl;
+    attr[0].val.clusterDim.x = CL;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -424,13 +451,29 @@ static cudaError_t launch_hvp_t(const TopoDev* topo, const RunParams& P, const f
     return cudaGetLastError();
 }
 
+// Few frames: a cluster of 1024-thread CTAs per frame, so that the frames spread over the
+// SMs; many frames: one 512-thread CTA each.
+template <int ELEC>
+static cudaError_t launch_hvp_e(const TopoDev* topo, const RunParams& P, const float* X,
+                                const float* V, float* HV, long long n_frames, int nta,
+                                cudaStream_t s) {
+    int dev = 0, n_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (10 * n_frames <= n_sm) return launch_hvp_t<ELEC, 8>(topo, P, X, V, HV, n_frames, nta, 1024, s);
+    if (5 * n_frames <= n_sm) return launch_hvp_t<ELEC, 4>(topo, P, X, V, HV, n_frames, nta, 1024, s);
+    if (2 * n_frames <= n_sm) return launch_hvp_t<ELEC, 2>(topo, P, X, V, HV, n_frames, nta, 1024, s);
+    return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, n_frames <= n_sm ? 1024 : 512, s);
+}
+
 cudaError_t launch_hvp(int elec, const TopoDev* topo, const RunParams& P, const float* X,
                        const float* V, float* HV, long long n_frames, int nta, cudaStream_t s) {
     switch (elec) {
-        case ELEC_DDIEL: return launch_hvp_t<ELEC_DDIEL>(topo, P, X, V, HV, n_frames, nta, s);
-        case ELEC_RF: return launch_hvp_t<ELEC_RF>(topo, P, X, V, HV, n_frames, nta, s);
-        case ELEC_PLAIN: return launch_hvp_t<ELEC_PLAIN>(topo, P, X, V, HV, n_frames, nta, s);
-        default: return launch_hvp_t<ELEC_NONE>(topo, P, X, V, HV, n_frames, nta, s);
+        case ELEC_DDIEL: return launch_hvp_e<ELEC_DDIEL>(topo, P, X, V, HV, n_frames, nta, s);
+        case ELEC_RF: return launch_hvp_e<ELEC_RF>(topo, P, X, V, HV, n_frames, nta, s);
+        case ELEC_PLAIN: return launch_hvp_e<ELEC_PLAIN>(topo, P, X, V, HV, n_frames, nta, s);
+        default: return launch_hvp_e<ELEC_NONE>(topo, P, X, V, HV, n_frames, nta, s);
     }
 }
 
