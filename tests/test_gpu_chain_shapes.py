@@ -102,3 +102,26 @@ def test_large_forces_match_the_oracle(torch_cuda, scale):
     assert np.abs(F[0] - Fr).max() <= 1e-5 * rms
     assert np.abs(Fr).max() > 2000.0  # beyond the first coarse word
     s.close()
+
+
+@pytest.mark.parametrize("n", [9, 64, 257, 559])
+def test_hvp_of_every_cluster_size_agrees(torch_cuda, n):
+    # 1e-5 of the rms, as for the other Hessian-vector products
+    torch = torch_cuda
+    c = cut(synth.make_chain(35, seed=1), n)
+    s = system(c)
+    g = np.random.default_rng(6)
+    X = torch.from_numpy((c.x_unfolded[None] + g.normal(0, 0.01, (180, n, 3))).astype(np.float32)).cuda()
+    V = torch.from_numpy(g.normal(0, 1, (180, n, 3)).astype(np.float32)).cuda()
+    whole = torch.empty_like(X)
+    s.hvp(0, X, V, whole)
+    for m in (60, 20, 3):
+        part = torch.empty_like(X[:m])
+        s.hvp(0, X[:m].contiguous(), V[:m].contiguous(), part)
+        assert torch.equal(whole[:m], part)
+    W = V.clone()
+    s.hvp(0, X, W, W)  # in place
+    assert torch.equal(whole, W)
+    _, ref = oracle.ForceField.from_chain(c).hvp(X[0].double().cpu().numpy(), V[0].double().cpu().numpy())
+    assert np.abs(whole[0].cpu().numpy() - ref).max() <= 1e-5 * np.sqrt((ref ** 2).sum(1).mean())
+    s.close()
