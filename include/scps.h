@@ -126,7 +126,7 @@ typedef struct {
     int32_t max_frames;     /* frames kept per replica (the oldest are overwritten) */
     /* execution */
     int32_t exec;           /* SCPS_EXEC_* */
-    int32_t cluster_size;   /* CTAs per replica in RESIDENT form: 0 = auto (1, 2 or 4), 1 or 2 */
+    int32_t cluster_size;   /* CTAs per replica in RESIDENT form: 0 = auto (1, 2, 4 or 8), 1 or 2 */
     int32_t threads;        /* threads per CTA in RESIDENT form: 0 = auto, else 128..1024
                                (at most 768 in a cluster of CTAs) */
     int32_t steps_per_graph;/* device-loop steps per CUDA-graph node: 0 = auto */
@@ -307,8 +307,8 @@ int scps_path_average(scps_system* s, int32_t n_sel, const int32_t* replicas, in
                       double* out);
 
 /* Autotuner of the resident form (chain replicas): times the launch plans
- * (SCPS_PLAN_*), cluster sizes {1, 2} and threads per CTA {256, 512, 1024} (768 in
- * place of 1024 for 2-CTA clusters) on the system itself, then, at the chosen shape, the
+ * (SCPS_PLAN_*), cluster sizes {1, 2} and threads per CTA {256, 512, 768} beside the current
+ * shape on the system itself, then, at the chosen shape, the
  * pair-list skin {0.06, 0.09, 0.12, 0.16, 0.2} nm (a larger skin adds pairs to every
  * step and makes list builds rarer: the rebuild cadence follows from the displacement
  * bound), probe_steps steps each from the current state (restored after every probe; no

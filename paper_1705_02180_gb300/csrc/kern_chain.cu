@@ -5,10 +5,17 @@
 
 namespace scps {
 
-SCPS_CHAIN_LAUNCHERS(extern, 1)
-SCPS_CHAIN_LAUNCHERS(extern, 2)
-SCPS_CHAIN_LAUNCHERS(extern, 4)
-SCPS_CHAIN_LAUNCHERS(extern, 8)
+SCPS_RESIDENT_LAUNCHERS(extern, 1, false)
+SCPS_RESIDENT_LAUNCHERS(extern, 1, true)
+SCPS_RESIDENT_LAUNCHERS(extern, 2, true)
+SCPS_RESIDENT_LAUNCHERS(extern, 4, true)
+SCPS_RESIDENT_LAUNCHERS(extern, 8, true)
+SCPS_EVAL_LAUNCHERS(extern, 1)
+SCPS_EVAL_LAUNCHERS(extern, 2)
+SCPS_EVAL_LAUNCHERS(extern, 4)
+SCPS_EVAL_LAUNCHERS(extern, 8)
+SCPS_MAX_CLUSTERS(extern, 4)
+SCPS_MAX_CLUSTERS(extern, 8)
 
 // Shared-memory bytes of the resident kernels for nta atom slots (plus the 8 sentinel
 // slots): positions with charges and LJ parameters, velocities, the xi array and the two
@@ -58,25 +65,24 @@ size_t launch_smem(int nta, int threads, int cl, int* lc_cap) {
     return base + cap * sizeof(CacheItem);
 }
 
-// Clusters of `cl` CTAs of the resident kernel that run at once.
+// Clusters of `cl` CTAs (4 or 8) of the resident kernel that run at once.
 int chain_max_clusters(int cl, int nta, int threads) {
-    switch (cl) {
-        case 8: return max_clusters_cl<8>(nta, threads);
-        case 4: return max_clusters_cl<4>(nta, threads);
-        case 2: return max_clusters_cl<2>(nta, threads);
-        default: return max_clusters_cl<1>(nta, threads);
-    }
+    return cl == 8 ? max_clusters_cl<8>(nta, threads) : max_clusters_cl<4>(nta, threads);
 }
 
 cudaError_t launch_resident(int elec, int cluster, const TopoDev* topos, const RepDev* reps,
                             const StateDev& st, const RunParams& P, int nta, int threads,
                             cudaStream_t stream) {
     switch (cluster) {
-        case 8: return launch_resident_cl<8>(elec, topos, reps, st, P, nta, threads, stream);
-        case 4: return launch_resident_cl<4>(elec, topos, reps, st, P, nta, threads, stream);
-        case 2: return launch_resident_cl<2>(elec, topos, reps, st, P, nta, threads, stream);
-        default: return launch_resident_cl<1>(elec, topos, reps, st, P, nta, threads, stream);
+        case 8: return launch_resident_cl<8, true>(elec, topos, reps, st, P, nta, threads, stream);
+        case 4: return launch_resident_cl<4, true>(elec, topos, reps, st, P, nta, threads, stream);
+        case 2: return launch_resident_cl<2, true>(elec, topos, reps, st, P, nta, threads, stream);
+        default: break;
     }
+    // (two CTAs per SM want the registers of the narrow form)
+    if (threads > 512 && threads <= kMaxThreadsPair)
+        return launch_resident_cl<1, true>(elec, topos, reps, st, P, nta, threads, stream);
+    return launch_resident_cl<1, false>(elec, topos, reps, st, P, nta, threads, stream);
 }
 
 cudaError_t launch_eval(int elec, const TopoDev* topo, const RunParams& P, const float* X,

@@ -10,9 +10,8 @@
 //   z(X) of Eq. (zrMD) from C_ij of Eq. (Cij) in float-float     collective coordinate
 //   ratchet of Eq. (FrMD) in FP64 (z < z_m: z_m = z, no bias)   bias force
 //   BAOAB update with Philox4x32-10 noise (Eq. Lang)
-// and writes a frame every save_interval steps. Every CTA of a cluster
-// integrates all atoms of the replica with the same total force, so their
-// copies of the state stay identical without being exchanged.
+// and writes a frame every save_interval steps. Each CTA of a cluster integrates a
+// share of the atoms and writes their new positions into every CTA's copy.
 //
 // Pair list. Atoms are grouped in blocks of 8 consecutive chain atoms. For each
 // block I the list holds, in ascending order, every atom j of a later block that
@@ -110,7 +109,7 @@ struct Shared {
 struct ListDev {
     uint16_t* jl;               // j entries of all blocks
     uint32_t* items;            // this CTA's item table
-    uint8_t* excl;              // exclusion masks of this CTA's items
+    uint8_t* excl;              // exclusion masks, kListMasks bytes per block
     int nbs;                    // blocks of the slab layout (nta / 8)
 };
 
@@ -131,7 +130,8 @@ struct Scalars {
     double zm, z, epot, T;
     float kb;           // the bias force on an atom is kb times its bias gradient
     uint16_t cnt[kMaxChainAtoms / 8], cntn[kMaxChainAtoms / 8];  // list chunks per block, near ones
-    long long red_z[2][32];  // per-warp shares of z (units of 2^-40), by parity
+    unsigned zw[2][3];       // this CTA's share of z by parity: sums of its bits 0..19, 20..39 and
+                             // 40 up (units of 2^-40), which 32-bit atomics add
     long long red_e[2][32];  // per-warp shares of the potential energy (units of 2^-20)
     // contact-map tube bias
     double sm, wm;                      // running minima of s_lambda and w_lambda
@@ -244,7 +244,7 @@ __device__ __forceinline__ ListDev list_of(unsigned char* slab, int nta, int ran
     const long long part = list_items_part(L.nbs, CL);  // items of one CTA of the cluster
     unsigned char* items = slab + list_jl_bytes(L.nbs);
     L.items = (uint32_t*)items + rank * part;
-    L.excl = items + list_items_bytes(L.nbs) + (long long)kListChunk * rank * part;
+    L.excl = items + list_items_bytes(L.nbs);
     return L;
 }
 
@@ -379,7 +379,8 @@ __device__ __forceinline__ void pair_batch(const Shared& sm, Scalars& sc, const 
             I = (int)(d >> 17);
             near = (d >> 16) & 1u;
             jj = __ldcg((const unsigned*)(L.jl + list_jl_off(L.nbs, I) + kListChunk * (int)(d & 0xffffu)) + l8);
-            if (near) xm = __ldcg((const uint16_t*)(L.excl + (long long)kListChunk * it) + l8);
+            if (near)
+                xm = __ldcg((const uint16_t*)(L.excl + kListMasks * I + kListChunk * (int)(d & 0xffffu)) + l8);
         }
     }
     const int j0 = (int)(jj & 0xffffu), j1 = (int)(jj >> 16);
@@ -844,7 +845,7 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
     const TopoDev& tp = sc.tp;
     const ListDev L = sc.list;
     const int n = tp.n_atoms, nb = (n + 7) >> 3;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = cta_rank<CL>();
     // scratch in the xi array (128 B per block): boxes (2 nb float4), the two prefix arrays
     // (nb ints each, one more for the total) and per warp the candidate blocks of its row
@@ -889,7 +890,7 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
             nc += __popc(cm);
         }
         __syncwarp();
-        int count = 0, n_near = 0;
+        int count = 0;
         for (int g = 0; g < nc; g += 8) {  // eight candidates at a time, two atoms per lane:
             // lane (c, s) tests atom s of candidates g + c and g + 4 + c, packed
             const int ca = g + (lane >> 3), cb = ca + 4;
@@ -914,9 +915,30 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
             count += __popc(ma);
             if (hb) out[count + __popc(mb & lt)] = (uint16_t)jb;
             count += __popc(mb);
-            n_near += __popc(__ballot_sync(kFull, ha && ja < i0 + 8 + 31)) +
-                      __popc(__ballot_sync(kFull, hb && jb < i0 + 8 + 31));
         }
+        // the entries near the block come first: lane s tests atom s after the block and writes
+        // its exclusion mask (bit a for block atom a; zero past the near entries)
+        const int jn = i0 + 8 + lane;
+        const bool in = lane < kExclWindow - 1 && jn < n;
+        const float4 xn = in ? sm.xq()[jn] : make_float4(1.0e18f, 0.f, 0.f, 0.f);
+        const unsigned long long exa = (lane < 8 && i0 + lane < n) ? tp.excl[i0 + lane] : 0ull;
+        float dn = 3.0e38f;
+        unsigned byte = 0u;
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+            const float4 xi = sm.xq()[i0 + a];
+            const float dx = xn.x - xi.x, dy = xn.y - xi.y, dz = xn.z - xi.z;
+            dn = fminf(dn, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+            const unsigned long long ex = __shfl_sync(kFull, exa, a);
+            const int dj = 8 + lane - a + kExclWindow;
+            if (dj < 2 * kExclWindow && ((ex >> dj) & 1ull)) byte |= 1u << a;
+        }
+        const bool hn = dn < rlist2;
+        const unsigned mn = __ballot_sync(kFull, hn);
+        const int n_near = __popc(mn);
+        uint8_t* mask = L.excl + kListMasks * I;
+        if (hn) mask[__popc(mn & lt)] = (uint8_t)byte;
+        if (lane >= n_near) mask[lane] = 0;
         __syncwarp();  // (the candidate list is overwritten by the warp's next row)
         const int chunks = (count + kListChunk - 1) / kListChunk;
         if (lane < kListChunk * chunks - count) out[count + lane] = (uint16_t)sm.nta;
@@ -929,30 +951,30 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
     __threadfence();  // entries are read back with L2 loads (also by the other CTAs)
     cluster_barrier<CL>();  // every block's entries and counts are complete
     if (warp == 0) {  // prefix sums over blocks: near chunks, then the remaining ones
+        const int per = (nb + 31) >> 5, I0 = min(per * lane, nb), I1 = min(I0 + per, nb);
         int runn = 0, runf = 0;
-        for (int I0 = 0; I0 < nb; I0 += 32) {
-            const int I = I0 + lane;
-            int cn = 0, cf = 0;
-            if (I < nb) {
-                cn = sc.cntn[I];
-                cf = sc.cnt[I] - cn;
-            }
-            int sn = cn, sf = cf;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int yn = __shfl_up_sync(kFull, sn, o), yf = __shfl_up_sync(kFull, sf, o);
-                if (lane >= o) {
-                    sn += yn;
-                    sf += yf;
-                }
-            }
-            if (I < nb) {
-                pren[I] = runn + sn - cn;
-                pref[I] = runf + sf - cf;
-            }
-            runn += __shfl_sync(kFull, sn, 31);
-            runf += __shfl_sync(kFull, sf, 31);
+        for (int I = I0; I < I1; ++I) {
+            runn += sc.cntn[I];
+            runf += sc.cnt[I] - sc.cntn[I];
         }
+        int sn = runn, sf = runf;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int yn = __shfl_up_sync(kFull, sn, o), yf = __shfl_up_sync(kFull, sf, o);
+            if (lane >= o) {
+                sn += yn;
+                sf += yf;
+            }
+        }
+        int pn = sn - runn, pf = sf - runf;
+        for (int I = I0; I < I1; ++I) {
+            pren[I] = pn;
+            pref[I] = pf;
+            pn += sc.cntn[I];
+            pf += sc.cnt[I] - sc.cntn[I];
+        }
+        runn = __shfl_sync(kFull, sn, 31);
+        runf = __shfl_sync(kFull, sf, 31);
         const int total = runn + runf;
         if (lane == 0) {
             sc.n_items = (total - rank + CL - 1) / CL;
@@ -968,45 +990,29 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
     __syncthreads();
     const int tot_near = pref[nb];
     const bool cached = sc.cached;
-    for (int I = warp; I < nb; I += nw) {
-        const int ct = sc.cnt[I], cn = sc.cntn[I];
-        for (int c = lane; c < ct; c += 32) {
-            const int k = c < cn ? pren[I] + c : tot_near + pref[I] + (c - cn);
-            if (k % CL == rank) {
-                const uint32_t d = ((uint32_t)I << 17) | ((uint32_t)(c < cn) << 16) | (uint32_t)c;
-                if (cached) {  // the chunk's entries: two 16-byte loads (chunks are 32-aligned)
-                    CacheItem& ci = sm.lc()[k / CL];
-                    const uint4* e = (const uint4*)(L.jl + list_jl_off(L.nbs, I) + kListChunk * c);
-                    ci.desc = d;
-                    ((uint4*)ci.j)[0] = __ldcg(e);
-                    ((uint4*)ci.j)[1] = __ldcg(e + 1);
-                } else {
-                    L.items[k / CL] = d;
-                }
-            }
+    // one item per thread: its block is the last whose first chunk number is not beyond it
+    for (int it = tid; it < sc.n_items; it += blockDim.x) {
+        const int k = it * CL + rank;
+        const bool near = k < tot_near;
+        const int* pre = near ? pren : pref;
+        const int key = near ? k : k - tot_near;
+        int lo = 0, hi = nb;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (pre[mid] <= key) lo = mid; else hi = mid;
         }
-        // excluded pairs of the near items: one byte per entry, bit a for block atom a; two
-        // chunks per pass, 16 lanes each, the block atoms' exclusion words held by lanes 0..7
-        // (other items take no masks)
-        const unsigned long long exa = (lane < 8 && 8 * I + lane < n) ? tp.excl[8 * I + lane] : 0ull;
-        const uint16_t* e = L.jl + list_jl_off(L.nbs, I);
-        for (int c0 = 0; c0 < cn; c0 += 2) {
-            const int c = c0 + (lane >> 4), sl = lane & 15;
-            const int jj = c < cn ? (int)__ldcg(e + kListChunk * c + sl) : 0;
-            unsigned byte = 0u;
-#pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                const unsigned long long ex = __shfl_sync(kFull, exa, a);
-                const int dj = jj - (8 * I + a) + kExclWindow;  // entries lie after the block
-                if (c < cn && dj < 2 * kExclWindow && ((ex >> dj) & 1ull)) byte |= 1u << a;
-            }
-            const int k = c < cn ? pren[I] + c : 0;
-            if (c < cn && k % CL == rank) {
-                if (cached)
-                    sm.lc()[k / CL].xm[sl] = (uint8_t)byte;
-                else
-                    L.excl[(long long)kListChunk * (k / CL) + sl] = (uint8_t)byte;
-            }
+        const int c = key - pre[lo] + (near ? 0 : (int)sc.cntn[lo]);
+        const uint32_t d = ((uint32_t)lo << 17) | ((uint32_t)near << 16) | (uint32_t)c;
+        if (cached) {  // the chunk's entries: two 16-byte loads (chunks are 32-aligned)
+            CacheItem& ci = sm.lc()[it];
+            const uint4* e = (const uint4*)(L.jl + list_jl_off(L.nbs, lo) + kListChunk * c);
+            const uint4 e0 = __ldcg(e), e1 = __ldcg(e + 1);
+            if (near) *(uint4*)ci.xm = __ldcg((const uint4*)(L.excl + kListMasks * lo + kListChunk * c));
+            ci.desc = d;
+            ((uint4*)ci.j)[0] = e0;
+            ((uint4*)ci.j)[1] = e1;
+        } else {
+            L.items[it] = d;
         }
     }
     __syncthreads();
@@ -1016,21 +1022,23 @@ __device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
 // Force evaluation
 // ---------------------------------------------------------------------------
 
+// First tile (of 32 atoms) of the share of nt tiles that CTA `rank` of cl integrates.
+__device__ __forceinline__ int own_lo(int nt, int rank, int cl) { return nt * rank / cl; }
+
 // Force evaluation of the configuration in shared memory (pair list current) for
 // the evaluated step of parity b. Work items come from the queue of this CTA; its
 // share goes to the parity-b partials. With noise_step >= 0 the CTA also draws the
-// Gaussian numbers of that step's O half step for all atoms (each CTA of a cluster
-// integrates every atom). Ends with a cluster barrier: the partials of every CTA are
+// Gaussian numbers of that step's O half step for the atoms it integrates. Ends with a cluster barrier: the partials of every CTA are
 // complete (the bias gradient of the tube bias is not: see finish_evaluation).
 template <int ELEC, bool ENERGY, int CL, bool TUBE>
 __device__ void evaluate_work(const Shared& sm, Scalars& sc, const RunParams& P, int b,
                               bool do_ratchet, uint32_t rep_id, long long noise_step) {
     const TopoDev& tp = sc.tp;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int nt = tp.n_tiles;
-    if (noise_step >= 0)
-        for (int q = warp; q < nt; q += nw) noise_chunk(sm, tp, P, rep_id, noise_step, q, lane);
-    const int rank = cta_rank<CL>();
+    const int nt = tp.n_tiles, rank = cta_rank<CL>();
+    if (noise_step >= 0)  // of the atoms this CTA integrates
+        for (int q = own_lo(nt, rank, CL) + warp; q < own_lo(nt, rank + 1, CL); q += nw)
+            noise_chunk(sm, tp, P, rep_id, noise_step, q, lane);
     // Work list of this CTA: pair batches (four items from its item table each), blocks
     // with themselves (four per batch), then its shares of the contact, bond and angle
     // chunks (global chunk g belongs to CTA g % CL). Under the contact-map tube bias the
@@ -1114,13 +1122,19 @@ __device__ void evaluate_work(const Shared& sm, Scalars& sc, const RunParams& P,
             }
         }
     }
-    zacc = warp_sum_ll(zacc);
+    if (ncon > 0 && !tube) {
+        const unsigned z0 = __reduce_add_sync(kFull, (unsigned)zacc & 0xfffffu),
+                       z1 = __reduce_add_sync(kFull, (unsigned)(zacc >> 20) & 0xfffffu),
+                       z2 = __reduce_add_sync(kFull, (unsigned)(zacc >> 40));
+        if (lane == 0) {
+            atomicAdd(&sc.zw[b][0], z0);
+            atomicAdd(&sc.zw[b][1], z1);
+            if (z2) atomicAdd(&sc.zw[b][2], z2);
+        }
+    }
     long long e = 0;
     if (ENERGY) e = warp_sum_ll((e18 << 2) + e20);  // 2^-18 pair energy units to 2^-20
-    if (lane == 0) {
-        sc.red_z[b][warp] = zacc;
-        sc.red_e[b][warp] = e;
-    }
+    if (ENERGY && lane == 0) sc.red_e[b][warp] = e;
     cluster_barrier<CL>();
 }
 
@@ -1140,11 +1154,14 @@ __device__ void finish_evaluation(const Shared& sm, Scalars& sc, const RunParams
     // shares of z, energy and flags from every CTA of the cluster (integer sums); all
     // remote loads are issued before any is used
     if (warp == 0) {
-        long long zq[CL], eq[CL];
+        unsigned zq[CL][3];
+        long long eq[CL];
         int fq[CL];
 #pragma unroll
         for (int q = 0; q < CL; ++q) {
-            zq[q] = lane < nw ? rank_ptr<CL>(&sc.red_z[b][0], q)[lane] : 0;
+            const unsigned* z = rank_ptr<CL>(&sc.zw[b][0], q);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) zq[q][c] = lane == 0 ? z[c] : 0u;
             eq[q] = (ENERGY && lane < nw) ? rank_ptr<CL>(&sc.red_e[b][0], q)[lane] : 0;
             fq[q] = lane == 0 ? *rank_ptr<CL>(&sc.flag[b], q) : 0;
         }
@@ -1152,11 +1169,10 @@ __device__ void finish_evaluation(const Shared& sm, Scalars& sc, const RunParams
         int fl = 0;
 #pragma unroll
         for (int q = 0; q < CL; ++q) {
-            zt += zq[q];
+            zt += ((long long)zq[q][2] << 40) + ((long long)zq[q][1] << 20) + (long long)zq[q][0];
             et += eq[q];
             fl |= fq[q];
         }
-        zt = warp_sum_ll(zt);
         if (ENERGY) et = warp_sum_ll(et);
         if (lane == 0) {
             if (ENERGY) sc.epot = (double)et * 9.5367431640625e-07;  // 2^-20
@@ -1164,14 +1180,20 @@ __device__ void finish_evaluation(const Shared& sm, Scalars& sc, const RunParams
             float kb = 0.f;
             int on = 0;
             if (P.bias == 1 || (P.bias == 5 && !tube)) {  // (frame evaluation: z as well)
-                const double z = (double)zt * 9.094947017729282e-13;  // 2^-40
+                // z = zt 2^-40: the count goes into the mantissa of 4096 (whose last bit is
+                // 2^-40), one FP64 subtraction instead of a conversion and a product (an FP64
+                // instruction costs about 70 clocks that every warp waits for)
+                const double z = zt < (1ll << 52)
+                                     ? __longlong_as_double(0x40B0000000000000ll | zt) - 4096.0
+                                     : (double)zt * 9.094947017729282e-13;
                 sc.z = z;
                 if (do_ratchet && P.bias == 1) {  // Eq. (FrMD) with theta(0) = 1
-                    if (z < sc.zm) {
+                    const double zm = sc.zm, dz = z - zm;
+                    if (below_zero(dz)) {  // z < z_m
                         sc.zm = z;
                     } else {
-                        const double factor = -P.k_R * (z - sc.zm);
-                        on = factor != 0.0;
+                        const double factor = -P.k_R * dz;
+                        on = (__double_as_longlong(factor) << 1) != 0;  // not zero
                         kb = -(float)factor * 4.0f * P.inv_r0sq;
                     }
                 }
@@ -1209,11 +1231,13 @@ __device__ __forceinline__ float4 far_slot(int i) {
 
 }  // namespace
 
-// A CTA of a cluster runs at most kMaxThreadsPair threads per CTA, which leaves 80 registers per
-// thread; a lone CTA per replica keeps 1024 threads, so that two 512-thread CTAs can share
-// an SM.
-template <int ELEC, int CL, bool TUBE>
-__global__ void __launch_bounds__(CL > 1 ? kMaxThreadsPair : 1024, 1)
+// WIDE: at most kMaxThreadsPair threads per CTA, which leaves 80 registers per thread (every
+// cluster of several CTAs, and a lone CTA that has an SM to itself: 1200 atoms 78.5 us per step
+// against 84.0 with 1024 threads of 64 registers, 304 atoms 14.3 against 15.4). Otherwise up to
+// 1024 threads of 64 registers, so that two 512-thread CTAs can share an SM (304 replicas of
+// 560 atoms: 68 us per step, against 73 with 80 registers, which leave one CTA per SM).
+template <int ELEC, int CL, bool TUBE, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kMaxThreadsPair : 1024, 1)
 k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, StateDev st,
            RunParams P, int nta, int lc_cap) {
     __shared__ Scalars sc;
@@ -1259,6 +1283,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         sc.work_next2[1] = 0;
         sc.vmax2[0] = 0u;
         sc.vmax2[1] = 0u;
+        for (int q = 0; q < 6; ++q) (&sc.zw[0][0])[q] = 0u;
         sc.sm = st.sm[r];
         sc.wm = st.wm[r];
     }
@@ -1283,8 +1308,11 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         // beside the ratchet decision that the other warps would wait for (the tube bias
         // completes its gradient after the decision and loads then).
         const bool grad = P.bias != 0;
+        // the atoms this CTA integrates; their new positions go to every CTA
+        const int a0 = kTile * own_lo(tp.n_tiles, rank, CL),
+                  a1 = min(n, kTile * own_lo(tp.n_tiles, rank + 1, CL));
         AtomSums first = {};
-        if (!TUBE && tid < n) first = load_sums<CL>(sm, sc, (int)(step & 1), rank, tid, grad);
+        if (!TUBE && a0 + tid < a1) first = load_sums<CL>(sm, sc, (int)(step & 1), rank, a0 + tid, grad);
         finish_evaluation<false, CL, TUBE>(sm, sc, P, (int)(step & 1), true);
         // position of `step` in the save cycle and ring slot of the next frame, kept as
         // counters so that the loop has no 64-bit divisions
@@ -1298,20 +1326,18 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             const bool save = do_b && save_phase == 0;
             const float kb = sc.kb;  // F_bias = kb G
             float vm2 = 0.f;  // largest |v after B|^2 + |v after O|^2 of this thread's atoms
-            for (int base = 0; base < nta; base += blockDim.x) {
+            // the other parity's partials were last read before this evaluation's cluster
+            // barrier (here and in the other CTAs): clear them for the next one
+            {
+                uint4* f = (uint4*)sm.F(nb).L;
+                uint4* g = (uint4*)sm.G(nb).L;
+                for (int i = tid; i < 3 * sm.na8() / 2; i += blockDim.x)
+                    f[i] = g[i] = make_uint4(0u, 0u, 0u, 0u);
+            }
+            for (int base = a0; base < a1; base += blockDim.x) {
                 const int i = base + tid;
-                if (i < n) {
-                    const AtomSums a = !TUBE && base == 0 ? first : load_sums<CL>(sm, sc, b, rank, i, grad);
-                    // the other parity's partials were last read before this evaluation's
-                    // cluster barrier (here and in the other CTAs): clear them for the next one
-                    const Part Fn = sm.F(nb), Gn = sm.G(nb);
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        Fn.L[3 * i + c] = 0u;
-                        Fn.H[3 * i + c] = 0;
-                        Gn.L[3 * i + c] = 0u;
-                        Gn.H[3 * i + c] = 0;
-                    }
+                if (i < a1) {
+                    const AtomSums a = !TUBE && base == a0 ? first : load_sums<CL>(sm, sc, b, rank, i, grad);
                     float4 v = sm.v()[i];
                     const float im = v.w;
                     float fx = a.fx, fy = a.fy, fz = a.fz;
@@ -1319,8 +1345,8 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         // (rounding spelled out: trajectories amplify the last bit)
                         const float bx = __fmul_rn(kb, a.gx), by = __fmul_rn(kb, a.gy),
                                     bz = __fmul_rn(kb, a.gz);
-                        if (do_b)
-                            sm.xi()[i].w = fmaf(bz, bz, fmaf(bx, bx, __fmul_rn(by, by))) * im;
+                        if (do_b)  // (rank 0 sums the bias functional)
+                            rank_ptr<CL>(sm.xi(), 0)[i].w = fmaf(bz, bz, fmaf(bx, bx, __fmul_rn(by, by))) * im;
                         fx = __fadd_rn(fx, bx);
                         fy = __fadd_rn(fy, by);
                         fz = __fadd_rn(fz, bz);
@@ -1330,7 +1356,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         v.x = fmaf(hdt * im, fx, v.x);
                         v.y = fmaf(hdt * im, fy, v.y);
                         v.z = fmaf(hdt * im, fz, v.z);
-                        if (save && rank == 0) {
+                        if (save) {
                             float* fr = st.frames + 3 * (rep.frame_off + (long long)slot * n + i);
                             fr[0] = x.x;
                             fr[1] = x.y;
@@ -1355,22 +1381,24 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         vm2 = fmaxf(vm2, v1 + fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)));
                         if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
                               isfinite(v.y) && isfinite(v.z)))
-                            atomicOr(&sc.status, SCPS_FLAG_NONFINITE);
-                        sm.xq()[i] = x;
+                            for (int q = 0; q < CL; ++q) atomicOr(rank_ptr<CL>(&sc.status, q), SCPS_FLAG_NONFINITE);
+#pragma unroll
+                        for (int q = 0; q < CL; ++q) rank_ptr<CL>(sm.xq(), q)[i] = x;
                     }
                     sm.v()[i] = v;
                 }
             }
             if (do_a) {  // largest speed of the step (positive floats order as their bits)
                 const unsigned wm = __reduce_max_sync(kFull, __float_as_uint(vm2));
-                if (lane == 0) atomicMax(&sc.vmax2[b], wm);
+                if (lane < CL && wm) atomicMax(rank_ptr<CL>(&sc.vmax2[b], lane), wm);
             }
             if (tid == 0) {
                 sc.flag[nb] = 0;
                 sc.vmax2[nb] = 0u;
+                sc.zw[nb][0] = sc.zw[nb][1] = sc.zw[nb][2] = 0u;
             }
-            __syncthreads();
-            if (warp == 0 && do_b && bias) {  // atoms in a fixed order, whatever the CTA shape
+            cluster_barrier<CL>();  // every CTA has the new positions
+            if (rank == 0 && warp == 0 && do_b && bias) {  // atoms in a fixed order, whatever the CTA shape
                 float tsum = 0.f;
                 for (int i = lane; i < n; i += 32) tsum += sm.xi()[i].w;
                 tsum = warp_sum_f(tsum);
@@ -1410,7 +1438,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                 evaluate_work<ELEC, true, CL, TUBE>(sm, sc, P, nb, true, rep.rep_id, step);
             else
                 evaluate_work<ELEC, false, CL, TUBE>(sm, sc, P, nb, true, rep.rep_id, step);
-            if (!TUBE && tid < n) first = load_sums<CL>(sm, sc, nb, rank, tid, grad);
+            if (!TUBE && a0 + tid < a1) first = load_sums<CL>(sm, sc, nb, rank, a0 + tid, grad);
             if (save_next)
                 finish_evaluation<true, CL, TUBE>(sm, sc, P, nb, true);
             else
@@ -1419,14 +1447,15 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         }
     }
     __syncthreads();
-    // write back the state (rank 0; every CTA holds the same copy)
+    // write back the state: each CTA the atoms it integrated, rank 0 the scalars
+    for (int i = kTile * own_lo(tp.n_tiles, rank, CL) + tid;
+         i < min(n, kTile * own_lo(tp.n_tiles, rank + 1, CL)); i += blockDim.x) {
+        const float4 x = sm.xq()[i];
+        st.x[rep.atom_off + i] = make_float4(x.x, x.y, x.z, 0.f);
+        const float4 v = sm.v()[i];
+        st.v[rep.atom_off + i] = make_float4(v.x, v.y, v.z, 0.f);
+    }
     if (rank == 0) {
-        for (int i = tid; i < n; i += blockDim.x) {
-            const float4 x = sm.xq()[i];
-            st.x[rep.atom_off + i] = make_float4(x.x, x.y, x.z, 0.f);
-            const float4 v = sm.v()[i];
-            st.v[rep.atom_off + i] = make_float4(v.x, v.y, v.z, 0.f);
-        }
         if (tid == 0) {
             st.zm[r] = sc.zm;
             st.z[r] = sc.z;
@@ -1479,6 +1508,7 @@ k_eval_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __
         sc.z = 0.0;
         sc.status = 0;
         sc.flag[0] = 0;
+        sc.zw[0][0] = sc.zw[0][1] = sc.zw[0][2] = 0u;
         sc.work_next[0] = 0;
     }
     cluster_barrier<CL>();  // every CTA of the cluster is initialised before any remote access
@@ -1529,12 +1559,12 @@ struct ClusterLaunch {
     }
 };
 
-template <int ELEC, int CL, bool TUBE>
+template <int ELEC, int CL, bool TUBE, bool WIDE>
 static cudaError_t launch_resident_t(const TopoDev* topos, const RepDev* reps, const StateDev& st,
                                      const RunParams& P, int nta, int threads, cudaStream_t stream) {
     int lc_cap = 0;
     const size_t smem = launch_smem(nta, threads, CL, &lc_cap);
-    auto kern = k_resident<ELEC, CL, TUBE>;
+    auto kern = k_resident<ELEC, CL, TUBE, WIDE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const ClusterLaunch<CL> L(P.n_replicas, threads, smem, stream);
@@ -1543,23 +1573,23 @@ static cudaError_t launch_resident_t(const TopoDev* topos, const RepDev* reps, c
     return cudaGetLastError();
 }
 
-template <int CL>
+template <int CL, bool WIDE>
 cudaError_t launch_resident_cl(int elec, const TopoDev* topos, const RepDev* reps,
                                       const StateDev& st, const RunParams& P, int nta, int threads,
                                       cudaStream_t stream) {
     if (P.bias == 5) {  // contact-map tube bias: its own instantiation
         switch (elec) {
-            case ELEC_DDIEL: return launch_resident_t<ELEC_DDIEL, CL, true>(topos, reps, st, P, nta, threads, stream);
-            case ELEC_RF: return launch_resident_t<ELEC_RF, CL, true>(topos, reps, st, P, nta, threads, stream);
-            case ELEC_PLAIN: return launch_resident_t<ELEC_PLAIN, CL, true>(topos, reps, st, P, nta, threads, stream);
-            default: return launch_resident_t<ELEC_NONE, CL, true>(topos, reps, st, P, nta, threads, stream);
+            case ELEC_DDIEL: return launch_resident_t<ELEC_DDIEL, CL, true, WIDE>(topos, reps, st, P, nta, threads, stream);
+            case ELEC_RF: return launch_resident_t<ELEC_RF, CL, true, WIDE>(topos, reps, st, P, nta, threads, stream);
+            case ELEC_PLAIN: return launch_resident_t<ELEC_PLAIN, CL, true, WIDE>(topos, reps, st, P, nta, threads, stream);
+            default: return launch_resident_t<ELEC_NONE, CL, true, WIDE>(topos, reps, st, P, nta, threads, stream);
         }
     }
     switch (elec) {
-        case ELEC_DDIEL: return launch_resident_t<ELEC_DDIEL, CL, false>(topos, reps, st, P, nta, threads, stream);
-        case ELEC_RF: return launch_resident_t<ELEC_RF, CL, false>(topos, reps, st, P, nta, threads, stream);
-        case ELEC_PLAIN: return launch_resident_t<ELEC_PLAIN, CL, false>(topos, reps, st, P, nta, threads, stream);
-        default: return launch_resident_t<ELEC_NONE, CL, false>(topos, reps, st, P, nta, threads, stream);
+        case ELEC_DDIEL: return launch_resident_t<ELEC_DDIEL, CL, false, WIDE>(topos, reps, st, P, nta, threads, stream);
+        case ELEC_RF: return launch_resident_t<ELEC_RF, CL, false, WIDE>(topos, reps, st, P, nta, threads, stream);
+        case ELEC_PLAIN: return launch_resident_t<ELEC_PLAIN, CL, false, WIDE>(topos, reps, st, P, nta, threads, stream);
+        default: return launch_resident_t<ELEC_NONE, CL, false, WIDE>(topos, reps, st, P, nta, threads, stream);
     }
 }
 
@@ -1595,7 +1625,7 @@ template <int CL>
 int max_clusters_cl(int nta, int threads) {
     int lc_cap = 0, n = 0;
     const size_t smem = launch_smem(nta, threads, CL, &lc_cap);
-    auto kern = k_resident<ELEC_DDIEL, CL, true>;
+    auto kern = k_resident<ELEC_DDIEL, CL, true, true>;
     const ClusterLaunch<CL> L(1, threads, smem, 0);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, kern, &L.cfg) != cudaSuccess) {
@@ -1605,14 +1635,15 @@ int max_clusters_cl(int nta, int threads) {
     return n;
 }
 
-#define SCPS_CHAIN_LAUNCHERS(PREFIX, CL)                                                            \
-    PREFIX template cudaError_t launch_resident_cl<CL>(int, const TopoDev*, const RepDev*,          \
-                                                       const StateDev&, const RunParams&, int, int, \
-                                                       cudaStream_t);                               \
+#define SCPS_RESIDENT_LAUNCHERS(PREFIX, CL, WIDE)                                                   \
+    PREFIX template cudaError_t launch_resident_cl<CL, WIDE>(int, const TopoDev*, const RepDev*,    \
+                                                             const StateDev&, const RunParams&,     \
+                                                             int, int, cudaStream_t);
+#define SCPS_EVAL_LAUNCHERS(PREFIX, CL)                                                             \
     PREFIX template cudaError_t launch_eval_cl<CL>(int, const TopoDev*, const RunParams&,           \
                                                    const float*, double*, float*, double*,          \
-                                                   long long, int, int, cudaStream_t);              \
-    PREFIX template int max_clusters_cl<CL>(int, int);
+                                                   long long, int, int, cudaStream_t);
+#define SCPS_MAX_CLUSTERS(PREFIX, CL) PREFIX template int max_clusters_cl<CL>(int, int);
 
 // bytes of the kernels' static shared block
 constexpr size_t kChainStaticSmem = sizeof(Scalars);

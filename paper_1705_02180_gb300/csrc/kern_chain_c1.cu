@@ -1,6 +1,7 @@
-// Chain kernels on clusters of 1 CTA per replica or frame.
+// Chain kernels: one CTA per replica (up to 1024 threads) or frame.
 #include "kern_chain.cuh"
 
 namespace scps {
-SCPS_CHAIN_LAUNCHERS(, 1)
+SCPS_RESIDENT_LAUNCHERS(, 1, false)
+SCPS_EVAL_LAUNCHERS(, 1)
 }  // namespace scps

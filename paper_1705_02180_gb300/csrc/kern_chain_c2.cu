@@ -1,6 +1,7 @@
-// Chain kernels on clusters of 2 CTAs per replica or frame.
+// Chain kernels: two CTAs per replica or frame.
 #include "kern_chain.cuh"
 
 namespace scps {
-SCPS_CHAIN_LAUNCHERS(, 2)
+SCPS_RESIDENT_LAUNCHERS(, 2, true)
+SCPS_EVAL_LAUNCHERS(, 2)
 }  // namespace scps

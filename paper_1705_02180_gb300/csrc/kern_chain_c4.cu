@@ -1,6 +1,8 @@
-// Chain kernels on clusters of 4 CTAs per replica or frame.
+// Chain kernels: four CTAs per replica or frame.
 #include "kern_chain.cuh"
 
 namespace scps {
-SCPS_CHAIN_LAUNCHERS(, 4)
+SCPS_RESIDENT_LAUNCHERS(, 4, true)
+SCPS_EVAL_LAUNCHERS(, 4)
+SCPS_MAX_CLUSTERS(, 4)
 }  // namespace scps

@@ -31,12 +31,6 @@ constexpr double kA1 = 30.0, kA2 = 20.0, kA3 = 6.0, kS1 = 1.0, kS2 = 2.0, kS3 = 
 constexpr double kW = 0.03, kYm = 0.0, kXm = 1.5;
 constexpr int kPlaneProducers = 3;  // warps drawing noise beside the stepping warp
 
-// d < 0 from the bits of d (no FP64 instruction; false for -0 and NaN).
-__device__ __forceinline__ bool below_zero(double d) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
-    return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
-}
-
 // The lanes of a stepping warp: 32 >> lg copies of each of 1 << lg replicas; lane l holds
 // copy l >> lg of replica l & ((1 << lg) - 1). With four copies or more, like terms are
 // computed one per copy and exchanged.

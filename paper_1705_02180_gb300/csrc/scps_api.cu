@@ -308,7 +308,21 @@ int atoms_per_replica(const scps_system* s, int r) {
     return is_2d(s->model) ? 1 : s->topos[s->rep_topo[r]].n;
 }
 
+// Threads of a resident CTA that shares its SM where its size allows two (256, 512).
 int auto_threads(int nta) {
+    if (nta <= 256) return 256;
+    if (nta <= 640) return 512;
+    return kMaxThreadsPair;
+}
+
+// Threads of a resident CTA with an SM to itself: 768, but 512 where a cluster leaves a CTA few
+// atoms (304 atoms on four CTAs 8.7 us per step against 9.2, 560 on eight 11.8 against 12.3).
+int cta_threads(int nta, int cluster) {
+    return cluster >= 4 && nta / cluster <= 96 ? 512 : kMaxThreadsPair;
+}
+
+// Threads of a frame evaluation with several frames per SM.
+int eval_threads(int nta) {
     if (nta <= 256) return 256;
     if (nta <= 640) return 512;
     return 1024;
@@ -330,16 +344,15 @@ void drop_graphs(scps_system* s) {
 }
 
 // CTAs per replica when the caller leaves the choice open: two while they leave no SM without a
-// replica of its own; four where the replicas are few enough for all clusters to run at once
-// and large enough to gain from it (us per step, one to twenty replicas: 1200 atoms 37.9
-// against 47.7 with two, 560 atoms 18.0 against 20.8, 304 atoms 11.0 against 11.1; a second
-// wave of clusters would double the time, and eight CTAs lose to the reads of each other's
-// partials: 46.7, 25.3 and 15.6).
+// replica of its own; four or eight where the replicas are few enough for all clusters to run at
+// once (a second wave would double the time) and large enough for each CTA to have work. Us per
+// step with 1, 2, 4, 8 CTAs: 1200 atoms 84.7, 46.0, 28.2, 21.4; 560 atoms 33.0, 19.3, 13.8, 12.3;
+// 304 atoms 15.5, 10.8, 9.2, 9.8; 200 atoms 10.6, 8.0, 7.0, 8.6; 128 atoms 7.0, 5.4, 5.5, 7.4.
 int auto_cluster(int R, int nta, int n_sm, int threads) {
     if (threads > kMaxThreadsPair || 2 * R > n_sm) return 1;
-    if (nta >= 448 && 4 * R <= n_sm &&
-        R <= chain_max_clusters(4, nta, threads ? threads : kMaxThreadsPair))
-        return 4;
+    const int th = threads ? threads : kMaxThreadsPair;
+    if (nta >= 512 && 8 * R <= n_sm && R <= chain_max_clusters(8, nta, th)) return 8;
+    if (nta >= 192 && 4 * R <= n_sm && R <= chain_max_clusters(4, nta, th)) return 4;
     return 2;
 }
 
@@ -623,8 +636,9 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
                          ? (2 * R <= n_sm && d->threads <= kMaxThreadsPair ? 2 : 1)
                          : auto_cluster(R, s->nta, n_sm, d->threads);
         const bool one_cta_per_sm = (long long)R * s->cluster <= n_sm;
-        s->threads = d->threads ? d->threads : (one_cta_per_sm ? 1024 : auto_threads(s->nta));
-        if (s->cluster > 1 && !d->threads) s->threads = std::min(s->threads, kMaxThreadsPair);
+        s->threads = d->threads ? d->threads
+                     : one_cta_per_sm ? cta_threads(s->nta, s->cluster)
+                                      : auto_threads(s->nta);
         s->steps_per_graph = d->steps_per_graph > 0 ? d->steps_per_graph : 1000;
         if (!s->is_box && d->exec == SCPS_EXEC_RESIDENT) {
             const size_t smem = resident_smem_bytes(s->nta);
@@ -1122,7 +1136,7 @@ int scps_energy_forces(scps_system* s, int32_t topo, int64_t n_frames, const flo
     for (long long f0 = 0; f0 < n_frames; f0 += per_launch) {
         const long long nf = std::min(per_launch, n_frames - f0);
         const int cl = eval_cluster(nf, n_sm);
-        const int threads = nf * cl <= n_sm ? 1024 : auto_threads(nta);
+        const int threads = nf * cl <= n_sm ? 1024 : eval_threads(nta);
         SCPS_CU(launch_eval(s->d.elec, s->d_topos + topo, P, X + f0 * n3, U + f0,
                             F ? F + f0 * n3 : nullptr, z ? z + f0 : nullptr, nf, nta, threads, cl,
                             (cudaStream_t)stream));
@@ -1721,7 +1735,7 @@ int scps_autotune(scps_system* s, int32_t probe_steps, int32_t use_cache, scps_t
     const int n_plans = sizes.size() > 1 ? 2 : 1;
     for (int plan = 0; plan < n_plans; ++plan)
         for (int cl : {1, 2})
-            for (int th : {256, 512, cl == 2 ? kMaxThreadsPair : 1024}) {
+            for (int th : {256, 512, kMaxThreadsPair}) {
                 std::vector<int> c{plan, cl, th};
                 if (c != cands[0]) cands.push_back(c);
             }

@@ -89,6 +89,12 @@ __device__ __forceinline__ float fix2f(long long v) {
     return fmaf((float)hi, 4294967296.0f, (float)lo) * kFixInv;
 }
 
+// d < 0 from the bits of d (no FP64 instruction; false for -0 and NaN).
+__device__ __forceinline__ bool below_zero(double d) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+    return b > 0x8000000000000000ull && b <= 0xfff0000000000000ull;
+}
+
 // ---------------------------------------------------------------------------
 // Two FP32 values per instruction (sm_100 and later). Each half is rounded as the scalar
 // operation would round it, so the packed forms give the same bits; the FMA pipe takes two

@@ -75,9 +75,10 @@ struct RepDev {
 //     sentinel slot nta; block I owns room for its 8 (nbs - 1 - I) later atoms in whole
 //     chunks, from offset list_jl_off(nbs, I);
 //   item tables (uint32), one per CTA of a cluster: (I << 17 | near << 16 | chunk);
-//   exclusion masks (kListChunk bytes), one per item of those tables: bit a of byte s set when
-//     chunk entry s and block atom a form an excluded pair (items near their block only).
+//   exclusion masks, kListMasks bytes per block: bit a of byte s set when the block's entry s and
+//     its atom a form an excluded pair (entries near the block, which come first).
 constexpr int kListChunk = 16;
+constexpr int kListMasks = 2 * kListChunk;  // entries less than kExclWindow beyond the block: < 32
 __host__ __device__ __forceinline__ long long list_jl_off(int nbs, int I) {
     // sum over k < I of 16 ceil((nbs - 1 - k) / 2)
     return 16ll * ((long long)I * (nbs >> 1) - ((long long)I * I >> 2));
@@ -97,7 +98,7 @@ __host__ __device__ __forceinline__ long long list_items_bytes(int nbs) {
 }
 __host__ __device__ __forceinline__ long long list_slab_bytes(int nta) {
     const int nbs = nta / 8;
-    return list_jl_bytes(nbs) + list_items_bytes(nbs) + kListChunk * (list_items_cap(nbs) + 16);
+    return list_jl_bytes(nbs) + list_items_bytes(nbs) + (long long)kListMasks * nbs;
 }
 
 // Replica state and outputs (device pointers).
