@@ -841,7 +841,7 @@ __device__ __forceinline__ AtomSums load_sums(const Shared& sm, Scalars& sc, int
 // thread of every CTA of the cluster; on return the CTA is synchronised (the counts are
 // written again only after the cluster barrier of an evaluation).
 template <int CL>
-__device__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
+__device__ __noinline__ void build_list(const Shared& sm, Scalars& sc, float rlist2) {
     const TopoDev& tp = sc.tp;
     const ListDev L = sc.list;
     const int n = tp.n_atoms, nb = (n + 7) >> 3;
