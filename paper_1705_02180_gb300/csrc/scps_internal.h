@@ -178,6 +178,8 @@ struct BoxDev {
     float4* pos_ref;  // positions at the last rebuild
     float4* clo;      // [replica][4 nt] boxes of the 8-slot clusters (clo.w: 1 = reference LJ only)
     float4* chi;
+    float4* tlo;      // [replica][nt] boxes of the tiles
+    float4* thi;
     uint32_t* ent;    // [replica][4 nt][max_ent] pair list of each 8-slot i cluster c: its own 8
                       // slots, then the slots j of clusters after c within r_list of some atom
                       // of c, ascending, padded to a multiple of 8 with kBoxNoSlot; an entry is
