@@ -203,8 +203,9 @@ __global__ void __launch_bounds__(kSortThreads) k_box_scan(BoxDev B, int r0) {
     }
 }
 
-// Rebuild, step 1d (atoms): scatter into the padded column layout. Within a key
-// the atomics give an arbitrary order, which step 1e replaces by atom-id order.
+// Rebuild, step 1d (atoms): the atom ids go into the padded column layout, positions and
+// velocities into atom order (step 1f gathers them). Within a key the atomics give an
+// arbitrary order, which step 1e replaces by atom-id order.
 __global__ void k_box_scatter(BoxDev B, int r0) {
     const int r = blockIdx.y + r0;
     if (!B.need[r]) return;
@@ -218,91 +219,43 @@ __global__ void k_box_scatter(BoxDev B, int r0) {
     const int p = atomicAdd(&B.hist[(size_t)r * kNumKeys + k], 1);
     const int c = k / B.nz;
     const int dst = col_tile[c] * 32 + (p - col_first[c]);
-    B.pos2[base + dst] = B.pos[base + s];
-    B.vel2[base + dst] = B.vel[base + s];
+    B.pos2[base + a] = B.pos[base + s];
+    B.vel2[base + a] = B.vel[base + s];
     B.id2[base + dst] = a;
 }
 
-// Rebuild, step 1e (keys): put each key's slots in atom-id order (a key holds a
-// few atoms); hist[k] now ends key k, so key k spans [hist[k - 1], hist[k]).
+// Rebuild, step 1e (slots): each key's atoms in id order, from id2 to id; a slot's rank is
+// the number of smaller ids of its key (a few loads side by side; an insertion sort per key, a
+// chain of dependent ones, took 51 us where this takes 8). hist[k] now ends key k, so
+// key k spans [hist[k - 1], hist[k]).
 __global__ void k_box_keyorder(BoxDev B, int r0) {
     const int r = blockIdx.y + r0;
     if (!B.need[r]) return;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= B.ncol * B.ncol * B.nz) return;
+    const int d = blockIdx.x * blockDim.x + threadIdx.x;
+    if (d >= B.np) return;
+    const size_t base = (size_t)r * B.np;
+    const int a = B.id2[base + d];
+    if (a < 0) {
+        B.id[base + d] = -1;
+        return;
+    }
     const int* hist = B.hist + (size_t)r * kNumKeys;
-    const int lo = k > 0 ? hist[k - 1] : 0, hi = hist[k];
-    if (hi - lo < 2) return;
     const int* col_first = B.colinfo + (size_t)r * 2 * (kMaxCols + 1);
     const int* col_tile = col_first + kMaxCols + 1;
+    const int k = B.key[base + B.slot_of[(size_t)r * B.n_atoms + a]];
     const int c = k / B.nz;
-    const size_t off = (size_t)r * B.np + col_tile[c] * 32 - col_first[c];
-    int* id2 = B.id2 + off;
-    float4* pos2 = B.pos2 + off;
-    float4* vel2 = B.vel2 + off;
-    for (int q = lo + 1; q < hi; ++q) {  // insertion sort by id
-        const int ia = id2[q];
-        const float4 pa = pos2[q], va = vel2[q];
-        int u = q - 1;
-        while (u >= lo && id2[u] > ia) {
-            id2[u + 1] = id2[u];
-            pos2[u + 1] = pos2[u];
-            vel2[u + 1] = vel2[u];
-            --u;
-        }
-        id2[u + 1] = ia;
-        pos2[u + 1] = pa;
-        vel2[u + 1] = va;
-    }
+    const int lo = k > 0 ? hist[k - 1] : 0, hi = hist[k];
+    const size_t off = base + col_tile[c] * 32 - col_first[c];
+    int rank = 0;
+    for (int q = lo; q < hi; ++q) rank += B.id2[off + q] < a ? 1 : 0;
+    B.id[off + lo + rank] = a;
 }
 
-// Rebuild, step 1f (one warp per tile): inside each tile, two halves of 16 by x,
-// each ordered by y (padding last), so that slots 8q .. 8q+7 form compact
-// clusters; final slot arrays, reference positions, LJ parameters, slot_of.
-__global__ void k_box_subsort(BoxDev B, const TopoDev* __restrict__ topo, int r0) {
-    const int r = blockIdx.y + r0;
-    if (!B.need[r]) return;
-    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= B.nt) return;
-    const int lane = threadIdx.x & 31;
-    const size_t base = (size_t)r * B.np;
-    const int s0 = t * 32 + lane;
-    const int a = B.id2[base + s0];
-    const bool valid = a >= 0;
-    const float4 p = B.pos2[base + s0];
-    const float4 v = B.vel2[base + s0];
-    const float kx = valid ? p.x : 3.0e38f, ky = valid ? p.y : 3.0e38f;
-    const int rx = warp_rank(kx, lane, true, kFullB);
-    const unsigned upper = __ballot_sync(kFullB, rx >= 16);
-    const bool hi = rx >= 16;
-    const int ry = warp_rank(ky, lane, true, hi ? upper : ~upper);
-    const int s = t * 32 + (hi ? 16 : 0) + ry;
-    if (valid) {
-        B.pos[base + s] = p;
-        B.vel[base + s] = v;
-        B.id[base + s] = a;
-        B.pos_ref[base + s] = p;
-        B.par[base + s] = topo->lj[a];
-        B.slot_of[(size_t)r * B.n_atoms + a] = s;
-    } else {
-        const float4 far = make_float4(1.0e5f * (float)(s + 1), 0.f, 0.f, 0.f);
-        B.pos[base + s] = far;
-        B.vel[base + s] = make_float4(0.f, 0.f, 0.f, 0.f);
-        B.id[base + s] = -1;
-        B.pos_ref[base + s] = far;
-        B.par[base + s] = make_float2(0.f, 0.f);
-    }
-}
-
-// Rebuild step 2 (one warp per tile): boxes of the tile and of each 8-slot cluster, and whether it holds
-// chain atoms or only atoms with the LJ parameters of the last atom (a solvent site), whose
-// pair constants the pair kernel then computes once.
-__global__ void k_box_tiles(BoxDev B, const TopoDev* __restrict__ topo, int r0) {
-    const int r = blockIdx.y + r0;
-    if (!B.need[r]) return;
-    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= B.nt) return;
-    const int lane = threadIdx.x & 31;
+// Rebuild step 2 (one warp per tile, once its slots are written): boxes of the tile and of each
+// 8-slot cluster, and whether the cluster holds chain atoms or only atoms with the LJ parameters
+// of the last atom (a solvent site), whose pair constants the pair kernel then computes once.
+__device__ __forceinline__ void box_tile_bounds(const BoxDev& B, const TopoDev* __restrict__ topo,
+                                                int r, int t, int lane) {
     const int s = t * 32 + lane;
     const float4 p = B.pos[(size_t)r * B.np + s];
     const int a = B.id[(size_t)r * B.np + s];
@@ -343,6 +296,46 @@ __global__ void k_box_tiles(BoxDev B, const TopoDev* __restrict__ topo, int r0) 
         B.tlo[(size_t)r * B.nt + t] = make_float4(lx, ly, lz, 0.f);
         B.thi[(size_t)r * B.nt + t] = make_float4(hx, hy, hz, 0.f);
     }
+}
+
+// Rebuild, step 1f (one warp per tile): inside each tile, two halves of 16 by x,
+// each ordered by y (padding last), so that slots 8q .. 8q+7 form compact
+// clusters; final slot arrays, reference positions, LJ parameters, slot_of.
+__global__ void k_box_subsort(BoxDev B, const TopoDev* __restrict__ topo, int r0) {
+    const int r = blockIdx.y + r0;
+    if (!B.need[r]) return;
+    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (t >= B.nt) return;
+    const int lane = threadIdx.x & 31;
+    const size_t base = (size_t)r * B.np;
+    const int s0 = t * 32 + lane;
+    const int a = B.id[base + s0];  // (the other lanes read theirs before any write below)
+    const bool valid = a >= 0;
+    const float4 p = B.pos2[base + max(a, 0)];
+    const float4 v = B.vel2[base + max(a, 0)];
+    const float kx = valid ? p.x : 3.0e38f, ky = valid ? p.y : 3.0e38f;
+    const int rx = warp_rank(kx, lane, true, kFullB);
+    const unsigned upper = __ballot_sync(kFullB, rx >= 16);
+    const bool hi = rx >= 16;
+    const int ry = warp_rank(ky, lane, true, hi ? upper : ~upper);
+    const int s = t * 32 + (hi ? 16 : 0) + ry;
+    if (valid) {
+        B.pos[base + s] = p;
+        B.vel[base + s] = v;
+        B.id[base + s] = a;
+        B.pos_ref[base + s] = p;
+        B.par[base + s] = topo->lj[a];
+        B.slot_of[(size_t)r * B.n_atoms + a] = s;
+    } else {
+        const float4 far = make_float4(1.0e5f * (float)(s + 1), 0.f, 0.f, 0.f);
+        B.pos[base + s] = far;
+        B.vel[base + s] = make_float4(0.f, 0.f, 0.f, 0.f);
+        B.id[base + s] = -1;
+        B.pos_ref[base + s] = far;
+        B.par[base + s] = make_float2(0.f, 0.f);
+    }
+    __syncwarp();
+    box_tile_bounds(B, topo, r, t, lane);
 }
 
 // Rebuild step 3 (one warp per 8-slot i cluster c): the pair list of c. Its own 8 slots
@@ -924,13 +917,15 @@ __global__ void __launch_bounds__(32 * kPairWarps, kPairRegWarps / kPairWarps) k
 __device__ __forceinline__ float4 take_nb_force(const BoxDev& B, int r, int s) {
     const size_t np = (size_t)B.np;
     unsigned* L = B.facc + 6 * (size_t)r * np + s;
+    unsigned w[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) w[d] = L[d * np];
     float f[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {  // 2^-13 to 2^-20 units
-        f[d] = fix2f(join_coarse((int)L[(3 + d) * np], L[d * np], kBoxShift) * 128);
-        L[d * np] = 0u;
-        L[(3 + d) * np] = 0u;
-    }
+    for (int d = 0; d < 3; ++d)  // 2^-13 to 2^-20 units
+        f[d] = fix2f(join_coarse((int)w[3 + d], w[d], kBoxShift) * 128);
+#pragma unroll
+    for (int d = 0; d < 6; ++d) L[d * np] = 0u;
     return make_float4(f[0], f[1], f[2], 0.f);
 }
 
@@ -1097,8 +1092,10 @@ __global__ void __launch_bounds__(512) k_box_chain(BoxDev B, const TopoDev* __re
 }
 
 // BAOAB half steps per slot: B closes the evaluated step, A starts the next one. The largest
-// squared displacement since the list build goes to the replica's bound with one atomic per
-// warp (every lane reaches the warp reduction; the slots of a warp share their replica).
+// squared displacement since the list build goes to the replica's bound with at most one atomic
+// per warp (every lane reaches the warp reduction; the slots of a warp share their replica).
+// Latency bounds it: loads ahead of all stores, and an atomic only where it raises the bound
+// (one per warp on 16 addresses of a line made it 48 us for 16 x 24 560 sites, now 19).
 __global__ void k_box_integrate(BoxDev B, const TopoDev* __restrict__ topo, StateDev st,
                                 RunParams P, const uint32_t* __restrict__ rep_ids, long long step,
                                 int do_b, int do_a, int step_from_state) {
@@ -1108,20 +1105,23 @@ __global__ void k_box_integrate(BoxDev B, const TopoDev* __restrict__ topo, Stat
     const size_t base = (size_t)r * B.np;
     float d2 = 0.f;
     if (s < B.np) {
-        float4 f = take_nb_force(B, r, s);  // also clears the j part (frozen replicas too)
+        // all loads that need nothing but the slot go out together
         const int a = B.id[base + s];
-        if (a >= 0 && st.status[r] == 0) {
-            const TopoDev& tp = *topo;
+        float4 v = B.vel[base + s];
+        float4 x = B.pos[base + s];
+        const float4 p0 = B.pos_ref[base + s];
+        const bool live = a >= 0 && st.status[r] == 0;
+        const TopoDev& tp = *topo;
+        const float im = tp.inv_m[max(a, 0)], sd = tp.noise_sd[max(a, 0)];
+        float4 f = take_nb_force(B, r, s);  // also clears the sums (frozen replicas too)
+        if (live) {
             if (a < B.n_chain) {
                 const float4 c = B.fch[(size_t)r * B.n_chain + a];
                 f.x += c.x;
                 f.y += c.y;
                 f.z += c.z;
             }
-            const float im = tp.inv_m[a];
             const float hdt = P.half_dt;
-            float4 v = B.vel[base + s];
-            float4 x = B.pos[base + s];
             if (do_b) {
                 v.x = fmaf(hdt * im, f.x, v.x);
                 v.y = fmaf(hdt * im, f.y, v.y);
@@ -1137,7 +1137,6 @@ __global__ void k_box_integrate(BoxDev B, const TopoDev* __restrict__ topo, Stat
                 const uint4 rb = philox4x32_10(make_uint4((uint32_t)a, rep_ids[r], (uint32_t)step, 0u),
                                                P.key0, P.key1);
                 const float4 xi = normals4_f32(rb);
-                const float sd = tp.noise_sd[a];
                 v.x = fmaf(P.c1, v.x, sd * xi.x);
                 v.y = fmaf(P.c1, v.y, sd * xi.y);
                 v.z = fmaf(P.c1, v.z, sd * xi.z);
@@ -1148,7 +1147,6 @@ __global__ void k_box_integrate(BoxDev B, const TopoDev* __restrict__ topo, Stat
                       isfinite(v.y) && isfinite(v.z)))
                     atomicOr(&st.status[r], SCPS_FLAG_NONFINITE);
                 B.pos[base + s] = x;
-                const float4 p0 = B.pos_ref[base + s];
                 const float ddx = x.x - p0.x, ddy = x.y - p0.y, ddz = x.z - p0.z;
                 d2 = fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz));
             }
@@ -1157,7 +1155,8 @@ __global__ void k_box_integrate(BoxDev B, const TopoDev* __restrict__ topo, Stat
     }
     if (do_a) {  // non-negative floats order as unsigned
         const unsigned m = __reduce_max_sync(kFullB, __float_as_uint(d2));
-        if ((threadIdx.x & 31) == 0 && m != 0u) atomicMax(&B.maxd2[r], m);
+        // (the bound only grows: a warp below it, whatever its age, has nothing to add)
+        if ((threadIdx.x & 31) == 0 && m > __ldcg(&B.maxd2[r])) atomicMax(&B.maxd2[r], m);
     }
 }
 
@@ -1208,10 +1207,9 @@ static void box_rebuild(const BoxDev& B, const TopoDev* topo, const StateDev& st
     k_box_key<<<dim3((B.np + 255) / 256, nr), 256, 0, s>>>(B, r0);
     k_box_scan<<<nr, kSortThreads, 0, s>>>(B, r0);
     k_box_scatter<<<dim3((B.n_atoms + 255) / 256, nr), 256, 0, s>>>(B, r0);
-    k_box_keyorder<<<dim3((B.ncol * B.ncol * B.nz + 255) / 256, nr), 256, 0, s>>>(B, r0);
+    k_box_keyorder<<<dim3((B.np + 255) / 256, nr), 256, 0, s>>>(B, r0);
     const dim3 gt((B.nt + 3) / 4, nr);       // one warp per tile
     k_box_subsort<<<gt, 128, 0, s>>>(B, topo, r0);
-    k_box_tiles<<<gt, 128, 0, s>>>(B, topo, r0);
     k_box_list<<<dim3(B.nt, nr), 128, 0, s>>>(B, st, r0);
 }
 
