@@ -7,8 +7,10 @@
 #include <cstdio>
 #include <cstring>
 #include <limits>
+#include <functional>
 #include <map>
 #include <mutex>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -130,6 +132,7 @@ struct scps_system {
         RepDev* d_reps = nullptr;  // this group's replicas (owned by `allocs`)
         int count = 0, nta = 0, cluster = 1, threads = 1024;
     };
+    bool auto_shape = false;  // the caller left cluster size and threads open
     std::vector<Group> groups;
     int plan = 0;  // 0: one launch, replicas by decreasing size; 1: one launch per size class
     std::vector<cudaStream_t> fork_streams;
@@ -308,12 +311,11 @@ int atoms_per_replica(const scps_system* s, int r) {
     return is_2d(s->model) ? 1 : s->topos[s->rep_topo[r]].n;
 }
 
-// Threads of a resident CTA that shares its SM where its size allows two (256, 512).
-int auto_threads(int nta) {
-    if (nta <= 256) return 256;
-    if (nta <= 640) return 512;
-    return kMaxThreadsPair;
-}
+// Threads of a resident CTA when there are more CTAs than SMs: 256 for small chains, so that
+// several share an SM, else one CTA of 768 at a time (304 replicas on 152 SMs: 560 atoms 62.9 us
+// per step against 68.2 with two CTAs of 512 threads per SM, 400 atoms 39.0 against 41.7, 304
+// atoms 28.4 against 28.9).
+int auto_threads(int nta) { return nta <= 256 ? 256 : kMaxThreadsPair; }
 
 // Threads of a resident CTA with an SM to itself: 768, but 512 where a cluster leaves a CTA few
 // atoms (304 atoms on four CTAs 8.7 us per step against 9.2, 560 on eight 11.8 against 12.3).
@@ -368,10 +370,53 @@ int eval_cluster(long long nf, int n_sm) {
 
 int tile_atoms(int n) { return ((n + kTile - 1) / kTile) * kTile; }
 
+// Measured time per step (us) of a chain of n atoms on one CTA and on a cluster of four
+// (within 10 % from 200 to 1200 atoms; only their ratios matter here).
+double step_cost_1(int n) { return 3.0 + 0.030 * n + 2.7e-5 * n * n; }
+double step_cost_4(int n) { return 4.5 + 0.0145 * n + 4.4e-6 * n * n; }
+
+// How many of the replicas of one CTA each (`atoms`: their sizes, decreasing) run as clusters
+// of four CTAs instead, started before the others. With a few more replicas than SMs the
+// last ones would run alone in a second wave; as clusters they take four SMs for a
+// third of the time. The choice is the one with the shortest makespan of one CTA per SM, longest
+// first, when it saves more than 5 % (170 replicas on 152 SMs: 560 atoms 44.9 us per step
+// against 62.9 without, 1200 atoms 105 against 154; from 230 replicas on nothing is gained).
+int split_clusters(const std::vector<int>& atoms, int n_sm) {
+    const int R = (int)atoms.size();
+    if (R <= n_sm || R > 16 * n_sm) return 0;
+    const int nta = tile_atoms(atoms[0]);
+    const int kmax = std::min({R, n_sm / 4, chain_max_clusters(4, nta, cta_threads(nta, 4))});
+    double best = 0.0, none = 0.0;
+    int best_k = 0;
+    for (int k = 0; k <= kmax; ++k) {
+        // SM k takes its jobs in turn: a heap of the times at which SMs become free
+        std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+        double end = 0.0;
+        for (int m = 0; m < n_sm; ++m) {
+            const double f = m < 4 * k ? step_cost_4(atoms[m / 4]) : 0.0;
+            end = std::max(end, f);
+            free_at.push(f);
+        }
+        for (int r = k; r < R; ++r) {
+            const double f = free_at.top() + step_cost_1(atoms[r]);
+            free_at.pop();
+            free_at.push(f);
+            end = std::max(end, f);
+        }
+        if (k == 0) none = best = end;
+        if (end < best) {
+            best = end;
+            best_k = k;
+        }
+    }
+    return best < 0.95 * none ? best_k : 0;
+}
+
 // Launch groups of the resident form. plan 0: one group, replicas by decreasing
-// size (large replicas start first, small ones fill the last wave); plan 1: one
-// group per size class (tile-rounded atom count), each with shared memory for its
-// own size. Every group gets the given cluster size and threads per CTA.
+// size (large replicas start first, small ones fill the last wave), before it a group of
+// four-CTA clusters where split_clusters asks for one (the launch shape left open by the
+// caller only); plan 1: one group per size class (tile-rounded atom count), each with shared
+// memory for its own size. Other groups get the given cluster size and threads per CTA.
 int set_groups(scps_system* s, int plan, int cluster, int threads) {
     if (cluster > 1 && threads > kMaxThreadsPair)
         return fail(SCPS_ERR_INVALID_ARG, "a CTA cluster takes at most %d threads per CTA",
@@ -383,8 +428,17 @@ int set_groups(scps_system* s, int plan, int cluster, int threads) {
         return s->topos[s->rep_topo[a]].n > s->topos[s->rep_topo[b]].n;
     });
     std::vector<std::vector<int>> members;
+    int n_split = 0;
+    if (plan == 0 && s->auto_shape && cluster == 1 && threads == kMaxThreadsPair) {
+        int n_sm = 0;
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
+        std::vector<int> atoms(R);
+        for (int k = 0; k < R; ++k) atoms[k] = s->topos[s->rep_topo[order[k]]].n;
+        n_split = split_clusters(atoms, n_sm);
+    }
     if (plan == 0) {
-        members.push_back(order);
+        if (n_split > 0) members.emplace_back(order.begin(), order.begin() + n_split);
+        members.emplace_back(order.begin() + n_split, order.end());
     } else {
         int last = -1;
         for (int r : order) {
@@ -401,8 +455,9 @@ int set_groups(scps_system* s, int plan, int cluster, int threads) {
         int na = 0;
         for (int r : m) na = std::max(na, s->topos[s->rep_topo[r]].n);
         g.nta = plan == 0 ? s->nta : tile_atoms(na);
-        g.cluster = cluster;
-        g.threads = threads;
+        const bool split = n_split > 0 && groups.empty();
+        g.cluster = split ? 4 : cluster;
+        g.threads = split ? cta_threads(g.nta, 4) : threads;
         std::vector<RepDev> reps(m.size());
         for (size_t k = 0; k < m.size(); ++k) {
             const int r = m[k];
@@ -646,6 +701,7 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
                 return bail(fail(SCPS_ERR_UNSUPPORTED,
                                  "%d atoms need %zu B of shared memory per CTA, above the limit; "
                                  "use the plain execution form", s->max_atoms, smem));
+            s->auto_shape = !d->cluster_size && !d->threads;
             rc = set_groups(s, 0, s->cluster, s->threads);
             if (rc) return bail(rc);
         }

@@ -125,3 +125,21 @@ def test_hvp_of_every_cluster_size_agrees(torch_cuda, n):
     _, ref = oracle.ForceField.from_chain(c).hvp(X[0].double().cpu().numpy(), V[0].double().cpu().numpy())
     assert np.abs(whole[0].cpu().numpy() - ref).max() <= 1e-5 * np.sqrt((ref ** 2).sum(1).mean())
     s.close()
+
+
+def test_replicas_beyond_one_per_sm_agree(torch_cuda):
+    # a few replicas more than SMs: some run as clusters of four beside the others
+    n_sm = torch_cuda.cuda.get_device_properties(0).multi_processor_count
+    c, R = cut(synth.make_chain(19, seed=1), 290), n_sm + 9
+    runs = []
+    for kw in (dict(), dict(cluster_size=1, threads=768)):
+        s = system(c, R=R, save_interval=10, max_frames=4, **kw)
+        assert s.info()["launch_groups"] == (1 if kw else 2)
+        s.step(25)
+        assert s.status()[0] == 0
+        st, paths = s.get_state(), s.collect_paths()
+        runs.append([st[k] for k in ("x", "v", "zm", "T", "step")] +
+                    [np.stack([p[k] for p in paths]) for k in ("frames", "z", "epot", "T")])
+        s.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
