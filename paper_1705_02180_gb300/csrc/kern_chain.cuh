@@ -828,6 +828,38 @@ __device__ __forceinline__ AtomSums load_sums(const Shared& sm, Scalars& sc, int
     return a;
 }
 
+// The same for the atom of a group of four lanes, one component per lane (a quarter of the remote
+// loads in a row); every lane of the group gets the result. Called by whole warps.
+template <int CL>
+__device__ __forceinline__ AtomSums load_sums4(const Shared& sm, Scalars& sc, int b, int rank, int i,
+                                               bool grad) {
+    const Part F = sm.F(b), G = sm.G(b);
+    const int lane = threadIdx.x & 31, k = 3 * i + min(lane & 3, 2);
+    int fh = F.H[k], hg = 0, flags = sc.flag[b];
+    unsigned fl = F.L[k], gl = grad ? G.L[k] : 0u;
+#pragma unroll
+    for (int q = 1; q < CL; ++q) {
+        const int p = (rank + q) & (CL - 1);
+        flags |= *rank_ptr<CL>(&sc.flag[b], p);
+        fh += rank_ptr<CL>(F.H, p)[k];
+        fl += rank_ptr<CL>(F.L, p)[k];
+        gl += grad ? rank_ptr<CL>(G.L, p)[k] : 0u;
+    }
+    if (grad && (flags & kFlagGradCoarse))
+        for (int p = 0; p < CL; ++p) hg += rank_ptr<CL>(G.H, p)[k];
+    const float f = fix2f(join_coarse(fh, fl, sm.fsh) * 128);
+    const float g = grad ? fix2f(join_coarse(hg, gl, sm.gsh)) : 0.f;
+    const int l0 = lane & ~3;
+    AtomSums a;
+    a.fx = __shfl_sync(kFull, f, l0);
+    a.fy = __shfl_sync(kFull, f, l0 + 1);
+    a.fz = __shfl_sync(kFull, f, l0 + 2);
+    a.gx = __shfl_sync(kFull, g, l0);
+    a.gy = __shfl_sync(kFull, g, l0 + 1);
+    a.gz = __shfl_sync(kFull, g, l0 + 2);
+    return a;
+}
+
 // ---------------------------------------------------------------------------
 // Pair list build
 // ---------------------------------------------------------------------------
@@ -1311,8 +1343,27 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         // the atoms this CTA integrates; their new positions go to every CTA
         const int a0 = kTile * own_lo(tp.n_tiles, rank, CL),
                   a1 = min(n, kTile * own_lo(tp.n_tiles, rank + 1, CL));
+        // One thread per atom, four lanes where the threads suffice (the first of them goes on
+        // to integrate it); warp 0, which decides, takes no atoms where the others suffice. The
+        // latency of the remote loads is what this part of a step waits for: one replica of 560
+        // atoms (eight CTAs) 11.7 -> 10.4 us per step, of 304 (four) 8.65 -> 8.06, 64 of 560
+        // (two, warp 0 freed) 19.2 -> 18.9.
+        const int own = a1 - a0;
+        const bool four = CL > 2 && 4 * own + 32 <= (int)blockDim.x;
+        const int it = own * (four ? 4 : 1) + 32 <= (int)blockDim.x ? tid - 32 : tid;
+        const int i0 = it < 0 ? a1 : a0 + (four ? it >> 2 : it);  // this thread's first atom
+        auto load_first = [&](int b) -> AtomSums {
+            AtomSums a = {};
+            if (four) {
+                if (it >= 0 && a0 + ((it & ~31) >> 2) < a1)
+                    a = load_sums4<CL>(sm, sc, b, rank, min(i0, a1 - 1), grad);
+            } else if (i0 < a1) {
+                a = load_sums<CL>(sm, sc, b, rank, i0, grad);
+            }
+            return a;
+        };
         AtomSums first = {};
-        if (!TUBE && a0 + tid < a1) first = load_sums<CL>(sm, sc, (int)(step & 1), rank, a0 + tid, grad);
+        if (!TUBE) first = load_first((int)(step & 1));
         finish_evaluation<false, CL, TUBE>(sm, sc, P, (int)(step & 1), true);
         // position of `step` in the save cycle and ring slot of the next frame, kept as
         // counters so that the loop has no 64-bit divisions
@@ -1334,10 +1385,10 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                 for (int i = tid; i < 3 * sm.na8() / 2; i += blockDim.x)
                     f[i] = g[i] = make_uint4(0u, 0u, 0u, 0u);
             }
-            for (int base = a0; base < a1; base += blockDim.x) {
-                const int i = base + tid;
-                if (i < a1) {
-                    const AtomSums a = !TUBE && base == a0 ? first : load_sums<CL>(sm, sc, b, rank, i, grad);
+            if (TUBE) first = load_first(b);
+            if (!four || (tid & 3) == 0) {
+                for (int i = i0; i < a1; i += blockDim.x) {
+                    const AtomSums a = i == i0 ? first : load_sums<CL>(sm, sc, b, rank, i, grad);
                     float4 v = sm.v()[i];
                     const float im = v.w;
                     float fx = a.fx, fy = a.fy, fz = a.fz;
@@ -1438,7 +1489,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                 evaluate_work<ELEC, true, CL, TUBE>(sm, sc, P, nb, true, rep.rep_id, step);
             else
                 evaluate_work<ELEC, false, CL, TUBE>(sm, sc, P, nb, true, rep.rep_id, step);
-            if (!TUBE && a0 + tid < a1) first = load_sums<CL>(sm, sc, nb, rank, a0 + tid, grad);
+            if (!TUBE) first = load_first(nb);
             if (save_next)
                 finish_evaluation<true, CL, TUBE>(sm, sc, P, nb, true);
             else
