@@ -345,16 +345,17 @@ void drop_graphs(scps_system* s) {
     s->graph_defs.clear();
 }
 
-// CTAs per replica when the caller leaves the choice open: two while they leave no SM without a
-// replica of its own; four or eight where the replicas are few enough for all clusters to run at
-// once (a second wave would double the time) and large enough for each CTA to have work. Us per
-// step with 1, 2, 4, 8 CTAs: 1200 atoms 84.7, 46.0, 28.2, 21.4; 560 atoms 33.0, 19.3, 13.8, 12.3;
-// 304 atoms 15.5, 10.8, 9.2, 9.8; 200 atoms 10.6, 8.0, 7.0, 8.6; 128 atoms 7.0, 5.4, 5.5, 7.4.
+// CTAs per replica when the caller leaves the choice open: four or eight where the replicas are
+// few enough for all clusters to run at once (a second wave would double the time), two while
+// they leave no SM without a replica of its own, and one for chains whose CTAs would have next to
+// no work. Us per step of one replica with 1, 2, 4, 8 CTAs: 64 atoms 3.8, 4.3, 4.1, 4.5; 128
+// atoms 6.0, 5.2, 4.6, 5.0; 200 atoms 9.6, 7.8, 6.8, 5.9; 304 atoms 14.0, 10.5, 8.1, 7.7; 560
+// atoms 30.4, 18.7, 12.3, 10.5; 1200 atoms 75.7, 43.9, 27.2, 18.6.
 int auto_cluster(int R, int nta, int n_sm, int threads) {
-    if (threads > kMaxThreadsPair || 2 * R > n_sm) return 1;
+    if (threads > kMaxThreadsPair || 2 * R > n_sm || nta < 112) return 1;
     const int th = threads ? threads : kMaxThreadsPair;
-    if (nta >= 512 && 8 * R <= n_sm && R <= chain_max_clusters(8, nta, th)) return 8;
-    if (nta >= 192 && 4 * R <= n_sm && R <= chain_max_clusters(4, nta, th)) return 4;
+    if (nta >= 192 && 8 * R <= n_sm && R <= chain_max_clusters(8, nta, th)) return 8;
+    if (4 * R <= n_sm && R <= chain_max_clusters(4, nta, th)) return 4;
     return 2;
 }
 

@@ -70,7 +70,7 @@ def test_frame_batches_of_every_cluster_size_agree(torch_cuda, n):
     s.close()
 
 
-@pytest.mark.parametrize("n", [447, 449, 560])
+@pytest.mark.parametrize("n", [96, 129, 193, 449, 560])
 def test_resident_clusters_agree(torch_cuda, n):
     c = cut(synth.make_chain(35, seed=1), n)
     runs = []
