@@ -394,7 +394,7 @@ def extra_config(torch, pkg, name, args, K, W):
         out = {"metric": "particle-steps/s", "value": 256 * toy.n_steps * K / durs.sum(),
                "unit": "particle-steps/s", "ms_per_step": durs.mean() * 1e3, "steps": K,
                "warmup": W, "config": {"workload": "256 replicas x 1e4 overdamped steps, FP64"},
-               "roofline": None, "note": "one thread per replica: launch and latency bound, no "
+               "roofline": None, "note": "a serial FP64 chain per replica: latency bound, no "
                                          "meaningful roofline",
                "gpu_launches": K, "clocks": clk}
         s.close()
@@ -480,8 +480,8 @@ def extra_config(torch, pkg, name, args, K, W):
         out = {"metric": "frames/s (forward + backward + double backward)", "value": T * K / durs.sum(),
                "unit": "frames/s", "ms_per_step": durs.mean() * 1e3, "steps": K, "warmup": W,
                "config": {"workload": "sum_t |grad U(X_t)|^2 over 1000 frames x 560 atoms, "
-                                      "checkpointing every 50 frames (the backward of a segment "
-                                      "recomputes its forces and applies H(X_t) 2 grad U(X_t))"},
+                                      "no forces kept (the backward recomputes them and applies "
+                                      "H(X_t) 2 grad U(X_t))"},
                "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                             "frac": ach / peak, "traffic": None, "in_cutoff_pairs": p_in},
                "clocks": clk}

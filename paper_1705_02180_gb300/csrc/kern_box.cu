@@ -251,11 +251,53 @@ __global__ void k_box_keyorder(BoxDev B, int r0) {
     B.id[off + lo + rank] = a;
 }
 
-// Rebuild step 2 (one warp per tile, once its slots are written): boxes of the tile and of each
-// 8-slot cluster, and whether the cluster holds chain atoms or only atoms with the LJ parameters
-// of the last atom (a solvent site), whose pair constants the pair kernel then computes once.
-__device__ __forceinline__ void box_tile_bounds(const BoxDev& B, const TopoDev* __restrict__ topo,
-                                                int r, int t, int lane) {
+// Rebuild, step 1f (one warp per tile): inside each tile, two halves of 16 by x,
+// each ordered by y (padding last), so that slots 8q .. 8q+7 form compact
+// clusters; final slot arrays, reference positions, LJ parameters, slot_of.
+__global__ void k_box_subsort(BoxDev B, const TopoDev* __restrict__ topo, int r0) {
+    const int r = blockIdx.y + r0;
+    if (!B.need[r]) return;
+    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (t >= B.nt) return;
+    const int lane = threadIdx.x & 31;
+    const size_t base = (size_t)r * B.np;
+    const int s0 = t * 32 + lane;
+    const int a = B.id[base + s0];  // (the other lanes read theirs before any write below)
+    const bool valid = a >= 0;
+    const float4 p = B.pos2[base + max(a, 0)];
+    const float4 v = B.vel2[base + max(a, 0)];
+    const float kx = valid ? p.x : 3.0e38f, ky = valid ? p.y : 3.0e38f;
+    const int rx = warp_rank(kx, lane, true, kFullB);
+    const unsigned upper = __ballot_sync(kFullB, rx >= 16);
+    const bool hi = rx >= 16;
+    const int ry = warp_rank(ky, lane, true, hi ? upper : ~upper);
+    const int s = t * 32 + (hi ? 16 : 0) + ry;
+    if (valid) {
+        B.pos[base + s] = p;
+        B.vel[base + s] = v;
+        B.id[base + s] = a;
+        B.pos_ref[base + s] = p;
+        B.par[base + s] = topo->lj[a];
+        B.slot_of[(size_t)r * B.n_atoms + a] = s;
+    } else {
+        const float4 far = make_float4(1.0e5f * (float)(s + 1), 0.f, 0.f, 0.f);
+        B.pos[base + s] = far;
+        B.vel[base + s] = make_float4(0.f, 0.f, 0.f, 0.f);
+        B.id[base + s] = -1;
+        B.pos_ref[base + s] = far;
+        B.par[base + s] = make_float2(0.f, 0.f);
+    }
+}
+
+// Rebuild step 2 (one warp per tile): boxes of the tile and of each 8-slot cluster, and whether
+// the cluster holds chain atoms or only atoms with the LJ parameters of the last atom (a solvent
+// site), whose pair constants the pair kernel then computes once.
+__global__ void k_box_tiles(BoxDev B, const TopoDev* __restrict__ topo, int r0) {
+    const int r = blockIdx.y + r0;
+    if (!B.need[r]) return;
+    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (t >= B.nt) return;
+    const int lane = threadIdx.x & 31;
     const int s = t * 32 + lane;
     const float4 p = B.pos[(size_t)r * B.np + s];
     const int a = B.id[(size_t)r * B.np + s];
@@ -296,46 +338,6 @@ __device__ __forceinline__ void box_tile_bounds(const BoxDev& B, const TopoDev* 
         B.tlo[(size_t)r * B.nt + t] = make_float4(lx, ly, lz, 0.f);
         B.thi[(size_t)r * B.nt + t] = make_float4(hx, hy, hz, 0.f);
     }
-}
-
-// Rebuild, step 1f (one warp per tile): inside each tile, two halves of 16 by x,
-// each ordered by y (padding last), so that slots 8q .. 8q+7 form compact
-// clusters; final slot arrays, reference positions, LJ parameters, slot_of.
-__global__ void k_box_subsort(BoxDev B, const TopoDev* __restrict__ topo, int r0) {
-    const int r = blockIdx.y + r0;
-    if (!B.need[r]) return;
-    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= B.nt) return;
-    const int lane = threadIdx.x & 31;
-    const size_t base = (size_t)r * B.np;
-    const int s0 = t * 32 + lane;
-    const int a = B.id[base + s0];  // (the other lanes read theirs before any write below)
-    const bool valid = a >= 0;
-    const float4 p = B.pos2[base + max(a, 0)];
-    const float4 v = B.vel2[base + max(a, 0)];
-    const float kx = valid ? p.x : 3.0e38f, ky = valid ? p.y : 3.0e38f;
-    const int rx = warp_rank(kx, lane, true, kFullB);
-    const unsigned upper = __ballot_sync(kFullB, rx >= 16);
-    const bool hi = rx >= 16;
-    const int ry = warp_rank(ky, lane, true, hi ? upper : ~upper);
-    const int s = t * 32 + (hi ? 16 : 0) + ry;
-    if (valid) {
-        B.pos[base + s] = p;
-        B.vel[base + s] = v;
-        B.id[base + s] = a;
-        B.pos_ref[base + s] = p;
-        B.par[base + s] = topo->lj[a];
-        B.slot_of[(size_t)r * B.n_atoms + a] = s;
-    } else {
-        const float4 far = make_float4(1.0e5f * (float)(s + 1), 0.f, 0.f, 0.f);
-        B.pos[base + s] = far;
-        B.vel[base + s] = make_float4(0.f, 0.f, 0.f, 0.f);
-        B.id[base + s] = -1;
-        B.pos_ref[base + s] = far;
-        B.par[base + s] = make_float2(0.f, 0.f);
-    }
-    __syncwarp();
-    box_tile_bounds(B, topo, r, t, lane);
 }
 
 // Rebuild step 3 (one warp per 8-slot i cluster c): the pair list of c. Its own 8 slots
@@ -1210,6 +1212,7 @@ static void box_rebuild(const BoxDev& B, const TopoDev* topo, const StateDev& st
     k_box_keyorder<<<dim3((B.np + 255) / 256, nr), 256, 0, s>>>(B, r0);
     const dim3 gt((B.nt + 3) / 4, nr);       // one warp per tile
     k_box_subsort<<<gt, 128, 0, s>>>(B, topo, r0);
+    k_box_tiles<<<gt, 128, 0, s>>>(B, topo, r0);
     k_box_list<<<dim3(B.nt, nr), 128, 0, s>>>(B, st, r0);
 }
 
