@@ -1,6 +1,5 @@
 // C ABI of the rMD engine (include/scps.h): validation, device tables, state,
-// launch plans and CUDA graphs. All compute runs in the kernels of
-// kern_chain.cu and kern_aux.cu.
+// launch plans and CUDA graphs. All compute runs in the kernels of the kern_*.cu files.
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -362,8 +361,11 @@ int auto_cluster(int R, int nta, int n_sm, int threads) {
 // CTAs per frame of a frame evaluation: two while they fit the SMs, four and eight only well
 // below that, since a cluster needs its SMs in one GPC (3 frames of 1199 atoms: 67, 51 and 47
 // us with two, four and eight; 9 frames of 560: 39, 35, 33; 20 of 304: 29, 26, 30; 50 of 560:
-// 42, 48, 76).
-int eval_cluster(long long nf, int n_sm) {
+// 42, 48, 76). Small chains take one: a cluster launch costs 2 us, and they gain nothing (28 frames
+// of 44 atoms 18.6, 20.6, 20.6 us with one, two and four, of 128 22.3, 22.6, 22.9, of 200 25.7,
+// 24.6, 23.1).
+int eval_cluster(long long nf, int nta, int n_sm) {
+    if (nta < kEvalClusterAtoms) return 1;
     if (10 * nf <= n_sm) return 8;
     if (5 * nf <= n_sm) return 4;
     return 2 * nf <= n_sm ? 2 : 1;
@@ -1197,7 +1199,7 @@ int scps_energy_forces(scps_system* s, int32_t topo, int64_t n_frames, const flo
     const int n3 = 3 * th.n;
     for (long long f0 = 0; f0 < n_frames; f0 += per_launch) {
         const long long nf = std::min(per_launch, n_frames - f0);
-        const int cl = eval_cluster(nf, n_sm);
+        const int cl = eval_cluster(nf, nta, n_sm);
         const int threads = nf * cl <= n_sm ? 1024 : eval_threads(nta);
         SCPS_CU(launch_eval(s->d.elec, s->d_topos + topo, P, X + f0 * n3, U + f0,
                             F ? F + f0 * n3 : nullptr, z ? z + f0 : nullptr, nf, nta, threads, cl,

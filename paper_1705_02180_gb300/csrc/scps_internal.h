@@ -57,6 +57,7 @@ constexpr int kMaxTubeK = 128;  // reference slices of the contact-map tube bias
 constexpr int kTubeItem = 8;    // contacts per work item of the tube passes (and of the
                                 // blocks in which the reference maps are stored)
 constexpr int kMaxThreadsPair = 768;  // threads per CTA of a cluster (80 registers each)
+constexpr int kEvalClusterAtoms = 160;  // smallest chains whose frames take clusters of CTAs
 
 // Per-replica addressing.
 struct RepDev {

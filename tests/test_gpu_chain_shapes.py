@@ -52,7 +52,7 @@ def evaluate(torch, s, X):
     return U.cpu().numpy(), F.cpu().numpy(), Z.cpu().numpy()
 
 
-@pytest.mark.parametrize("n", [17, 64, 129, 449, 560])
+@pytest.mark.parametrize("n", [17, 129, 160, 161, 449, 560])
 def test_frame_batches_of_every_cluster_size_agree(torch_cuda, n):
     torch = torch_cuda
     c = cut(synth.make_chain(35, seed=1), n)
@@ -104,7 +104,7 @@ def test_large_forces_match_the_oracle(torch_cuda, scale):
     s.close()
 
 
-@pytest.mark.parametrize("n", [9, 64, 257, 559])
+@pytest.mark.parametrize("n", [9, 64, 161, 257, 559])
 def test_hvp_of_every_cluster_size_agrees(torch_cuda, n):
     # 1e-5 of the rms, as for the other Hessian-vector products
     torch = torch_cuda
