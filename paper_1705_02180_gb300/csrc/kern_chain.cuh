@@ -1266,8 +1266,9 @@ __device__ __forceinline__ float4 far_slot(int i) {
 // WIDE: at most kMaxThreadsPair threads per CTA, which leaves 80 registers per thread (every
 // cluster of several CTAs, and a lone CTA that has an SM to itself: 1200 atoms 78.5 us per step
 // against 84.0 with 1024 threads of 64 registers, 304 atoms 14.3 against 15.4). Otherwise up to
-// 1024 threads of 64 registers, so that two 512-thread CTAs can share an SM (304 replicas of
-// 560 atoms: 68 us per step, against 73 with 80 registers, which leave one CTA per SM).
+// 1024 threads of 64 registers: for small chains, several of which share an SM, and for callers who
+// ask for 1024 threads or for two 512-thread CTAs per SM (304 replicas of 560 atoms: 68 us per
+// step, 73 with 80 registers, which leave one CTA per SM).
 template <int ELEC, int CL, bool TUBE, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? kMaxThreadsPair : 1024, 1)
 k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, StateDev st,
