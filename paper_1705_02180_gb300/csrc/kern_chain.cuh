@@ -117,7 +117,10 @@ struct Scalars {
     TopoDev tp;         // the replica's topology and list slab (shared memory: read where
     ListDev list;       // needed instead of held in registers)
     int work_next[2];   // this CTA's work counter, by parity of the evaluated step
-    int status;         // replica status (identical in every CTA of a cluster)
+    int status;         // replica status (identical in every CTA of a cluster): written by this
+                        // CTA's warp 0 alone, before the barrier that ends a decision
+    int nonfinite[2];   // NONFINITE bit of the update, by parity: raised by any CTA of the cluster
+                        // before the barrier that closes the update, read only after it
     int bias_on;
     int flag[2];        // force-range bits raised during the evaluation of a given parity
     int n_items;        // pair items in this CTA's item table
@@ -1316,6 +1319,8 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         sc.work_next2[1] = 0;
         sc.vmax2[0] = 0u;
         sc.vmax2[1] = 0u;
+        sc.nonfinite[0] = 0;
+        sc.nonfinite[1] = 0;
         for (int q = 0; q < 6; ++q) (&sc.zw[0][0])[q] = 0u;
         sc.sm = st.sm[r];
         sc.wm = st.wm[r];
@@ -1433,7 +1438,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         vm2 = fmaxf(vm2, v1 + fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)));
                         if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
                               isfinite(v.y) && isfinite(v.z)))
-                            for (int q = 0; q < CL; ++q) atomicOr(rank_ptr<CL>(&sc.status, q), SCPS_FLAG_NONFINITE);
+                            for (int q = 0; q < CL; ++q) atomicOr(rank_ptr<CL>(&sc.nonfinite[b], q), SCPS_FLAG_NONFINITE);
 #pragma unroll
                         for (int q = 0; q < CL; ++q) rank_ptr<CL>(sm.xq(), q)[i] = x;
                     }
@@ -1447,6 +1452,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             if (tid == 0) {
                 sc.flag[nb] = 0;
                 sc.vmax2[nb] = 0u;
+                sc.nonfinite[nb] = 0;  // (last read after the barrier of the step before)
                 sc.zw[nb][0] = sc.zw[nb][1] = sc.zw[nb][2] = 0u;
             }
             cluster_barrier<CL>();  // every CTA has the new positions
@@ -1468,10 +1474,14 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                     sc.n_saved += 1;
                 }
             }
-            // leave after the last B, or when the new state is non-finite (identical in
-            // every CTA of the cluster: same inputs, same arithmetic)
+            // leave after the last B, when a force was out of range, or when the new state is
+            // non-finite. Every thread of the cluster must leave at the same place, so each word
+            // read here is one that no CTA can write before all have read it: the force-range bit
+            // belongs to a decision and the other word to an update, with a cluster barrier
+            // between either and its next writer. (One word for both would let a CTA that is
+            // already in the next update stop one that still has to take it.)
             if (save) slot = slot + 1 == P.max_frames ? 0 : slot + 1;
-            if (!do_a || sc.status != 0) break;
+            if (!do_a || sc.status != 0 || sc.nonfinite[b] != 0) break;
             ++step;
             if (save_phase >= 0) save_phase = save_phase + 1 == P.save_interval ? 0 : save_phase + 1;
             // |x_new - x_old| <= dt/2 (|v after B| + |v after O|) <= dt/2 sqrt(2 vmax2) per
@@ -1499,6 +1509,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         }
     }
     __syncthreads();
+    const int status = sc.status | sc.nonfinite[0] | sc.nonfinite[1];
     // write back the state: each CTA the atoms it integrated, rank 0 the scalars
     for (int i = kTile * own_lo(tp.n_tiles, rank, CL) + tid;
          i < min(n, kTile * own_lo(tp.n_tiles, rank + 1, CL)); i += blockDim.x) {
@@ -1514,10 +1525,10 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             st.sm[r] = sc.sm;
             st.wm[r] = sc.wm;
             st.T[r] = sc.T;
-            st.status[r] = sc.status;
+            st.status[r] = status;
             st.step[r] = step;
             st.n_saved[r] = sc.n_saved;
-            if (st.pair_slots && sc.status == 0 && P.n_steps > 0) st.pair_slots[r] = sc.pair_slots;
+            if (st.pair_slots && status == 0 && P.n_steps > 0) st.pair_slots[r] = sc.pair_slots;
             if (st.list_builds) st.list_builds[r] = builds;
         }
     }
