@@ -432,9 +432,11 @@ __global__ void __launch_bounds__(128) k_box_list(BoxDev B, StateDev st, int r0)
         for (int u = 0; u < 2; ++u) {
             float d = u ? d2.y : d2.x;
             if (in[u] && !(dm[u] < 0.5f * B.L)) {  // the shift may not be the minimum image
-                const float bx = fmaxf(0.f, fabsf(px[u] - cx) - hx),
-                            by = fmaxf(0.f, fabsf(py[u] - cy) - hy),
-                            bz = fmaxf(0.f, fabsf(pz[u] - cz) - hz);
+                // box distance of the atom's own nearest image (in a small box not the
+                // cluster's), which bounds that of every image
+                const float bx = fmaxf(0.f, fabsf(min_img(x[u].x - cx, B.L, B.invL)) - hx),
+                            by = fmaxf(0.f, fabsf(min_img(x[u].y - cy, B.L, B.invL)) - hy),
+                            bz = fmaxf(0.f, fabsf(min_img(x[u].z - cz, B.L, B.invL)) - hz);
                 d = 3.0e38f;
                 if (fmaf(bx, bx, fmaf(by, by, bz * bz)) < B.rlist2)
                     for (int t = 0; t < 8; ++t) {
