@@ -606,7 +606,7 @@ struct BoxCluster {
 };
 
 // Adds an integer vector (2^-13 units) to the force sums of slot s (acc: the replica's three
-// modular, then three coarse arrays of np words); the coarse words only when a component rounds
+// modular, three coarse and three upper arrays of np words); the coarse words only when a component rounds
 // to a non-zero multiple of 2^kBoxShift. (Six words per slot side by side, which need fewer
 // address computations, touch more sectors per atomic: 409 against 388 us.)
 __device__ __forceinline__ void box_red3(const BoxDev& B, unsigned* acc, int s, int vx, int vy, int vz) {
@@ -626,12 +626,21 @@ __device__ __forceinline__ void box_red3(const BoxDev& B, unsigned* acc, int s, 
     }
 }
 
-// The same for one 64-bit component (d = 0, 1, 2).
+// The same for one 64-bit component (d = 0, 1, 2). WIDE: of its coarse count only the low kBoxUpper
+// bits (signed) go to the coarse word; the rest, which takes a term beyond 1.3e8 kJ mol^-1 nm^-1
+// (colliding sites), goes to the upper word, so that the three together hold what a 64-bit sum would.
+template <bool WIDE>
 __device__ __forceinline__ void box_red64(const BoxDev& B, unsigned* acc, int s, int d, long long v) {
-    unsigned* L = acc + s + d * (size_t)B.np;
+    const size_t np = (size_t)B.np;
+    unsigned* L = acc + s + d * np;
     atomicAdd(L, (unsigned)v);
-    const int h = (int)(((v >> (kBoxShift - 1)) + 1) >> 1);
-    if (h) atomicAdd((int*)L + 3 * (size_t)B.np, h);
+    const long long h = ((v >> (kBoxShift - 1)) + 1) >> 1;
+    const int lo = WIDE ? (int)((unsigned)h << (32 - kBoxUpper)) >> (32 - kBoxUpper) : (int)h;
+    if (lo) atomicAdd((int*)L + 3 * np, lo);
+    if (WIDE && lo != h) {
+        atomicAdd(L + 6 * np, (unsigned)((h - lo) >> kBoxUpper));
+        *B.big = 1;
+    }
 }
 
 // The pairs of two list entries per lane with the 8 atoms of the i cluster: at iteration t
@@ -753,12 +762,12 @@ __device__ __noinline__ long long box_chunk_slow(const BoxDev& B, const PairCons
         const float s13 = s * kPairScale;
         const long long tx = __float2ll_rn(s13 * dx), ty = __float2ll_rn(s13 * dy),
                         tz = __float2ll_rn(s13 * dz);
-        box_red64(B, acc, si0 + ii, 0, tx);
-        box_red64(B, acc, si0 + ii, 1, ty);
-        box_red64(B, acc, si0 + ii, 2, tz);
-        box_red64(B, acc, sj, 0, -tx);
-        box_red64(B, acc, sj, 1, -ty);
-        box_red64(B, acc, sj, 2, -tz);
+        box_red64<true>(B, acc, si0 + ii, 0, tx);
+        box_red64<true>(B, acc, si0 + ii, 1, ty);
+        box_red64<true>(B, acc, si0 + ii, 2, tz);
+        box_red64<true>(B, acc, sj, 0, -tx);
+        box_red64<true>(B, acc, sj, 1, -ty);
+        box_red64<true>(B, acc, sj, 2, -tz);
         if (ENERGY) e18 += __float2ll_rn(ep * kPairEScale);
     }
     return e18;
@@ -777,7 +786,7 @@ __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDe
     const size_t cl = (size_t)r * 4 * B.nt + c;
     const uint32_t* lst = B.ent + cl * B.max_ent;
     const int n = B.nent[cl];
-    unsigned* acc = B.facc + 6 * base;
+    unsigned* acc = B.facc + 9 * base;
     const float2 ref = tp.lj[B.n_atoms - 1];
     const LJPair u1 = lj_pair(ref.x + ref.x, ref.y * ref.y, P.pc);
     const LJPair2 U = {dup2(u1.sig2), dup2(u1.eps24 * kPairScale), dup2(u1.c6), dup2(u1.a_ljc * kPairScale)};
@@ -879,9 +888,9 @@ __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDe
         ai[d] += __shfl_xor_sync(kFullB, ai[d], 8);
         ai[d] += __shfl_xor_sync(kFullB, ai[d], 16);
     }
-    if (lane < 8 && ci.id[lane] >= 0) {
+    if (lane < 8 && ci.id[lane] >= 0) {  // (sums of up to 2^8 chunks, each below 2^31)
 #pragma unroll
-        for (int d = 0; d < 3; ++d) box_red64(B, acc, 8 * c + lane, d, -ai[d]);
+        for (int d = 0; d < 3; ++d) box_red64<false>(B, acc, 8 * c + lane, d, -ai[d]);
     }
     if (ENERGY) {
 #pragma unroll
@@ -922,14 +931,21 @@ __global__ void __launch_bounds__(32 * kPairWarps, kPairRegWarps / kPairWarps) k
 // next evaluation.
 __device__ __forceinline__ float4 take_nb_force(const BoxDev& B, int r, int s) {
     const size_t np = (size_t)B.np;
-    unsigned* L = B.facc + 6 * (size_t)r * np + s;
+    unsigned* L = B.facc + 9 * (size_t)r * np + s;
     unsigned w[6];
+    const int big = *B.big;
 #pragma unroll
     for (int d = 0; d < 6; ++d) w[d] = L[d * np];
     float f[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d)  // 2^-13 to 2^-20 units
         f[d] = fix2f(join_coarse((int)w[3 + d], w[d], kBoxShift) * 128);
+    if (big)  // some upper word has been added to
+        for (int d = 0; d < 3; ++d) {
+            const long long up = (long long)L[(6 + d) * np] << kBoxUpper;
+            f[d] = fix2f(join_coarse((int)w[3 + d] + up, w[d], kBoxShift) * 128);
+            L[(6 + d) * np] = 0u;
+        }
 #pragma unroll
     for (int d = 0; d < 6; ++d) L[d * np] = 0u;
     return make_float4(f[0], f[1], f[2], 0.f);

@@ -757,9 +757,10 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
         BALLOC(B.par, np);
         BALLOC(B.id, np);
         BALLOC(B.id2, np);
-        BALLOC(B.facc, 6 * np);
+        BALLOC(B.facc, 9 * np);
+        BALLOC(B.big, 1);
         BALLOC(B.epair, Rs);
-        if (cudaMemset(B.facc, 0, sizeof(unsigned) * 6 * np) != cudaSuccess ||
+        if (cudaMemset(B.facc, 0, sizeof(unsigned) * 9 * np) != cudaSuccess ||
             cudaMemset(B.epair, 0, sizeof(long long) * Rs) != cudaSuccess)
             return bail(fail(SCPS_ERR_CUDA, "cudaMemset failed"));
         BALLOC(B.pos2, np);

@@ -165,9 +165,11 @@ struct BoxDev {
     float2* par;      // (sigma/2, sqrt(24 eps))
     int* id;          // atom id of each slot, -1 for padding
     int* id2;         // sort buffer of id
-    unsigned* facc;   // [replica][6][np] non-bonded force on the slot: three sums modulo 2^32 of
-                      // 2^-13 units, then three coarse sums (int) in units of 2^kBoxShift
-                      // (order-free; cleared by whoever consumes them)
+    unsigned* facc;   // [replica][9][np] non-bonded force on the slot: three sums modulo 2^32 of
+                      // 2^-13 units, three coarse sums (int) in units of 2^kBoxShift and three
+                      // upper ones in units of 2^(kBoxShift + kBoxUpper) (order-free; cleared by
+                      // whoever consumes them)
+    int* big;         // [1] set once an upper word has been added to (they are read from then on)
     long long* epair; // [replica] pair energy of energy evaluations, fixed point 2^-18
                       // (cleared by whoever consumes it)
     float4* pos2;     // sort buffers
@@ -201,6 +203,7 @@ struct BoxDev {
 };
 
 constexpr int kBoxShift = 21;  // a slot takes at most 2047 chunk sums (join_coarse stays exact)
+constexpr int kBoxUpper = 20;  // bits of a 64-bit term's coarse count that the coarse word takes
 constexpr uint32_t kBoxNoSlot = 0x7fffffu;  // padding entry of a box pair list
 
 // Step graphs of the periodic box (variants: regular, last step of a call, save step, save
