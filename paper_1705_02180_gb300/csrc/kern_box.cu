@@ -24,6 +24,8 @@
 // batch rebuild together. Forces are integer sums of per-pair terms (order-free);
 // positions are wrapped into the box at each rebuild, so runs that rebuild at
 // other steps agree to rounding.
+#include <type_traits>
+
 #include "scps_internal.h"
 
 namespace scps {
@@ -148,9 +150,10 @@ __global__ void k_box_key(BoxDev B, int r0) {
 
 // Rebuild, step 1c (one CTA of 1024 threads per replica): exclusive scan of the
 // key counts (they become running cursors); first compact position and first
-// tile of every column (each column starts a tile).
+// tile of every column (each column starts a tile); the coarse unit of the force sums.
 __global__ void __launch_bounds__(kSortThreads) k_box_scan(BoxDev B, int r0) {
     __shared__ int wtot[32];
+    __shared__ int tiles[kMaxCols], most;
     const int r = blockIdx.x + r0;
     if (!B.need[r]) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -193,14 +196,53 @@ __global__ void __launch_bounds__(kSortThreads) k_box_scan(BoxDev B, int r0) {
     const int ncols = B.ncol * B.ncol;
     for (int c = tid; c <= ncols; c += blockDim.x) col_first[c] = c < ncols ? hist[c * B.nz] : B.n_atoms;
     __syncthreads();
-    if (tid == 0) {
-        int t = 0;
-        for (int c = 0; c < ncols; ++c) {
-            col_tile[c] = t;
-            t += (col_first[c + 1] - col_first[c] + 31) >> 5;
+    if (warp == 0) {  // prefix sums of the columns' tiles, kMaxCols / 32 columns per lane
+        constexpr int kCols = kMaxCols / 32;
+        int nt[kCols], sum = 0;
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) {
+            const int c = kCols * lane + q;
+            nt[q] = c < ncols ? (col_first[c + 1] - col_first[c] + 31) >> 5 : 0;
+            sum += nt[q];
         }
-        col_tile[ncols] = t;  // <= nt by the capacity ceil(n/32) + ncol^2
+        int x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFullB, x, o);
+            if (lane >= o) x += y;
+        }
+        int t = x - sum;
+#pragma unroll
+        for (int q = 0; q < kCols; ++q) {
+            const int c = kCols * lane + q;
+            if (c <= ncols) col_tile[c] = t;  // (the end: <= nt by the capacity ceil(n/32) + ncol^2)
+            t += nt[q];
+        }
+        if (lane == 31 && ncols == kMaxCols) col_tile[ncols] = t;
+        if (lane == 0) most = 0;
     }
+    __syncthreads();
+    // A slot takes one sum from every list it is in and one for its own cluster's share. Only
+    // clusters of the columns in reach can list it (k_box_list), so four times the most tiles in
+    // reach of a column bounds the lists; the coarse unit is chosen for that many terms.
+    const int reach = (int)ceilf(sqrtf(B.rlist2) / (B.L / (float)B.ncol));
+    const int span = min(2 * reach + 1, B.ncol);  // columns in reach, per axis
+    for (int c = tid; c < ncols; c += blockDim.x) {
+        int sum = 0;
+        for (int d = 0; d < span; ++d) {
+            const int q = c / B.ncol * B.ncol + (c % B.ncol + d) % B.ncol;
+            sum += col_tile[q + 1] - col_tile[q];
+        }
+        tiles[c] = sum;  // of `span` columns from c on in y
+    }
+    __syncthreads();
+    for (int c = tid; c < ncols; c += blockDim.x) {
+        int sum = 0;
+        for (int d = 0; d < span; ++d) sum += tiles[(c / B.ncol + d) % B.ncol * B.ncol + c % B.ncol];
+        atomicMax(&most, sum);  // (of the span x span columns from c on: every centre comes up once)
+    }
+    __syncthreads();
+    if (tid == 0) B.shift[r] = coarse_shift(4ll * most + 1, kBoxShift);
 }
 
 // Rebuild, step 1d (atoms): the atom ids go into the padded column layout, positions and
@@ -603,42 +645,43 @@ struct BoxCluster {
     float2 lj[8];
     int id[8];
     unsigned long long ex[8];  // exclusion masks of its chain atoms
+    unsigned redo[kBoxMaxEnt / 512];  // quarters of chunks to redo pair by pair, 8 chunks per word
 };
 
 // Adds an integer vector (2^-13 units) to the force sums of slot s (acc: the replica's three
-// modular, three coarse and three upper arrays of np words); the coarse words only when a component rounds
-// to a non-zero multiple of 2^kBoxShift. (Six words per slot side by side, which need fewer
+// modular, three coarse and three upper arrays of np words); the coarse words only when a component
+// rounds to a non-zero multiple of 2^sh. (Six words per slot side by side, which need fewer
 // address computations, touch more sectors per atomic: 409 against 388 us.)
-__device__ __forceinline__ void box_red3(const BoxDev& B, unsigned* acc, int s, int vx, int vy, int vz) {
+__device__ __forceinline__ void box_red3(const BoxDev& B, unsigned* acc, int sh, int s, int vx, int vy, int vz) {
     unsigned* L = acc + s;
     const size_t np = (size_t)B.np;
     atomicAdd(L, (unsigned)vx);
     atomicAdd(L + np, (unsigned)vy);
     atomicAdd(L + 2 * np, (unsigned)vz);
-    const unsigned half = 1u << (kBoxShift - 1);
-    if ((((unsigned)vx + half) | ((unsigned)vy + half) | ((unsigned)vz + half)) >> kBoxShift) {
+    const unsigned half = 1u << (sh - 1);
+    if ((((unsigned)vx + half) | ((unsigned)vy + half) | ((unsigned)vz + half)) >> sh) {
         int* H = (int*)L + 3 * np;
-        const int hx = ((vx >> (kBoxShift - 1)) + 1) >> 1, hy = ((vy >> (kBoxShift - 1)) + 1) >> 1,
-                  hz = ((vz >> (kBoxShift - 1)) + 1) >> 1;
+        const int hx = ((vx >> (sh - 1)) + 1) >> 1, hy = ((vy >> (sh - 1)) + 1) >> 1,
+                  hz = ((vz >> (sh - 1)) + 1) >> 1;
         if (hx) atomicAdd(H, hx);
         if (hy) atomicAdd(H + np, hy);
         if (hz) atomicAdd(H + 2 * np, hz);
     }
 }
 
-// The same for one 64-bit component (d = 0, 1, 2). WIDE: of its coarse count only the low kBoxUpper
-// bits (signed) go to the coarse word; the rest, which takes a term beyond 1.3e8 kJ mol^-1 nm^-1
-// (colliding sites), goes to the upper word, so that the three together hold what a 64-bit sum would.
-template <bool WIDE>
-__device__ __forceinline__ void box_red64(const BoxDev& B, unsigned* acc, int s, int d, long long v) {
+// The same for one 64-bit component (d = 0, 1, 2). Of its coarse count only the low sh bits (signed)
+// go to the coarse word, so that as many terms as the coarse unit is chosen for keep it within 31
+// bits; the rest, which takes a term beyond 2.7e8 kJ mol^-1 nm^-1 at the usual unit (colliding
+// sites), goes to the upper word. The three together hold what a 64-bit sum would.
+__device__ __forceinline__ void box_red64(const BoxDev& B, unsigned* acc, int sh, int s, int d, long long v) {
     const size_t np = (size_t)B.np;
     unsigned* L = acc + s + d * np;
     atomicAdd(L, (unsigned)v);
-    const long long h = ((v >> (kBoxShift - 1)) + 1) >> 1;
-    const int lo = WIDE ? (int)((unsigned)h << (32 - kBoxUpper)) >> (32 - kBoxUpper) : (int)h;
+    const long long h = ((v >> (sh - 1)) + 1) >> 1;
+    const int lo = (int)((unsigned)h << (32 - sh)) >> (32 - sh);
     if (lo) atomicAdd((int*)L + 3 * np, lo);
-    if (WIDE && lo != h) {
-        atomicAdd(L + 6 * np, (unsigned)((h - lo) >> kBoxUpper));
+    if (lo != h) {
+        atomicAdd(L + 6 * np, (unsigned)((h - lo) >> sh));
         *B.big = 1;
     }
 }
@@ -651,9 +694,9 @@ __device__ __forceinline__ void box_red64(const BoxDev& B, unsigned* acc, int s,
 // 32-bit registers. MASKED: bit a of the low (first entry) or second byte of xm leaves out the
 // pair with cluster atom a (the cluster's own slots, whose pairs count once, excluded pairs,
 // and with the per-pair minimum image, MINIMG, empty slots). FAST: every atom has the reference
-// LJ parameters, whose pair constants U are computed once. Returns false for the quarters where
-// some |s| exceeds pc.s_lim / 2 (their 32-bit sums of 16 terms could overflow; the caller
-// redoes them pair by pair).
+// LJ parameters, whose pair constants U are computed once. Returns the lanes where some |s|
+// exceeds pc.s_lim / 2 (the 32-bit sums of 16 terms of their quarters could overflow; the caller
+// redoes those pair by pair at the end of the list).
 //
 // FAST takes 24 packed operations, two rsqrt and six roundings per two pairs; all roundings as
 // conversions would make the XU pipe (2.1 clocks an instruction) the bound, so z goes through
@@ -661,9 +704,9 @@ __device__ __forceinline__ void box_red64(const BoxDev& B, unsigned* acc, int s,
 // places wait for instructions (1.3 of 7 clocks between two of a warp; a step of 16 x 24 560
 // sites 515 -> 499 us, 504 unrolled by two).
 template <int ELEC, bool ENERGY, bool MASKED, bool MINIMG, bool FAST>
-__device__ __forceinline__ bool box_chunk(const BoxDev& B, const PairConst& pc, const LJPair2& U,
-                                          const BoxCluster& ci, const Entries& n, unsigned xm,
-                                          int lane, int* fi, int (*fj)[3], long long& e18) {
+__device__ __forceinline__ unsigned box_chunk(const BoxDev& B, const PairConst& pc, const LJPair2& U,
+                                              const BoxCluster& ci, const Entries& n, unsigned xm,
+                                              int lane, int* fi, int (*fj)[3], long long& e18) {
     const int l8 = lane & 7, q = lane >> 3;
     const float lim = 0.5f * kPairScale * pc.s_lim;
     int fx = 0, fy = 0, ax = 0, ay = 0, bx = 0, by = 0;
@@ -731,23 +774,27 @@ __device__ __forceinline__ bool box_chunk(const BoxDev& B, const PairConst& pc, 
     fj[1][0] = bx;
     fj[1][1] = by;
     fj[1][2] = (int)(bz - bias8);
-    const bool good = !((__ballot_sync(kFullB, bad) >> (8 * q)) & 0xffu);
-    if (ENERGY && good) e18 += ech;
-    return good;
+    const unsigned over = __ballot_sync(kFullB, bad);
+    if (ENERGY && !((over >> (8 * q)) & 0xffu)) e18 += ech;
+    return over;
 }
 
-// Slow path of the entries of a quarter that failed the fast path, one entry per lane: every
-// pair term, rounded to 2^-13 units as on the fast path, goes to both slots' sums in
-// 64-bit, so the forces are the same integers on either path.
+// Eight entries per quarter warp (mine: the quarter has some) that failed the fast path, one
+// per lane, pair by pair: every pair term, rounded to 2^-13 units as on the fast path, is summed
+// in 64 bits, so the forces are the same integers on either path. As there, the entry's slot gets
+// one sum and the cluster's atoms' sums move from lane to lane and come home (ai, with the
+// entries' sign). For whole warps, once the list has been gone through: inside that loop it costs
+// the loop registers (up to 39 us for 2 x 6400 sites, which take 34.4).
 template <int ELEC, bool ENERGY, bool MINIMG>
-__device__ __noinline__ long long box_chunk_slow(const BoxDev& B, const PairConst& pc,
-                                                 const BoxCluster& ci, float4 xj, float2 lj, int sj,
-                                                 int si0, unsigned xm, unsigned* acc) {
+__device__ __forceinline__ void box_chunk_slow(const BoxDev& B, const PairConst& pc, const BoxCluster& ci,
+                                               float4 xj, float2 lj, int sj, unsigned xm, bool mine,
+                                               unsigned* acc, int sh, long long* ai, long long& e18) {
     const int l8 = threadIdx.x & 7;
-    long long e18 = 0;
+    long long fi[3] = {}, fj[3] = {};
+#pragma unroll 1
     for (int t = 0; t < 8; ++t) {
-        const int ii = (l8 + t) & 7;
-        const float4 xi = ci.x[ii];
+        const int a = l8 ^ t;
+        const float4 xi = ci.x[a];
         float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
         if (MINIMG) {
             dx = min_img(dx, B.L, B.invL);
@@ -755,38 +802,50 @@ __device__ __noinline__ long long box_chunk_slow(const BoxDev& B, const PairCons
             dz = min_img(dz, B.L, B.invL);
         }
         const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        if (!(r2 < pc.rc2) || ((xm >> ii) & 1u)) continue;
-        float ep = 0.f;
-        const float2 li = ci.lj[ii];
-        const float s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &ep);
-        const float s13 = s * kPairScale;
-        const long long tx = __float2ll_rn(s13 * dx), ty = __float2ll_rn(s13 * dy),
-                        tz = __float2ll_rn(s13 * dz);
-        box_red64<true>(B, acc, si0 + ii, 0, tx);
-        box_red64<true>(B, acc, si0 + ii, 1, ty);
-        box_red64<true>(B, acc, si0 + ii, 2, tz);
-        box_red64<true>(B, acc, sj, 0, -tx);
-        box_red64<true>(B, acc, sj, 1, -ty);
-        box_red64<true>(B, acc, sj, 2, -tz);
-        if (ENERGY) e18 += __float2ll_rn(ep * kPairEScale);
+        if (mine && r2 < pc.rc2 && !((xm >> a) & 1u)) {
+            float ep = 0.f;
+            const float2 li = ci.lj[a];
+            const float s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &ep);
+            const float ms13 = -s * kPairScale;
+            const float f[3] = {ms13 * dx, ms13 * dy, ms13 * dz};
+            // (one pair of a quarter is beyond the fast path's limit, few are beyond 32 bits)
+            const bool small = fmaxf(fabsf(f[0]), fmaxf(fabsf(f[1]), fabsf(f[2]))) < 2.1e9f && s == s;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {  // (sums modulo 2^64)
+                const long long q = small ? (long long)__float2int_rn(f[k]) : __float2ll_rn(f[k]);
+                fi[k] = (long long)((unsigned long long)fi[k] + (unsigned long long)q);
+                fj[k] = (long long)((unsigned long long)fj[k] + (unsigned long long)q);
+            }
+            if (ENERGY) e18 += __float2ll_rn(ep * kPairEScale);
+        }
+        const int m = (t ^ (t + 1)) & 7;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) fi[k] = __shfl_xor_sync(kFullB, fi[k], m);
     }
-    return e18;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        ai[k] = (long long)((unsigned long long)ai[k] + (unsigned long long)fi[k]);
+        if (mine && sj != (int)kBoxNoSlot) box_red64(B, acc, sh, sj, k, fj[k]);
+    }
 }
 
 // Non-bonded forces of one 8-slot i cluster on one warp, each pair once (Newton's third
 // law): its list 64 entries at a time, two per lane. After a chunk each lane adds its entries'
 // sums to their slots and its share of a cluster atom's sums to 64-bit registers, which go to
-// the cluster's slots at the end. Entries
-// carry their periodic shift unless MINIMG; padding entries sit far away from everything.
-template <int ELEC, bool ENERGY, bool EXCL, bool MINIMG>
+// the cluster's slots at the end. Entries carry their periodic shift unless MINIMG; padding
+// entries sit far away from everything.
+// SHIFT: the coarse unit when the replica has the usual one (a constant in the loop: 33.7 us for
+// 2 x 6400 sites, and 34.6 with a variable), else 0.
+template <int ELEC, bool ENERGY, bool EXCL, bool MINIMG, int SHIFT>
 __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDev& tp,
                                                    const RunParams& P, int r, int c, int lane,
-                                                   bool ipure, const BoxCluster& ci) {
+                                                   bool ipure, BoxCluster& ci) {
     const size_t base = (size_t)r * B.np;
     const size_t cl = (size_t)r * 4 * B.nt + c;
     const uint32_t* lst = B.ent + cl * B.max_ent;
     const int n = B.nent[cl];
     unsigned* acc = B.facc + 9 * base;
+    const int sh = SHIFT ? SHIFT : B.shift[r];
     const float2 ref = tp.lj[B.n_atoms - 1];
     const LJPair u1 = lj_pair(ref.x + ref.x, ref.y * ref.y, P.pc);
     const LJPair2 U = {dup2(u1.sig2), dup2(u1.eps24 * kPairScale), dup2(u1.c6), dup2(u1.a_ljc * kPairScale)};
@@ -795,6 +854,7 @@ __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDe
     if (MINIMG) empty = __ballot_sync(kFullB, lane < 8 && ci.id[l8] < 0) & 0xffu;
     long long ai[3] = {};  // minus this lane's share of cluster atom l8
     long long e18 = 0;
+    bool redo = false;
     auto entry = [&](int k) -> uint32_t { return k < n ? __ldg(lst + k) : (kBoxNoSlot | (1u << 30)); };
     auto position = [&](uint32_t e) -> float4 {
         const int sj = (int)(e & kBoxNoSlot);
@@ -853,33 +913,48 @@ __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDe
         unsigned xm = 0u;
         if (EXCL || MINIMG || k0 == 0) xm = mask(e[0], k0 + lane) | (mask(e[1], k0 + 32 + lane) << 8);
         int fi[3], fj[2][3];
-        bool good;
+        unsigned over;
         if (EXCL || MINIMG || k0 == 0) {
             if (fast)
-                good = box_chunk<ELEC, ENERGY, true, MINIMG, true>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
+                over = box_chunk<ELEC, ENERGY, true, MINIMG, true>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
             else
-                good = box_chunk<ELEC, ENERGY, true, MINIMG, false>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
+                over = box_chunk<ELEC, ENERGY, true, MINIMG, false>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
         } else {
             if (fast)
-                good = box_chunk<ELEC, ENERGY, false, MINIMG, true>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
+                over = box_chunk<ELEC, ENERGY, false, MINIMG, true>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
             else
-                good = box_chunk<ELEC, ENERGY, false, MINIMG, false>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
+                over = box_chunk<ELEC, ENERGY, false, MINIMG, false>(B, P.pc, U, ci, en, xm, lane, fi, fj, e18);
+        }
+        const bool good = !((over >> (lane & 24)) & 0xffu);
+        if (over) {  // (uniform in the warp)
+            redo = true;
+            const unsigned bad = __ballot_sync(kFullB, !good && l8 == 0);  // bits 0, 8, 16, 24
+            if (lane == 0) ci.redo[k0 >> 9] |= ((bad * 0x01020408u) >> 24 & 0xfu) << (k0 >> 4 & 28);
         }
         if (good) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) ai[d] += fi[d];
-        }
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int sj = (int)(e[k] & kBoxNoSlot);
-            if (sj == (int)kBoxNoSlot) continue;
-            if (good) {
-                box_red3(B, acc, sj, fj[k][0], fj[k][1], fj[k][2]);
-            } else {  // (the slow path uses the general form)
-                e18 += box_chunk_slow<ELEC, ENERGY, MINIMG>(B, P.pc, ci, shifted(e[k], position(e[k])),
-                                                           entry_lj(e[k]), sj, 8 * c,
-                                                           (xm >> (8 * k)) & 0xffu, acc);
+            for (int k = 0; k < 2; ++k) {
+                const int sj = (int)(e[k] & kBoxNoSlot);
+                if (sj != (int)kBoxNoSlot) box_red3(B, acc, sh, sj, fj[k][0], fj[k][1], fj[k][2]);
             }
+        }
+    }
+    __syncwarp();
+    for (int w = 0; redo && w < (n + 511) >> 9; ++w) {
+        unsigned m = ci.redo[w];
+        while (m) {  // two failed quarters of 16 entries at a time, eight entries per quarter warp
+            const int q0 = __ffs(m) - 1;
+            m &= m - 1u;
+            const int q1 = m ? __ffs(m) - 1 : -1;
+            m &= m - 1u;
+            const int qq = lane < 16 ? q0 : q1;
+            const bool mine = qq >= 0;
+            const int k = mine ? 512 * w + 64 * (qq >> 2) + 8 * (qq & 3) + 32 * (lane >> 3 & 1) + l8 : n;
+            const uint32_t e = entry(k);
+            box_chunk_slow<ELEC, ENERGY, MINIMG>(B, P.pc, ci, shifted(e, position(e)), entry_lj(e),
+                                                 (int)(e & kBoxNoSlot), mask(e, k), mine, acc, sh, ai, e18);
         }
     }
     // the four quarters' shares of each cluster atom
@@ -888,9 +963,9 @@ __device__ __forceinline__ void box_cluster_forces(const BoxDev& B, const TopoDe
         ai[d] += __shfl_xor_sync(kFullB, ai[d], 8);
         ai[d] += __shfl_xor_sync(kFullB, ai[d], 16);
     }
-    if (lane < 8 && ci.id[lane] >= 0) {  // (sums of up to 2^8 chunks, each below 2^31)
+    if (lane < 8 && ci.id[lane] >= 0) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) box_red64<false>(B, acc, 8 * c + lane, d, -ai[d]);
+        for (int d = 0; d < 3; ++d) box_red64(B, acc, sh, 8 * c + lane, d, -ai[d]);
     }
     if (ENERGY) {
 #pragma unroll
@@ -917,14 +992,22 @@ __global__ void __launch_bounds__(32 * kPairWarps, kPairRegWarps / kPairWarps) k
         ci[w].id[lane] = a;
         ci[w].ex[lane] = (a >= 0 && a < B.n_chain) ? tp.excl[a] : 0ull;
     }
+    if (lane < kBoxMaxEnt / 512) ci[w].redo[lane] = 0u;
     __syncwarp();
     const int fl = B.cflag[(size_t)r * 4 * B.nt + c];
     const bool pure = (fl & 4) != 0;
-    switch (fl & 3) {
-        case 0: box_cluster_forces<ELEC, ENERGY, false, false>(B, tp, P, r, c, lane, pure, ci[w]); break;
-        case 1: box_cluster_forces<ELEC, ENERGY, true, false>(B, tp, P, r, c, lane, pure, ci[w]); break;
-        default: box_cluster_forces<ELEC, ENERGY, true, true>(B, tp, P, r, c, lane, pure, ci[w]); break;
-    }
+    auto forces = [&](auto shift) {
+        constexpr int S = decltype(shift)::value;
+        switch (fl & 3) {
+            case 0: box_cluster_forces<ELEC, ENERGY, false, false, S>(B, tp, P, r, c, lane, pure, ci[w]); break;
+            case 1: box_cluster_forces<ELEC, ENERGY, true, false, S>(B, tp, P, r, c, lane, pure, ci[w]); break;
+            default: box_cluster_forces<ELEC, ENERGY, true, true, S>(B, tp, P, r, c, lane, pure, ci[w]); break;
+        }
+    };
+    if (B.shift[r] == kBoxShift)
+        forces(std::integral_constant<int, kBoxShift>());
+    else
+        forces(std::integral_constant<int, 0>());
 }
 
 // Total non-bonded force on slot s of replica r (fixed point), which is cleared for the
@@ -933,17 +1016,17 @@ __device__ __forceinline__ float4 take_nb_force(const BoxDev& B, int r, int s) {
     const size_t np = (size_t)B.np;
     unsigned* L = B.facc + 9 * (size_t)r * np + s;
     unsigned w[6];
-    const int big = *B.big;
+    const int big = *B.big, sh = B.shift[r];
 #pragma unroll
     for (int d = 0; d < 6; ++d) w[d] = L[d * np];
     float f[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d)  // 2^-13 to 2^-20 units
-        f[d] = fix2f(join_coarse((int)w[3 + d], w[d], kBoxShift) * 128);
+        f[d] = fix2f(join_coarse((int)w[3 + d], w[d], sh) * 128);
     if (big)  // some upper word has been added to
         for (int d = 0; d < 3; ++d) {
-            const long long up = (long long)L[(6 + d) * np] << kBoxUpper;
-            f[d] = fix2f(join_coarse((int)w[3 + d] + up, w[d], kBoxShift) * 128);
+            const long long up = (long long)L[(6 + d) * np] << sh;
+            f[d] = fix2f(join_coarse((int)w[3 + d] + up, w[d], sh) * 128);
             L[(6 + d) * np] = 0u;
         }
 #pragma unroll

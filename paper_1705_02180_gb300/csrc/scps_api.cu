@@ -737,7 +737,7 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
             const double rho = t.n_atoms / (d->box * d->box * d->box);
             const double rr = d->cutoff + 0.75;
             const double full = rho * 4.18879020478639 * rr * rr * rr;
-            B.max_ent = std::min(1 << 14, 8 + 8 * (int)std::ceil(full / 8.0));
+            B.max_ent = std::min(kBoxMaxEnt, 8 + 8 * (int)std::ceil(full / 8.0));
         }
         B.rebuild_every = d->rebuild_every > 0 ? d->rebuild_every : 20;
         B.L = (float)d->box;
@@ -759,6 +759,7 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
         BALLOC(B.id2, np);
         BALLOC(B.facc, 9 * np);
         BALLOC(B.big, 1);
+        BALLOC(B.shift, Rs);  // (set by every list build)
         BALLOC(B.epair, Rs);
         if (cudaMemset(B.facc, 0, sizeof(unsigned) * 9 * np) != cudaSuccess ||
             cudaMemset(B.epair, 0, sizeof(long long) * Rs) != cudaSuccess)

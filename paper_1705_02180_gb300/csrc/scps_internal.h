@@ -42,13 +42,12 @@ struct TopoDev {
     int f_shift, g_shift;      // coarse unit of the force / bias-gradient partials (coarse_shift)
 };
 
-// Partials of the resident chain kernels: each is a 32-bit sum modulo 2^32 of integer terms
-// and a signed coarse sum of round(term / 2^shift), which most terms leave at zero. The
+// Partials of the chain kernels and force sums of the box: each is a 32-bit sum modulo 2^32 of
+// integer terms and a signed coarse sum of round(term / 2^shift), which most terms leave at zero. The
 // coarse sum is within (number of terms) 2^(shift - 1) of the total, so that sum and the
 // modular one give the total exactly while that stays below 2^31 (see join_coarse). The
 // largest shift for which it does, up to 2^22 units (512 kJ mol^-1 nm^-1 of a force).
-inline int coarse_shift(long long max_terms) {
-    int shift = 22;
+__host__ __device__ inline int coarse_shift(long long max_terms, int shift = 22) {
     while (shift > 1 && max_terms << (shift - 1) >= 1ll << 31) --shift;
     return shift;
 }
@@ -166,9 +165,10 @@ struct BoxDev {
     int* id;          // atom id of each slot, -1 for padding
     int* id2;         // sort buffer of id
     unsigned* facc;   // [replica][9][np] non-bonded force on the slot: three sums modulo 2^32 of
-                      // 2^-13 units, three coarse sums (int) in units of 2^kBoxShift and three
-                      // upper ones in units of 2^(kBoxShift + kBoxUpper) (order-free; cleared by
-                      // whoever consumes them)
+                      // 2^-13 units, three coarse sums (int) in units of 2^shift and three
+                      // upper ones in units of 2^(2 shift) (order-free; cleared by whoever
+                      // consumes them)
+    int* shift;       // [replica] coarse unit, from the lists a slot can be in (k_box_scan)
     int* big;         // [1] set once an upper word has been added to (they are read from then on)
     long long* epair; // [replica] pair energy of energy evaluations, fixed point 2^-18
                       // (cleared by whoever consumes it)
@@ -202,8 +202,8 @@ struct BoxDev {
     double* eb;       // [replica] bonded energy (save steps)
 };
 
-constexpr int kBoxShift = 21;  // a slot takes at most 2047 chunk sums (join_coarse stays exact)
-constexpr int kBoxUpper = 20;  // bits of a 64-bit term's coarse count that the coarse word takes
+constexpr int kBoxShift = 21;  // largest coarse unit of the box sums: that of up to 2047 lists per slot
+constexpr int kBoxMaxEnt = 1 << 14;  // most entries of a cluster's list
 constexpr uint32_t kBoxNoSlot = 0x7fffffu;  // padding entry of a box pair list
 
 // Step graphs of the periodic box (variants: regular, last step of a call, save step, save

@@ -57,3 +57,38 @@ def test_colliding_sites(r):
     again, U1 = forces(torch, pkg, s, x0)  # nothing of the collision is left
     assert np.array_equal(plain, again) and U0 == U1
     s.close()
+
+
+def test_more_lists_than_the_coarsest_unit_allows():
+    # A strongly charged site in the focus of a ring of 25 800 weakly charged ones, all later in slot
+    # order than the ring: it is in some 3 200 lists, each of which adds a force below half the
+    # coarsest unit (128 kJ mol^-1 nm^-1) with the same sign, 2.86e5 in all: beyond the 2^31 units
+    # of 2^-13 that the modular word holds. (A ring, so that no single list holds all of it.) Its
+    # force is the plain shifted-force Coulomb sum (no LJ), in FP64 from the FP32 positions.
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1705_02180_gb300 as pkg
+    L, rc, n, shells = 5.0, 2.0, 25800, 6
+    k = np.arange(n // shells) + 0.5
+    c0, c1 = np.cos(np.radians((40.0, 50.0)))
+    cos = c0 - k / len(k) * (c0 - c1)  # Fibonacci points between 40 and 50 degrees from -x
+    phi, sin = np.pi * (1.0 + 5.0 ** 0.5) * k, np.sqrt(1.0 - cos * cos)
+    ring = np.stack([-cos, sin * np.cos(phi), sin * np.sin(phi)], 1)
+    focus = np.array([4.2, 2.5, 2.5])
+    x = np.concatenate([[focus]] + [focus + r * ring for r in np.linspace(1.78, 1.82, shells)])
+    x = x.astype(np.float32).astype(np.float64)
+    q = np.full(len(x), 0.001)
+    q[0] = 1930.0
+    t = sites(x, q, eps=0.0)
+    s = pkg.System(topologies=[t], replica_topology=[0], x0=x, cutoff=rc, elec=pkg.ELEC_PLAIN, box=L, dt=0.002,
+                   gamma=1.0, kT=2.494, seed=5, skin=0.05, save_interval=1, max_frames=1)
+    F, _ = forces(torch, pkg, s, x)
+    s.step(1)
+    assert s.status()[0] == 0  # (the lists fit)
+    s.close()
+    d = x[0] - x[1:]
+    r = np.linalg.norm(d, axis=1)
+    ref = (138.935458 * q[0] * q[1] * (1.0 / r ** 2 - 1.0 / rc ** 2) / r)[:, None] * d
+    assert 2.0 ** 31 / 8192 < ref.sum(0)[0] and 8 * ref[:, 0].max() < 128.0
+    assert np.abs(F[0] - ref.sum(0)).max() <= 1e-5 * np.abs(ref.sum(0)).max()
