@@ -61,7 +61,7 @@ enum { SCPS_ELEC_NONE = 0, SCPS_ELEC_DDIEL = 1, SCPS_ELEC_RF = 2, SCPS_ELEC_PLAI
 enum { SCPS_INT_BAOAB = 0, SCPS_INT_EM = 1 };
 /* execution form of scps_step_replicas:
  *   RESIDENT: every replica stays on chip for the whole call (one CTA or one
- *     CTA cluster per replica, all replicas in one launch, CUDA graph);
+ *     CTA cluster per replica, CUDA graph);
  *   PLAIN: reference form - one replica per kernel launch per step, FP32 float
  *     atomics in global memory, no graph. Same physics, same noise. */
 enum { SCPS_EXEC_RESIDENT = 0, SCPS_EXEC_PLAIN = 1 };
@@ -190,7 +190,8 @@ typedef struct {
                                            box: 64 per chunk of 8 list entries of an 8-slot
                                            cluster (synchronises) */
     size_t device_bytes;                /* device memory held by the system */
-    int32_t launch_groups;              /* resident form: launches per step call chunk */
+    int32_t launch_groups;              /* resident form: launches per step call chunk (the
+                                           cluster_size and threads above are those of the last) */
     int32_t plan;                       /* resident form: SCPS_PLAN_* */
     double list_skin;                   /* pair-list skin r_list - r_c (nm) */
     double steps_per_list_build;        /* resident chains: mean steps per pair-list build in
@@ -200,7 +201,11 @@ typedef struct {
 } scps_info;
 
 /* launch plans of the resident form */
-enum { SCPS_PLAN_ONE_LAUNCH = 0,        /* one launch, replicas by decreasing size */
+enum { SCPS_PLAN_ONE_LAUNCH = 0,        /* one launch, replicas by decreasing size; with a few
+                                           replicas more than SMs and the launch shape left
+                                           open, the largest of them run as clusters of four
+                                           CTAs in a launch of their own beside it
+                                           (launch_groups is then 2) */
        SCPS_PLAN_PER_SIZE_CLASS = 1 };  /* one launch per size class (tile-rounded atom
                                            count), shared memory sized per class, the
                                            launches running side by side */

@@ -132,6 +132,7 @@ struct scps_system {
         int count = 0, nta = 0, cluster = 1, threads = 1024;
     };
     bool auto_shape = false;  // the caller left cluster size and threads open
+    int n_split = 0;          // plan 0: replicas of the leading group of four-CTA clusters
     std::vector<Group> groups;
     int plan = 0;  // 0: one launch, replicas by decreasing size; 1: one launch per size class
     std::vector<cudaStream_t> fork_streams;
@@ -415,12 +416,24 @@ int split_clusters(const std::vector<int>& atoms, int n_sm) {
     return best < 0.95 * none ? best_k : 0;
 }
 
+// Replicas of a leading group of four-CTA clusters in the shape (plan, cluster, threads): what
+// split_clusters asks for where the caller left the launch shape open, else none.
+int auto_split(const scps_system* s, int plan, int cluster, int threads) {
+    if (plan != 0 || !s->auto_shape || cluster != 1 || threads != kMaxThreadsPair) return 0;
+    int n_sm = 0;
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
+    std::vector<int> atoms;
+    for (int t : s->rep_topo) atoms.push_back(s->topos[t].n);
+    std::sort(atoms.begin(), atoms.end(), std::greater<int>());
+    return split_clusters(atoms, n_sm);
+}
+
 // Launch groups of the resident form. plan 0: one group, replicas by decreasing
 // size (large replicas start first, small ones fill the last wave), before it a group of
-// four-CTA clusters where split_clusters asks for one (the launch shape left open by the
-// caller only); plan 1: one group per size class (tile-rounded atom count), each with shared
-// memory for its own size. Other groups get the given cluster size and threads per CTA.
-int set_groups(scps_system* s, int plan, int cluster, int threads) {
+// the first n_split of them as four-CTA clusters; plan 1: one group per size class
+// (tile-rounded atom count), each with shared memory for its own size. Other groups get the
+// given cluster size and threads per CTA.
+int set_groups(scps_system* s, int plan, int cluster, int threads, int n_split) {
     if (cluster > 1 && threads > kMaxThreadsPair)
         return fail(SCPS_ERR_INVALID_ARG, "a CTA cluster takes at most %d threads per CTA",
                     kMaxThreadsPair);
@@ -431,14 +444,6 @@ int set_groups(scps_system* s, int plan, int cluster, int threads) {
         return s->topos[s->rep_topo[a]].n > s->topos[s->rep_topo[b]].n;
     });
     std::vector<std::vector<int>> members;
-    int n_split = 0;
-    if (plan == 0 && s->auto_shape && cluster == 1 && threads == kMaxThreadsPair) {
-        int n_sm = 0;
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, s->device);
-        std::vector<int> atoms(R);
-        for (int k = 0; k < R; ++k) atoms[k] = s->topos[s->rep_topo[order[k]]].n;
-        n_split = split_clusters(atoms, n_sm);
-    }
     if (plan == 0) {
         if (n_split > 0) members.emplace_back(order.begin(), order.begin() + n_split);
         members.emplace_back(order.begin() + n_split, order.end());
@@ -458,7 +463,7 @@ int set_groups(scps_system* s, int plan, int cluster, int threads) {
         int na = 0;
         for (int r : m) na = std::max(na, s->topos[s->rep_topo[r]].n);
         g.nta = plan == 0 ? s->nta : tile_atoms(na);
-        const bool split = n_split > 0 && groups.empty();
+        const bool split = plan == 0 && n_split > 0 && groups.empty();
         g.cluster = split ? 4 : cluster;
         g.threads = split ? cta_threads(g.nta, 4) : threads;
         std::vector<RepDev> reps(m.size());
@@ -487,6 +492,7 @@ int set_groups(scps_system* s, int plan, int cluster, int threads) {
     s->plan = plan;
     s->cluster = cluster;
     s->threads = threads;
+    s->n_split = plan == 0 ? n_split : 0;
     drop_graphs(s);
     return SCPS_OK;
 }
@@ -705,7 +711,7 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
                                  "%d atoms need %zu B of shared memory per CTA, above the limit; "
                                  "use the plain execution form", s->max_atoms, smem));
             s->auto_shape = !d->cluster_size && !d->threads;
-            rc = set_groups(s, 0, s->cluster, s->threads);
+            rc = set_groups(s, 0, s->cluster, s->threads, auto_split(s, 0, s->cluster, s->threads));
             if (rc) return bail(rc);
         }
     }
@@ -1725,7 +1731,7 @@ int scps_autotune(scps_system* s, int32_t probe_steps, int32_t use_cache, scps_t
                       std::to_string(s->bias_kind);
     for (auto& kv : sizes) key += "|" + std::to_string(kv.first) + "x" + std::to_string(kv.second);
     static std::mutex mu;
-    static std::map<std::string, std::vector<int>> cache;  // plan, cluster, threads, skin (pm)
+    static std::map<std::string, std::vector<int>> cache;  // plan, cluster, threads, split, skin (pm)
     scps_tune_result res{};
     res.plan = s->plan;
     res.cluster_size = s->cluster;
@@ -1740,9 +1746,9 @@ int scps_autotune(scps_system* s, int32_t probe_steps, int32_t use_cache, scps_t
             if (it != cache.end()) hit = it->second;
         }
         if (!hit.empty()) {
-            int rc = set_groups(s, hit[0], hit[1], hit[2]);
+            int rc = set_groups(s, hit[0], hit[1], hit[2], hit[3]);
             if (rc) return rc;
-            set_skin(s, 1e-3 * hit[3]);
+            set_skin(s, 1e-3 * hit[4]);
             drop_graphs(s);
             res.plan = hit[0];
             res.cluster_size = hit[1];
@@ -1795,14 +1801,13 @@ int scps_autotune(scps_system* s, int32_t probe_steps, int32_t use_cache, scps_t
     cudaEventCreate(&e1);
     RunParams P = s->base;
     P.save_interval = 0;
-    const int initial[3] = {s->plan, s->cluster, s->threads};
     std::vector<std::vector<int>> cands;
-    cands.push_back({initial[0], initial[1], initial[2]});
+    cands.push_back({s->plan, s->cluster, s->threads, s->n_split});
     const int n_plans = sizes.size() > 1 ? 2 : 1;
     for (int plan = 0; plan < n_plans; ++plan)
         for (int cl : {1, 2})
             for (int th : {256, 512, kMaxThreadsPair}) {
-                std::vector<int> c{plan, cl, th};
+                std::vector<int> c{plan, cl, th, auto_split(s, plan, cl, th)};
                 if (c != cands[0]) cands.push_back(c);
             }
     const size_t smem_limit = resident_smem_limit();
@@ -1836,7 +1841,7 @@ int scps_autotune(scps_system* s, int32_t probe_steps, int32_t use_cache, scps_t
     };
     for (size_t k = 0; k < cands.size(); ++k) {
         const std::vector<int>& c = cands[k];
-        if (set_groups(s, c[0], c[1], c[2]) != SCPS_OK) continue;
+        if (set_groups(s, c[0], c[1], c[2], c[3]) != SCPS_OK) continue;
         bool fits = true;
         for (auto& g : s->groups)
             fits = fits && resident_smem_bytes(g.nta) <= smem_limit;
@@ -1853,7 +1858,7 @@ int scps_autotune(scps_system* s, int32_t probe_steps, int32_t use_cache, scps_t
             best_c = c;
         }
     }
-    int rc = set_groups(s, best_c[0], best_c[1], best_c[2]);
+    int rc = set_groups(s, best_c[0], best_c[1], best_c[2], best_c[3]);
     if (rc) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
