@@ -126,7 +126,8 @@ typedef struct {
     int32_t max_frames;     /* frames kept per replica (the oldest are overwritten) */
     /* execution */
     int32_t exec;           /* SCPS_EXEC_* */
-    int32_t cluster_size;   /* CTAs per replica in RESIDENT form: 0 = auto (1, 2, 4 or 8), 1 or 2 */
+    int32_t cluster_size;   /* CTAs per replica in RESIDENT form: 0 = auto, 1, 2, 4 or 8 (periodic
+                               box and PLAIN form: 0, 1 or 2, without effect) */
     int32_t threads;        /* threads per CTA in RESIDENT form: 0 = auto, else 128..1024
                                (at most 768 in a cluster of CTAs) */
     int32_t steps_per_graph;/* device-loop steps per CUDA-graph node: 0 = auto */

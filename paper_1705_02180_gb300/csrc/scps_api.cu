@@ -554,13 +554,17 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
         return fail(SCPS_ERR_INVALID_ARG, "save_interval > 0 needs max_frames > 0");
     if (d->exec != SCPS_EXEC_RESIDENT && d->exec != SCPS_EXEC_PLAIN)
         return fail(SCPS_ERR_INVALID_ARG, "unknown exec form %d", d->exec);
-    if (d->cluster_size < 0 || d->cluster_size > 2)
-        return fail(SCPS_ERR_UNSUPPORTED, "cluster_size %d not supported (0, 1 or 2)", d->cluster_size);
+    // (clusters of four and eight CTAs are chain launch shapes, which scps_get_info reports)
+    const bool wide_ok = d->model == SCPS_MODEL_CHAIN && d->box == 0.0 && d->exec == SCPS_EXEC_RESIDENT;
+    if (d->cluster_size < 0 ||
+        (d->cluster_size > 2 && !(wide_ok && (d->cluster_size == 4 || d->cluster_size == 8))))
+        return fail(SCPS_ERR_UNSUPPORTED, "cluster_size %d not supported (0, 1 or 2%s)", d->cluster_size,
+                    wide_ok ? ", 4 or 8" : "");
     if (d->threads != 0 && (d->threads < 128 || d->threads > 1024 || d->threads % 32))
         return fail(SCPS_ERR_INVALID_ARG, "threads must be 0 or a multiple of 32 in [128, 1024]");
-    if (d->cluster_size == 2 && d->threads > kMaxThreadsPair)
-        return fail(SCPS_ERR_INVALID_ARG, "a 2-CTA cluster takes at most %d threads per CTA",
-                    kMaxThreadsPair);
+    if (d->cluster_size >= 2 && d->threads > kMaxThreadsPair)
+        return fail(SCPS_ERR_INVALID_ARG, "a %d-CTA cluster takes at most %d threads per CTA",
+                    d->cluster_size, kMaxThreadsPair);
     scps_system* s = new scps_system();
     s->d = *d;
     s->d.topologies = nullptr;

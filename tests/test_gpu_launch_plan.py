@@ -25,3 +25,44 @@ def test_a_cached_plan_is_the_plan_that_was_timed(torch_cuda, n, first):  # noqa
         got.append([s.info()[q] for q in SHAPE])
         s.close()
     assert got[0] == got[1]
+
+
+def run(s):
+    s.step(30)
+    assert s.status()[0] == 0
+    st = s.get_state()
+    s.close()
+    return [st[q] for q in ("x", "v", "zm", "T")]
+
+
+@pytest.mark.parametrize("n,R", [(560, 1), (560, 24), (304, 6)])
+def test_a_reported_shape_can_be_asked_for(torch_cuda, n, R):  # noqa: F811
+    c = cut(synth.make_chain(35, seed=1), n)
+    a = system(c, R=R)
+    info = a.info()
+    assert info["cluster_size"] >= 4
+    b = system(c, R=R, cluster_size=info["cluster_size"], threads=info["threads"])
+    assert [b.info()[q] for q in SHAPE] == [info[q] for q in SHAPE]
+    for x, y in zip(run(a), run(b)):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("n", [17, 64, 129])
+def test_more_ctas_than_tiles(torch_cuda, n):  # noqa: F811
+    c = cut(synth.make_chain(35, seed=1), n)
+    runs = [run(system(c, R=3, cluster_size=k)) for k in (1, 4, 8)]
+    for r in runs[1:]:
+        for x, y in zip(runs[0], r):
+            assert np.array_equal(x, y)
+
+
+def test_shapes_that_are_refused(torch_cuda):  # noqa: F811
+    import paper_1705_02180_gb300 as pkg
+    c = cut(synth.make_chain(35, seed=1), 64)
+    for kw, code in ((dict(cluster_size=3), -7), (dict(cluster_size=16), -7), (dict(cluster_size=-1), -7),
+                     (dict(cluster_size=8, threads=1024), -1),
+                     (dict(cluster_size=4, exec_form=pkg.EXEC_PLAIN), -7),
+                     (dict(cluster_size=4, box=9.0, elec=pkg.ELEC_RF), -7)):
+        with pytest.raises(pkg.ScpsError) as e:
+            system(c, **kw)
+        assert e.value.code == code, kw
