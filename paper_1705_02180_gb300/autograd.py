@@ -102,11 +102,13 @@ class ForceNormAction(torch.autograd.Function):
         F = torch.empty_like(X)
         system.energy_forces(topo, X, U, F)
         ctx.save_for_backward(X)
-        ctx.system, ctx.topo = system, topo
+        ctx.system, ctx.topo, ctx.segment = system, topo, segment
         return (F.double() ** 2).sum()
 
     @staticmethod
     def backward(ctx, g):
+        if ctx.segment < 1:
+            raise ValueError("segment must be at least 1")
         (X,) = ctx.saved_tensors
         U = torch.empty(X.shape[0], dtype=torch.float64, device=X.device)
         G = torch.empty_like(X)
@@ -119,5 +121,6 @@ class ForceNormAction(torch.autograd.Function):
 def force_norm_action(system, X, topo=0, segment=50):
     """sum_t |grad U(X_t)|^2 over the frames; the backward recomputes the forces (activation
     checkpointing over path frames). `segment` bounded the frames whose forces were live at a
-    time; the backward needs no memory for them any more, so every value gives the same."""
+    time; the backward needs no memory for them any more, so every value from 1 on gives the
+    same (smaller ones are refused by the backward)."""
     return ForceNormAction.apply(X, system, topo, segment)
