@@ -291,10 +291,9 @@ struct Term {
     double f[5];
 };
 
-// Tube bias on a path of kTubeWarpMin slices or more: one replica per warp, slice k on lane
-// k & 31 (NB slices per lane, kept in registers for up to 128 slices; NB = 0 reads them from
-// memory). 512 replicas x 100 slices: 11 us per step against 146 us with one lane per replica
-// walking all slices. Every sum keeps the order of that plain walk (the lane-tree sums that
+// Tube bias, one replica per warp (see tube_by_warps): slice k on lane k & 31 (NB slices per lane,
+// kept in registers for up to 128 slices; NB = 0 reads them from memory). 512 replicas x 100
+// slices: 12.5 us per step against 145 us with one lane per replica walking all slices. Every sum keeps the order of that plain walk (the lane-tree sums that
 // would save a quarter of the time change the last bits, which these trajectories amplify to
 // 1e-6 of the bias functional within a round), so results depend neither on the lanes nor on
 // how many replicas run beside one another.
@@ -439,10 +438,20 @@ k_plane_tube(StateDev st, RunParams P, const uint32_t* __restrict__ rep_ids) {
     if (!(isfinite(p.x) && isfinite(p.y))) st.status[r] = 1;
 }
 
-// Slices from which a warp per replica takes the tube sums: below it most lanes would idle in
-// the exp that dominates a slice (16 of about 30 FP64 instructions), and a lane per replica
-// finishes as early. The line depends on the path alone, not on the replica count.
+// Whether a warp per replica takes the tube sums (k_plane_tube), or a lane per replica (k_plane).
+// Below eight slices most lanes of a warp would idle in the exp that dominates a slice. Above,
+// a step of a warp is shorter by far, but a quarter of an SM takes the lanes of a warp (32
+// replicas) in the time of one, and warps one after another, so the lanes win with many replicas:
+// the cheaper of waves x measured time per step wins (40 steps, us: a warp 207 with 8 slices,
+// 435 with 100; a lane 656 and 5130. 4096 replicas x 8 slices: 1429 us as warps, 660 as lanes;
+// 32 768 x 100: 22 667 and 11 694). Both sum in the same order: the bits are the same.
 constexpr int kTubeWarpMin = 8;
+
+bool tube_by_warps(int R, int K, int n_sm) {
+    if (K < kTubeWarpMin) return false;
+    const long long warps = (R + 4ll * n_sm - 1) / (4 * n_sm), lanes = (R + 128ll * n_sm - 1) / (128 * n_sm);
+    return warps * (163 + 1.4 * K + 33 * ((K + 31) / 32)) < lanes * (230 + 54.0 * K);
+}
 
 cudaError_t launch_toy(const StateDev& st, const RunParams& P, const uint32_t* rep_ids,
                        cudaStream_t stream) {
@@ -451,7 +460,7 @@ cudaError_t launch_toy(const StateDev& st, const RunParams& P, const uint32_t* r
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int R = P.n_replicas;
-    if (P.bias == 4 && P.tube_k >= kTubeWarpMin) {
+    if (P.bias == 4 && tube_by_warps(R, P.tube_k, n_sm)) {
         // one warp per quarter of an SM, spread over all SMs first
         const int per = std::min(4, (R + n_sm - 1) / n_sm);
         const dim3 grid((R + per - 1) / per);
