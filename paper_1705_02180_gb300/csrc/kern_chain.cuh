@@ -49,6 +49,7 @@ namespace scps {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
+constexpr unsigned kNonFinite = 0xffffffffu;  // Scalars::vmax2: beyond the bits of any float
 constexpr int kFlagGradCoarse = 256;  // Scalars::flag: coarse words of G were touched
 constexpr int kChunk = 32;    // contacts / bonds / angles per work item (one per lane)
 
@@ -119,15 +120,15 @@ struct Scalars {
     int work_next[2];   // this CTA's work counter, by parity of the evaluated step
     int status;         // replica status (identical in every CTA of a cluster): written by this
                         // CTA's warp 0 alone, before the barrier that ends a decision
-    int nonfinite[2];   // NONFINITE bit of the update, by parity: raised by any CTA of the cluster
-                        // before the barrier that closes the update, read only after it
     int bias_on;
     int flag[2];        // force-range bits raised during the evaluation of a given parity
     int n_items;        // pair items in this CTA's item table
     int cached;         // 1: the items are held in shared memory (Shared::lc)
     int n_diag;         // blocks whose inner pairs this CTA evaluates
     int build_next;     // block counter of a list build
-    unsigned vmax2[2];  // largest |v1|^2 + |v2|^2 of the update, by parity (float bits)
+    unsigned vmax2[2];  // largest |v1|^2 + |v2|^2 of the update, by parity (float bits), or
+                        // kNonFinite: some CTA's new state is not finite. Raised by every CTA
+                        // before the barrier that closes the update, read only after it
     long long pair_slots;  // pairs one evaluation with the current list takes
     long long n_saved;
     double zm, z, epot, T;
@@ -1319,8 +1320,6 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         sc.work_next2[1] = 0;
         sc.vmax2[0] = 0u;
         sc.vmax2[1] = 0u;
-        sc.nonfinite[0] = 0;
-        sc.nonfinite[1] = 0;
         for (int q = 0; q < 6; ++q) (&sc.zw[0][0])[q] = 0u;
         sc.sm = st.sm[r];
         sc.wm = st.wm[r];
@@ -1331,6 +1330,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
     }
     long long step = st.step[r];
     int builds = 0;  // pair-list builds in this launch
+    bool nonfinite = false;  // an update left the FP32 range (the same in all threads of the cluster)
     cluster_barrier<CL>();  // every CTA of the cluster is initialised before any remote access
     const float hdt = P.half_dt;
     if (sc.status == 0 && P.n_steps > 0) {
@@ -1383,6 +1383,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             const bool save = do_b && save_phase == 0;
             const float kb = sc.kb;  // F_bias = kb G
             float vm2 = 0.f;  // largest |v after B|^2 + |v after O|^2 of this thread's atoms
+            bool finite = true;
             // the other parity's partials were last read before this evaluation's cluster
             // barrier (here and in the other CTAs): clear them for the next one
             {
@@ -1436,9 +1437,8 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                         x.y = fmaf(hdt, v.y, x.y);
                         x.z = fmaf(hdt, v.z, x.z);
                         vm2 = fmaxf(vm2, v1 + fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)));
-                        if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
-                              isfinite(v.y) && isfinite(v.z)))
-                            for (int q = 0; q < CL; ++q) atomicOr(rank_ptr<CL>(&sc.nonfinite[b], q), SCPS_FLAG_NONFINITE);
+                        finite = finite && isfinite(x.x) && isfinite(x.y) && isfinite(x.z) &&
+                                 isfinite(v.x) && isfinite(v.y) && isfinite(v.z);
 #pragma unroll
                         for (int q = 0; q < CL; ++q) rank_ptr<CL>(sm.xq(), q)[i] = x;
                     }
@@ -1446,13 +1446,12 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
                 }
             }
             if (do_a) {  // largest speed of the step (positive floats order as their bits)
-                const unsigned wm = __reduce_max_sync(kFull, __float_as_uint(vm2));
+                const unsigned wm = __reduce_max_sync(kFull, finite ? __float_as_uint(vm2) : kNonFinite);
                 if (lane < CL && wm) atomicMax(rank_ptr<CL>(&sc.vmax2[b], lane), wm);
             }
             if (tid == 0) {
                 sc.flag[nb] = 0;
                 sc.vmax2[nb] = 0u;
-                sc.nonfinite[nb] = 0;  // (last read after the barrier of the step before)
                 sc.zw[nb][0] = sc.zw[nb][1] = sc.zw[nb][2] = 0u;
             }
             cluster_barrier<CL>();  // every CTA has the new positions
@@ -1477,17 +1476,19 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
             // leave after the last B, when a force was out of range, or when the new state is
             // non-finite. Every thread of the cluster must leave at the same place, so each word
             // read here is one that no CTA can write before all have read it: the force-range bit
-            // belongs to a decision and the other word to an update, with a cluster barrier
+            // belongs to a decision and the speed bound to an update, with a cluster barrier
             // between either and its next writer. (One word for both would let a CTA that is
             // already in the next update stop one that still has to take it.)
             if (save) slot = slot + 1 == P.max_frames ? 0 : slot + 1;
-            if (!do_a || sc.status != 0 || sc.nonfinite[b] != 0) break;
+            const unsigned vmax = sc.vmax2[b];
+            nonfinite = do_a && vmax == kNonFinite;
+            if (!do_a || sc.status != 0 || nonfinite) break;
             ++step;
             if (save_phase >= 0) save_phase = save_phase + 1 == P.save_interval ? 0 : save_phase + 1;
             // |x_new - x_old| <= dt/2 (|v after B| + |v after O|) <= dt/2 sqrt(2 vmax2) per
             // atom; a pair inside r_c now was inside r_c + 2 disp at the build, so the list
             // stays complete while 2 disp < skin (a 1 % margin covers the FP32 rounding)
-            disp += hdt * sqrtf(2.0f * __uint_as_float(sc.vmax2[b]));
+            disp += hdt * sqrtf(2.0f * __uint_as_float(vmax));
             ++since;
             if (disp >= 0.99f * P.skin_half || (P.rebuild_every > 0 && since >= P.rebuild_every)) {
                 build_list<CL>(sm, sc, P.rlist2);
@@ -1509,7 +1510,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
         }
     }
     __syncthreads();
-    const int status = sc.status | sc.nonfinite[0] | sc.nonfinite[1];
+    const int status = sc.status | (nonfinite ? SCPS_FLAG_NONFINITE : 0);
     // write back the state: each CTA the atoms it integrated, rank 0 the scalars
     for (int i = kTile * own_lo(tp.n_tiles, rank, CL) + tid;
          i < min(n, kTile * own_lo(tp.n_tiles, rank + 1, CL)); i += blockDim.x) {
