@@ -51,6 +51,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned kNonFinite = 0xffffffffu;  // Scalars::vmax2: beyond the bits of any float
 constexpr int kFlagGradCoarse = 256;  // Scalars::flag: coarse words of G were touched
+constexpr float kForceLimit13 = 8.192e12f;  // 1e9 kJ mol^-1 nm^-1 in 2^-13 units
 constexpr int kChunk = 32;    // contacts / bonds / angles per work item (one per lane)
 
 extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -117,6 +118,7 @@ struct ListDev {
 struct Scalars {
     TopoDev tp;         // the replica's topology and list slab (shared memory: read where
     ListDev list;       // needed instead of held in registers)
+    PairConst pc;       // for the slow path of a pair item
     int work_next[2];   // this CTA's work counter, by parity of the evaluated step
     int status;         // replica status (identical in every CTA of a cluster): written by this
                         // CTA's warp 0 alone, before the barrier that ends a decision
@@ -196,7 +198,7 @@ __device__ __forceinline__ void red3_64(const Part& p, int k, long long vx, long
 __device__ __forceinline__ void add_pair13(const Part& F, int* flag, int sh, int i, int j, float s13,
                                            float dx, float dy, float dz) {
     const float tx = s13 * dx, ty = s13 * dy, tz = s13 * dz;
-    const float lim = 8.192e12f;  // 1e9 in 2^-13 units
+    const float lim = kForceLimit13;
     if (!(fabsf(tx) <= lim && fabsf(ty) <= lim && fabsf(tz) <= lim)) atomicOr(flag, SCPS_FLAG_FORCE_RANGE);
     const long long qx = __float2ll_rn(tx), qy = __float2ll_rn(ty), qz = __float2ll_rn(tz);
     red3_64(F, i, qx, qy, qz, sh);
@@ -258,8 +260,13 @@ __device__ __forceinline__ ListDev list_of(unsigned char* slab, int nta, int ran
 // move by one xor exchange per iteration and component, those of the entries stay in the
 // lane; all are integers in 32-bit registers. Items near their block (NEARX) take the excluded
 // pairs from the masks xm (low byte entry j0, high byte j1). Returns false (and adds nothing)
-// when some |s| of the quarter warp exceeds pc.s_lim / 2, for which the integer sums of the
-// item (16 terms for a block atom) could overflow; the caller then takes the slow path.
+// when the integer sums of the item could overflow; the caller then takes the slow path. They
+// cannot while every |s| of the quarter warp is up to pc.s_lim / 2 (16 terms for a block atom, 8
+// for an entry), nor, looked at only where one is larger, while every |s| is up to pc.s_lim and
+// the lanes' largest |s| add up to no more than 4 pc.s_lim (a block atom takes two terms from
+// each lane). Close atoms mostly meet one at a time, and a launch waits for its slowest frame: 28
+// frames of 44 atoms 16.5 -> 9.9 us, of 100 atoms 18.3 -> 12.0, against every item with an |s|
+// beyond pc.s_lim / 2 on the slow path.
 //
 // Bound by the FMA pipe: 33 packed operations per two pairs, and next to it the XU pipe (two
 // rsqrt, six conversions, 2.1 clocks each). Packing the two entries, which stay in registers,
@@ -271,10 +278,10 @@ __device__ __forceinline__ bool pair_item_fast(const Shared& sm, const Part& F,
                                                unsigned xm, int lane, long long& e18) {
     const int l8 = lane & 7, q = lane >> 3;
     const Entries n = pack_entries(sm.xq()[j0], sm.xq()[j1], sm.lj()[j0], sm.lj()[j1]);
-    const float lim = 0.5f * kPairScale * pc.s_lim;
     int fix = 0, fiy = 0, fiz = 0;
     int fax = 0, fay = 0, faz = 0, fbx = 0, fby = 0, fbz = 0;
     long long ei = 0;
+    float most = 0.0f;  // largest |s| of this lane, times 2^13 (NaN: some pair's is)
     bool bad = false;
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
@@ -296,7 +303,7 @@ __device__ __forceinline__ bool pair_item_fast(const Shared& sm, const Part& F,
         float2 ms = pair_ms2<ELEC, ENERGY>(r2, lj, make_float2(xi.w * n.q.x, xi.w * n.q.y), pc, &e);
         ms.x = ok0 ? ms.x : 0.0f;
         ms.y = ok1 ? ms.y : 0.0f;
-        bad = bad || !(fabsf(ms.x) <= lim) || !(fabsf(ms.y) <= lim);
+        most = max_nan(most, max_nan(fabsf(ms.x), fabsf(ms.y)));
         const float2 fx = mul2(ms, dx), fy = mul2(ms, dy), fz = mul2(ms, dz);
         // (the terms come out negated: they are the entries' share)
         const int ax = __float2int_rn(fx.x), bx = __float2int_rn(fx.y);
@@ -322,7 +329,15 @@ __device__ __forceinline__ bool pair_item_fast(const Shared& sm, const Part& F,
             fiz = __shfl_xor_sync(kFull, fiz, t ^ (t + 1));
         }
     }
-    if ((__ballot_sync(kFull, bad) >> (8 * q)) & 0xffu) return false;
+    const float lim = kPairScale * pc.s_lim;
+    unsigned over = __ballot_sync(kFull, bad || !(most <= 0.5f * lim));
+    if (over) {
+        float sum = most;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(kFull, sum, o);
+        over = __ballot_sync(kFull, bad || !(most <= lim) || !(sum <= 4.0f * lim));
+        if ((over >> (8 * q)) & 0xffu) return false;
+    }
     red3(F, 8 * I + (l8 ^ 7), fix, fiy, fiz, sm.fsh);  // lane l ends with atom l ^ 7's sums
     red3(F, j0, fax, fay, faz, sm.fsh);
     red3(F, j1, fbx, fby, fbz, sm.fsh);
@@ -330,34 +345,55 @@ __device__ __forceinline__ bool pair_item_fast(const Shared& sm, const Part& F,
     return true;
 }
 
-// Slow path of an item, one entry per lane: every pair term goes to both atoms in 64-bit
-// (rounded per pair as on the fast path) with the range check (a force beyond 1e9 kJ/mol/nm
-// or a non-finite one freezes the replica).
+// Slow path of an item: the same pairs with 64-bit sums (rounded per pair as on the fast path) and
+// the range check (a force beyond 1e9 kJ/mol/nm or a non-finite one freezes the replica). As
+// there, the block atoms' sums move from lane to lane and the entries' stay, and each goes to the
+// partials once. Its first call in a launch costs about 5 us (it is small, and reads the pair
+// constants and masks from shared memory, so that little has to come from far: 8 us with them
+// read from the launch parameters and tables and with atomics for every pair).
 template <int ELEC, bool ENERGY>
-__device__ __noinline__ long long pair_item_slow(Shared sm, int b, Scalars* sc, const RunParams& P,
-                                                 int I, int j) {
+__device__ __noinline__ long long pair_item_slow(Shared sm, int b, Scalars* sc, int I, int j0, int j1,
+                                                 unsigned xm) {
     const int l8 = threadIdx.x & 7;
+    const unsigned quarter = 0xffu << (threadIdx.x & 24);  // (the quarter's lanes all come here)
     const Part F = sm.F(b);
-    const TopoDev& tp = sc->tp;
-    const PairConst& pc = P.pc;
+    const PairConst& pc = sc->pc;
     long long e18 = 0;
-    const float4 xj = sm.xq()[j];
-    const float2 lj = sm.lj()[j];
-    for (int t = 0; t < 8; ++t) {
-        const int i = 8 * I + ((l8 + t) & 7);
-        const float4 xi = sm.xq()[i];
-        const float2 li = sm.lj()[i];
-        const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        bool ok = r2 < pc.rc2;
-        const int dj = j - i + kExclWindow;
-        if (dj >= 0 && dj < 2 * kExclWindow && i < tp.n_atoms) ok = ok && !((tp.excl[i] >> dj) & 1ull);
-        if (!ok) continue;
-        float e = 0.f;
-        const float s = pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y, xi.w * xj.w, pc, &e);
-        add_pair13(F, &sc->flag[b], sm.fsh, i, j, s * kPairScale, dx, dy, dz);
-        if (ENERGY) e18 += __float2ll_rn(e * kPairEScale);
+    bool out = false;
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+        const int j = u ? j1 : j0;
+        const float4 xj = sm.xq()[j];
+        const float2 lj = sm.lj()[j];
+        long long fi[3] = {}, fj[3] = {};
+#pragma unroll 1
+        for (int t = 0; t < 8; ++t) {
+            const int a = l8 ^ t, i = 8 * I + a;
+            const float4 xi = sm.xq()[i];
+            const float2 li = sm.lj()[i];
+            const float dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            if (r2 < pc.rc2 && !((xm >> (8 * u + a)) & 1u)) {
+                float e = 0.f;
+                const float s13 = kPairScale * pair_s<ELEC, ENERGY>(r2, li.x + lj.x, li.y * lj.y,
+                                                                    xi.w * xj.w, pc, &e);
+                const float f[3] = {s13 * dx, s13 * dy, s13 * dz};
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const long long q = __float2ll_rn(f[c]);
+                    out = out || !(fabsf(f[c]) <= kForceLimit13);
+                    fi[c] += q;
+                    fj[c] -= q;
+                }
+                if (ENERGY) e18 += __float2ll_rn(e * kPairEScale);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) fi[c] = __shfl_xor_sync(quarter, fi[c], (t ^ (t + 1)) & 7);
+        }
+        red3_64(F, 8 * I + l8, fi[0], fi[1], fi[2], sm.fsh);  // (the last exchange brought them home)
+        red3_64(F, j, fj[0], fj[1], fj[2], sm.fsh);
     }
+    if (out) atomicOr(&sc->flag[b], SCPS_FLAG_FORCE_RANGE);
     return e18;
 }
 
@@ -395,9 +431,8 @@ __device__ __forceinline__ void pair_batch(const Shared& sm, Scalars& sc, const 
     else
         done = pair_item_fast<ELEC, ENERGY, false>(sm, F, P.pc, I, j0, j1, 0u, lane, e18);
     if (!done) {
-        const long long ea = pair_item_slow<ELEC, ENERGY>(sm, b, &sc, P, I, j0);
-        const long long eb = pair_item_slow<ELEC, ENERGY>(sm, b, &sc, P, I, j1);
-        if (ENERGY) e18 += ea + eb;
+        const long long es = pair_item_slow<ELEC, ENERGY>(sm, b, &sc, I, j0, j1, near ? xm : 0u);
+        if (ENERGY) e18 += es;
     }
 }
 
@@ -1283,6 +1318,7 @@ k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, S
     const int rank = cta_rank<CL>();
     if (threadIdx.x == 0) {
         sc.tp = topos[rep.topo];
+        sc.pc = P.pc;
         sc.list = list_of<CL>(P.list_base + rep.list_off, nta, rank);
     }
     __syncthreads();
@@ -1550,6 +1586,7 @@ k_eval_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __
     const int rank = cta_rank<CL>();
     if (threadIdx.x == 0) {
         sc.tp = *topo_ptr;
+        sc.pc = P.pc;
         sc.list = list_of<CL>(P.list_base + (blockIdx.x / CL) * P.list_slab, nta, rank);
     }
     __syncthreads();

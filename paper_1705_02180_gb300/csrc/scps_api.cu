@@ -835,8 +835,8 @@ int scps_create_system(const scps_system_desc* d, scps_system** out) {
     const double krf = (d->eps_rf - 1.0) / ((2.0 * d->eps_rf + 1.0) * rcut * rcut * rcut);
     P.pc.krf = (float)krf;
     P.pc.crf = (float)(1.0 / rcut + krf * rcut * rcut);
-    // the 2^-13 pair terms of one item (8 per accumulator) stay below 2^31 while
-    // |s| r_c 2^13 8 < 2^31; larger |s| take the exact slow path
+    // eight 2^-13 pair terms in one accumulator stay below 2^31 while |s| r_c 2^13 8 < 2^31
+    // (16 while |s| is half that); the kernels take larger |s| pair by pair in 64 bits
     P.pc.s_lim = (float)(32000.0 / rcut);
     // pair list of the resident chain kernels (the periodic box keeps its own)
     const double skin = d->skin > 0.0 ? d->skin : (s->is_box ? 0.15 : kDefaultChainSkin);

@@ -107,6 +107,13 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
+// The larger of two values, NaN when either is.
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 // 1/sqrt(x) with denormal x taken as zero: the bits of rsqrtf for every normal x, without
 // the rescaling that rsqrtf carries for denormal ones.
 __device__ __forceinline__ float rsqrt_ftz(float x) {
