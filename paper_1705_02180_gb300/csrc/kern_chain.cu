@@ -70,6 +70,24 @@ int chain_max_clusters(int cl, int nta, int threads) {
     return cl == 8 ? max_clusters_cl<8>(nta, threads) : max_clusters_cl<4>(nta, threads);
 }
 
+// Whether `count` lone CTAs run in the wide form: the narrow form's 64 registers spill more
+// (300 replicas of 64 atoms 7.1 us per step, 6.6 in the wide form; 128 atoms 13.2 and 12.2), but
+// more of its CTAs share an SM, which pays where that saves a wave (600 of 128 atoms 23.4 and
+// 26.4; 304 of 560 on 512 threads 68 and 73).
+static bool wide_form(int count, int nta, int threads) {
+    int dev = 0, n_sm = 0, per_sm = 0, reserved = 0, lc_cap = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    const int smem = (int)(launch_smem(nta, threads, 1, &lc_cap) + kChainStaticSmem) + reserved;
+    auto waves = [&](int regs) {
+        const int fit = std::max(1, std::min(65536 / (regs * threads), per_sm / smem));
+        return (count + fit * n_sm - 1) / std::max(1, fit * n_sm);
+    };
+    return waves(80) <= waves(64);
+}
+
 cudaError_t launch_resident(int elec, int cluster, const TopoDev* topos, const RepDev* reps,
                             const StateDev& st, const RunParams& P, int nta, int threads,
                             cudaStream_t stream) {
@@ -79,8 +97,7 @@ cudaError_t launch_resident(int elec, int cluster, const TopoDev* topos, const R
         case 2: return launch_resident_cl<2, true>(elec, topos, reps, st, P, nta, threads, stream);
         default: break;
     }
-    // (two CTAs per SM want the registers of the narrow form)
-    if (threads > 512 && threads <= kMaxThreadsPair)
+    if (threads <= kMaxThreadsPair && wide_form(P.n_replicas, nta, threads))
         return launch_resident_cl<1, true>(elec, topos, reps, st, P, nta, threads, stream);
     return launch_resident_cl<1, false>(elec, topos, reps, st, P, nta, threads, stream);
 }

@@ -312,10 +312,11 @@ int atoms_per_replica(const scps_system* s, int r) {
 }
 
 // Threads of a resident CTA when there are more CTAs than SMs: 256 for small chains, so that
-// several share an SM, else one CTA of 768 at a time (304 replicas on 152 SMs: 560 atoms 62.9 us
-// per step against 68.2 with two CTAs of 512 threads per SM, 400 atoms 39.0 against 41.7, 304
-// atoms 28.4 against 28.9).
-int auto_threads(int nta) { return nta <= 256 ? 256 : kMaxThreadsPair; }
+// several share an SM, 192 for the smallest (300 replicas of 64 atoms 6.6 us per step against
+// 7.8 with 256, 9.4 with 128), else one CTA of 768 at a time (304 replicas on 152 SMs: 560 atoms
+// 62.9 us per step against 68.2 with two CTAs of 512 threads per SM, 400 atoms 39.0 against
+// 41.7, 304 atoms 28.4 against 28.9).
+int auto_threads(int nta) { return nta <= 64 ? 192 : nta <= 256 ? 256 : kMaxThreadsPair; }
 
 // Threads of a resident CTA with an SM to itself: 768, but 512 where a cluster leaves a CTA few
 // atoms (304 atoms on four CTAs 8.7 us per step against 9.2, 560 on eight 11.8 against 12.3).
