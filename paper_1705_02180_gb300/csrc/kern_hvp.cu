@@ -31,7 +31,7 @@ namespace {
 
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kHvpSeg = 32;          // candidate blocks J per work unit (one per lane)
-constexpr int kHvpMaxBlocks = 512;   // 8-atom blocks per frame (4096 atoms)
+constexpr int kHvpMaxBlocks = kMaxChainAtoms / 8;  // 8-atom blocks per frame
 
 struct HvpShared {
     float4* xq;      // (x, y, z, qs)
@@ -40,7 +40,8 @@ struct HvpShared {
     unsigned long long* ex;  // exclusion mask per atom slot
     // 2^-20 fixed-point partials v of 3 components per slot: the low 20 bits (unsigned), the
     // rest q = v >> 20 as a sum modulo 2^32 and coarse sums of round(q / 2^22), which only the
-    // largest terms (stiff bonds) touch
+    // largest terms (stiff bonds) touch. (A slot takes at most 256 sums as an entry, 40 as a block
+    // atom, and its bonds and angles; up to 1023 terms are exact, see coarse_shift.)
     unsigned *L0, *L1;
     int* H;
     float4* blo;     // boxes of the 8-atom blocks
@@ -451,6 +452,18 @@ static cudaError_t launch_hvp_t(const TopoDev* topo, const RunParams& P, const f
     return cudaGetLastError();
 }
 
+// Threads of a lone CTA: a chain has as many work units as 8-atom blocks, or a few more, so that
+// many threads of a small one only wait at its barriers and keep other frames off the SM. 1000
+// frames of 17 atoms 32.3 us with 512 threads, 19.2 with 256, 13.5 with 128; of 44 atoms 36.0,
+// 25.0, 21.2 (but 200 frames 11.2, 10.9, 13.5); of 100 atoms 60.9, 49.0; of 160 atoms 83.3, 79.1
+// (200 frames 25.9, 30.4).
+static int lone_threads(long long n_frames, int nta, int n_sm) {
+    if (nta <= 32) return 128;
+    if (nta <= 64) return 256;
+    if (n_frames <= n_sm) return nta <= 128 ? 512 : 1024;
+    return nta <= 128 ? 256 : 512;
+}
+
 // Few frames: a cluster of 1024-thread CTAs per frame, so that the frames spread over the
 // SMs; many frames, or small ones (28 frames of 64 atoms 12.3 us with one CTA, 13.8 with two; of
 // 200 atoms 24.2, and 20.5 with four): one CTA each.
@@ -462,12 +475,12 @@ static cudaError_t launch_hvp_e(const TopoDev* topo, const RunParams& P, const f
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (nta < kEvalClusterAtoms)
-        return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, n_frames <= n_sm ? 1024 : 512, s);
+    const int lone = lone_threads(n_frames, nta, n_sm);
+    if (nta < kEvalClusterAtoms) return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, lone, s);
     if (10 * n_frames <= n_sm) return launch_hvp_t<ELEC, 8>(topo, P, X, V, HV, n_frames, nta, 1024, s);
     if (5 * n_frames <= n_sm) return launch_hvp_t<ELEC, 4>(topo, P, X, V, HV, n_frames, nta, 1024, s);
     if (2 * n_frames <= n_sm) return launch_hvp_t<ELEC, 2>(topo, P, X, V, HV, n_frames, nta, 1024, s);
-    return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, n_frames <= n_sm ? 1024 : 512, s);
+    return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, lone, s);
 }
 
 cudaError_t launch_hvp(int elec, const TopoDev* topo, const RunParams& P, const float* X,
