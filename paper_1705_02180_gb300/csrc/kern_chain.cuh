@@ -20,8 +20,8 @@
 // chunk (128 pairs) on a quarter warp: lane l keeps entries 2 l and 2 l + 1 of the chunk
 // and takes block atom l ^ t against both at its iteration t, two FP32 pairs per packed
 // operation, so the i-force accumulators move by one xor exchange per iteration while the
-// j-forces stay in place (64 replicas x 560 atoms: 21.8 us per step, against 26.7 with chunks of 8, one
-// entry per lane and scalar operations; the same bits). Pairs inside a block form 28-pair
+// j-forces stay in place (64 replicas x 560 atoms: 18.9 us per step; these items alone took it
+// from 26.7, with chunks of 8, one entry per lane and scalar operations, to 21.8; the same bits). Pairs inside a block form 28-pair
 // items of their own. The list is rebuilt when a bound on the largest displacement
 // since the last build reaches skin/2, or after rebuild_every steps, so no pair
 // inside r_c is ever missing.
@@ -1303,11 +1303,10 @@ __device__ __forceinline__ float4 far_slot(int i) {
 }  // namespace
 
 // WIDE: at most kMaxThreadsPair threads per CTA, which leaves 80 registers per thread (every
-// cluster of several CTAs, and a lone CTA that has an SM to itself: 1200 atoms 78.5 us per step
-// against 84.0 with 1024 threads of 64 registers, 304 atoms 14.3 against 15.4). Otherwise up to
-// 1024 threads of 64 registers: for small chains, several of which share an SM, and for callers who
-// ask for 1024 threads or for two 512-thread CTAs per SM (304 replicas of 560 atoms: 68 us per
-// step, 73 with 80 registers, which leave one CTA per SM).
+// cluster of several CTAs, and a lone CTA that has an SM to itself: 1200 atoms 78.0 us per step
+// against 84.0 with 1024 threads of 64 registers, 304 atoms 14.4 against 15.4). Otherwise up to
+// 1024 threads of 64 registers: for callers who ask for more threads, and where more CTAs on an SM
+// save a wave (wide_form).
 template <int ELEC, int CL, bool TUBE, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? kMaxThreadsPair : 1024, 1)
 k_resident(const TopoDev* __restrict__ topos, const RepDev* __restrict__ reps, StateDev st,

@@ -62,9 +62,9 @@ __device__ __forceinline__ double2 normals2_f64(uint32_t a, uint32_t b) {
 constexpr float kFixScale = 1048576.0f;         // 2^20
 constexpr float kFixInv = 9.5367431640625e-07f;  // 2^-20
 // Non-bonded pair terms: each s (x_j - x_i) is rounded to 2^-13 units (summed in 32-bit
-// registers over a few pairs, then moved to the 2^-20 accumulators), each pair energy to
-// 2^-18 units (finer: the many small energies near r_c share one sign, so their rounding
-// does not average out); larger pair energies take the 64-bit path.
+// registers over a few pairs, then in 2^-13 partials modulo 2^32 with coarse words beside them, see
+// coarse_shift), each pair energy to 2^-18 units (finer: the many small energies near r_c share
+// one sign, so their rounding does not average out); larger pair energies take the 64-bit path.
 constexpr float kPairScale = 8192.0f;     // 2^13
 constexpr float kPairEScale = 262144.0f;  // 2^18
 constexpr float kPairEMax = 8000.0f;
@@ -265,7 +265,7 @@ enum { ELEC_NONE = 0, ELEC_DDIEL = 1, ELEC_RF = 2, ELEC_PLAIN = 3 };
 struct PairConst {
     float rc, rc2, inv_rc, inv_rc2, inv_rc3;
     float krf, crf;  // reaction field: k_rf, c_rf
-    float s_lim;     // largest |s| whose pair terms the 2^-13 integer sums of one item hold
+    float s_lim;     // largest |s| of which eight 2^-13 pair terms stay below 2^31 in one sum
 };
 
 // LJ constants of one pair: sigma^2, 24 eps, and (sigma / r_c)^6 with the
