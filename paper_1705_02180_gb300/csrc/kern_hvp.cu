@@ -240,7 +240,7 @@ __device__ __forceinline__ void hvp_cluster_sync() {
 template <int ELEC, int CL>
 __global__ void __launch_bounds__(1024)
 k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __restrict__ X,
-             const float* V, float* HV, int nta) {  // (HV may be V)
+             const float* V, float* HV, int nta, int split) {  // (HV may be V)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int next_row, n_units;
     __shared__ int upre[kHvpMaxBlocks];  // first work unit of each row of blocks
@@ -312,7 +312,10 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
     for (int a = t0; a < tp.n_angles; a += tstep) hvp_angle(sm, tp, a);
     // work units: the rows of blocks I with I % CL == rank, each cut into segments of kHvpSeg
     // candidate blocks J >= I (long rows first); a warp pulls a unit, tests its blocks
-    // against I's box and their atoms against I's, and takes the hits 64 at a time
+    // against I's box and their atoms against I's, and takes the hits 64 at a time. In a cluster
+    // `split` warps may share a unit: each makes the tests and takes its chunks of 64 (the
+    // same chunks, so the same sums)
+    const int parts = CL == 1 ? 1 : split;
     if (warp == 0) {
         int run = 0;
         for (int r0 = 0; r0 < nbs; r0 += 32) {
@@ -334,7 +337,9 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
         int u = 0;
         if (lane == 0) u = atomicAdd(&next_row, 1);
         u = __shfl_sync(kFullMask, u, 0);
-        if (u >= n_units) break;
+        if (u >= n_units * parts) break;
+        const int part = u % parts;
+        u /= parts;
         int lo = 0, hi = nbs;  // the last row whose first unit is <= u
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -383,7 +388,7 @@ k_hvp_frames(const TopoDev* __restrict__ topo_ptr, RunParams P, const float* __r
             count += __popc(nm);
         }
         __syncwarp();
-        for (int k0 = 0; k0 < count; k0 += 64) {
+        for (int k0 = 64 * part; k0 < count; k0 += 64 * parts) {
             const int k = k0 + 2 * lane;
             const bool live0 = k < count, live1 = k + 1 < count;
             const int ja = live0 ? sm.buf[k] : 8 * I, jb = live1 ? sm.buf[k + 1] : 8 * I;
@@ -431,6 +436,11 @@ template <int ELEC, int CL>
 static cudaError_t launch_hvp_t(const TopoDev* topo, const RunParams& P, const float* X,
                                 const float* V, float* HV, long long n_frames, int nta, int threads,
                                 cudaStream_t s) {
+    // A small chain has fewer units than a cluster has warps, and the longest sets the time: 4
+    // frames of 160 atoms 16.6 -> 13.1 us, of 304 20.6 -> 16.4; 28 frames (four CTAs) 16.9 -> 13.7 and
+    // 21.7 -> 19.2; 76 frames of 304 atoms (two CTAs) 25.4 -> 23.2. With 560 atoms the tests made
+    // more than once cost more (27.8 -> 33.8).
+    const int split = nta > 320 ? 1 : CL >= 4 ? 4 : 2;
     const size_t smem = hvp_smem_bytes(nta, threads);
     auto kern = k_hvp_frames<ELEC, CL>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -447,7 +457,7 @@ static cudaError_t launch_hvp_t(const TopoDev* topo, const RunParams& P, const f
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, topo, P, X, V, HV, nta);
+    e = cudaLaunchKernelEx(&cfg, kern, topo, P, X, V, HV, nta, split);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
