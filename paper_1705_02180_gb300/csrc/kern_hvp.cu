@@ -475,8 +475,8 @@ static int lone_threads(long long n_frames, int nta, int n_sm) {
 }
 
 // Few frames: a cluster of 1024-thread CTAs per frame, so that the frames spread over the
-// SMs; many frames, or small ones (28 frames of 64 atoms 12.3 us with one CTA, 13.8 with two; of
-// 200 atoms 24.2, and 20.5 with four): one CTA each.
+// SMs; many frames, or small ones (28 frames of 44 atoms 9.3 us with one CTA, 10.9 with two or four;
+// of 100 atoms 13.0, and 12.1 with four; of 200 atoms 21.8, and 15.1 with four): one CTA each.
 template <int ELEC>
 static cudaError_t launch_hvp_e(const TopoDev* topo, const RunParams& P, const float* X,
                                 const float* V, float* HV, long long n_frames, int nta,
@@ -486,7 +486,7 @@ static cudaError_t launch_hvp_e(const TopoDev* topo, const RunParams& P, const f
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int lone = lone_threads(n_frames, nta, n_sm);
-    if (nta < kEvalClusterAtoms) return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, lone, s);
+    if (nta <= 64) return launch_hvp_t<ELEC, 1>(topo, P, X, V, HV, n_frames, nta, lone, s);
     if (10 * n_frames <= n_sm) return launch_hvp_t<ELEC, 8>(topo, P, X, V, HV, n_frames, nta, 1024, s);
     if (5 * n_frames <= n_sm) return launch_hvp_t<ELEC, 4>(topo, P, X, V, HV, n_frames, nta, 1024, s);
     if (2 * n_frames <= n_sm) return launch_hvp_t<ELEC, 2>(topo, P, X, V, HV, n_frames, nta, 1024, s);

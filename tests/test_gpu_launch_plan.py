@@ -66,3 +66,21 @@ def test_shapes_that_are_refused(torch_cuda):  # noqa: F811
         with pytest.raises(pkg.ScpsError) as e:
             system(c, **kw)
         assert e.value.code == code, kw
+
+
+@pytest.mark.parametrize("n", [65, 100, 128, 300])
+def test_shared_rows_of_hessian_vector_products(torch_cuda, n):  # noqa: F811
+    # the warps of a cluster share the rows of small chains chunk by chunk: the same sums
+    torch = torch_cuda
+    c = cut(synth.make_chain(35, seed=1), n)
+    s = system(c)
+    g = np.random.default_rng(6)
+    X = torch.from_numpy((c.x_unfolded[None] + g.normal(0, 0.01, (180, n, 3))).astype(np.float32)).cuda()
+    V = torch.from_numpy(g.normal(0, 1, (180, n, 3)).astype(np.float32)).cuda()
+    whole = torch.empty_like(X)
+    s.hvp(0, X, V, whole)  # one CTA per frame
+    for m in (152, 60, 20, 3):  # one with more threads, two, four, eight
+        part = torch.empty_like(X[:m])
+        s.hvp(0, X[:m].contiguous(), V[:m].contiguous(), part)
+        assert torch.equal(whole[:m], part)
+    s.close()
